@@ -83,8 +83,9 @@ typedef struct lb_options {
     int32_t mdt_override;  /* > 0: use this MDT instead of the histogram (0) */
     int32_t hp_threshold;  /* HP switches to WD below this list size (1024);
                               a negative value disables the switch */
-    int32_t loop_mode;     /* 0: device-resident loop (CUDA graph with a
-                              conditional WHILE node); 1: host loop with a
+    int32_t loop_mode;     /* 0: device-resident loop (WD: the whole query in
+                              one cooperative launch; other strategies: a CUDA
+                              graph with a conditional WHILE node); 1: host loop with a
                               worklist-size readback per iteration, as in the
                               paper's drivers (0) */
     int32_t wd_tile;       /* largest WD tile in worklist edges: 256..32768,
@@ -121,14 +122,14 @@ typedef struct lb_options {
                               sub-lists keep the last one (Sec. III-C leaves
                               the depth of the hierarchy to the user) */
     int32_t small_edges;   /* WD: while the worklist has at most this many
-                              edges, levels run inside one persistent launch
-                              (one CTA per SM, a grid barrier between levels)
-                              instead of a launch per level: high-diameter
-                              graphs have thousands of such levels.
-                              0..16777216; 0 = off (65536) */
+                              edges, its levels run on a team of CTAs with a
+                              barrier of its own (device loop) or inside one
+                              persistent launch (host loop) instead of on the
+                              whole grid: high-diameter graphs have thousands
+                              of such levels.  0..16777216; 0 = off (a graph
+                              starts with 16384) */
     int32_t test_barrier_skip; /* test hook, 0 in normal use: 1 makes CTA 1 of
-                              the small-list launch leave before its first
-                              grid barrier, so the other CTAs' bounded waits
+                              a WD query leave before its first grid barrier, so the other CTAs' bounded waits
                               run out (2 s) and the query returns
                               LB_ERR_TIMEOUT with the device still usable */
     int32_t bitmap_place;  /* 0..7 (0): where the visited / queued bitmap
@@ -189,8 +190,7 @@ typedef struct lb_step_record {
     int32_t level;         /* super-iteration (BFS level of the list) */
     int32_t mode;          /* 0 relax, 1 HP sub-iteration, 2 HP WD step,
                               3 HP degree-binned step (hp_mode 1), 4 WD
-                              level inside the persistent small-list
-                              launch */
+                              level on the small-list team */
     int64_t list_size;     /* entries in the list this step consumed */
     int64_t edges;         /* edges relaxed by this step */
     int64_t t_ns;          /* device time at the end of the step, in ns from

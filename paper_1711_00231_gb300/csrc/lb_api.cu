@@ -80,8 +80,7 @@ struct DeviceGuard {
 
 constexpr int kStrategies = 7;
 
-// Default small_edges.  Measured (R-MAT scale 24 BFS / 4096^2 grid BFS):
-// 65536 edges 2.12 / 65.8 ms, 16384 edges 2.12 / 58.7 ms, off 2.09 / 118 ms.
+// Default small_edges.
 #ifndef LB_SMALL_EDGES_DEFAULT
 #define LB_SMALL_EDGES_DEFAULT 16384
 #endif
@@ -162,6 +161,8 @@ struct lb_graph {
 
     cudaGraphExec_t exec[kStrategies][2]{};
     int grid[kStrategies][2]{};
+    int query_grid[2]{};        // whole-query WD launch (0: not yet computed)
+    uint32_t query_number = 0;  // whole-query WD launches so far
 
     // batched host-output queries: the second result buffer, one error
     // word per query, the copy stream and the events that order each
@@ -460,6 +461,18 @@ int step_grid(lb_graph *g, int s, bool sssp) {
     return gr;
 }
 
+// Grid of the whole-query WD launch: every CTA resident (a cooperative
+// launch), at most ctas_per_sm per SM.
+int query_grid(lb_graph *g, bool sssp) {
+    int &gr = g->query_grid[sssp ? 1 : 0];
+    if (gr == 0) {
+        int occ = query_wd_blocks_per_sm(sssp);
+        if (g->opt.ctas_per_sm > 0 && g->opt.ctas_per_sm < occ) occ = g->opt.ctas_per_sm;
+        gr = occ * g->sms;
+    }
+    return gr;
+}
+
 // CTAs of the persistent small-list launch (all resident: a cooperative launch).
 int small_grid(const lb_graph *g) { return g->sms * small_ctas_per_sm(); }
 
@@ -496,42 +509,7 @@ lb_status build_exec(lb_graph *g, int s, bool sssp, cudaGraphExec_t *out) {
     p.use_cond = 1;
     p.cond = h;
     const int grid = step_grid(g, s, sssp);
-    // WD with small-list levels: the loop body starts with an IF node whose
-    // body is the persistent small-list launch; the step kernel sets its
-    // condition for the next pass (the last kSmallAfter lists had at most
-    // small_edges edges), so other levels launch nothing extra.  Off on the
-    // first pass (default 0).
-    cudaGraphNode_t if_node = nullptr;
-    if (p.small_edges > 0) {
-        cudaGraphConditionalHandle hs;
-        e = cudaGraphConditionalHandleCreate(&hs, body, 0, cudaGraphCondAssignDefault);
-        alignas(cudaGraphNodeParams) unsigned char ip_store[sizeof(cudaGraphNodeParams)];
-        memset(ip_store, 0, sizeof(ip_store));
-        cudaGraphNodeParams &ip = *reinterpret_cast<cudaGraphNodeParams *>(ip_store);
-        ip.type = cudaGraphNodeTypeConditional;
-        ip.conditional.handle = hs;
-        ip.conditional.type = cudaGraphCondTypeIf;
-        ip.conditional.size = 1;
-        if (e == cudaSuccess) e = cudaGraphAddNode(&if_node, body, nullptr, nullptr, 0, &ip);
-        if (e == cudaSuccess) {
-            p.use_cond_small = 1;
-            p.cond_small = hs;
-            e = cudaStreamBeginCaptureToGraph(g->stream, ip.conditional.phGraph_out[0], nullptr, nullptr, 0,
-                                              cudaStreamCaptureModeThreadLocal);
-            if (e == cudaSuccess) {
-                const cudaError_t le = launch_small_levels(sssp, p, small_grid(g), g->stream);
-                cudaGraph_t captured = nullptr;
-                e = cudaStreamEndCapture(g->stream, &captured);
-                if (le != cudaSuccess) e = le;
-            }
-        }
-        if (e != cudaSuccess) {
-            cudaGraphDestroy(graph);
-            return fail(LB_ERR_CUDA, "building the small-list node failed: %s", cudaGetErrorString(e));
-        }
-    }
-    e = cudaStreamBeginCaptureToGraph(g->stream, body, if_node ? &if_node : nullptr, nullptr, if_node ? 1 : 0,
-                                      cudaStreamCaptureModeThreadLocal);
+    e = cudaStreamBeginCaptureToGraph(g->stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         cudaError_t le = cudaSuccess;
         if (hp_needs_mdt_kernel(g, s)) le = launch_hp_mdt(p, 2 * g->sms, g->stream);
@@ -573,9 +551,27 @@ lb_status run_query(lb_graph *g, int kind, int s, int32_t src, void *out_dev, in
     StepParams p = make_params(g, s);
     const uint32_t max_levels = (uint32_t)(g->n + 1 < 0xFFFFFFF0ll ? g->n + 1 : 0xFFFFFFF0ll);
     const uint64_t max_steps = (uint64_t)1 << 40;
-    const int grid = step_grid(g, s, sssp);
-    LB_CU(cudaEventRecord(g->ev_start, st));
     const uint64_t time_limit_ns = (uint64_t)120 * 1000000000ull;  // safety net; no query comes close
+    const int grid = g->opt.loop_mode == 0 && s == LB_WD ? query_grid(g, sssp) : step_grid(g, s, sssp);
+    LB_CU(cudaEventRecord(g->ev_start, st));
+    if (g->opt.loop_mode == 0 && s == LB_WD) {
+        QueryArgs a;
+        a.status = (uint32_t *)out_dev;
+        a.src = src;
+        a.max_levels = max_levels;
+        a.time_limit_ns = time_limit_ns;
+        a.number = g->query_number;
+        a.team = small_grid(g) < grid ? small_grid(g) : grid;
+        LB_CU(launch_query_wd(sssp, p, a, grid, st));
+        ++g->query_number;
+        if (parents_dev) LB_CU(launch_parents(p, sssp, parents_dev, st));
+        LB_CU(cudaEventRecord(g->ev_stop, st));
+        LB_CU(cudaEventRecord(g->ev_done, st));
+        g->last_stream = st;
+        g->has_last = true;
+        g->last_strategy = s;
+        return LB_OK;
+    }
     LB_CU(launch_prepare(p, src, (uint32_t *)out_dev, kind, max_levels, max_steps, time_limit_ns, st));
     LB_CU(launch_init(p, grid, st));
     if (g->opt.loop_mode == 0) {
@@ -871,6 +867,7 @@ lb_status lb_set_options(lb_graph *g, const lb_options *o) {
     if (g->has_last) cudaEventSynchronize(g->ev_done);
     drop_execs(g);
     memset(g->grid, 0, sizeof(g->grid));
+    memset(g->query_grid, 0, sizeof(g->query_grid));
     if (n.hist_bins != g->opt.hist_bins || n.mdt_override != g->opt.mdt_override) {
         g->mdt = -1;
         g->ns_children = -1;

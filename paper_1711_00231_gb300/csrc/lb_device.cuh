@@ -38,6 +38,19 @@ namespace lbk {
 constexpr int kWB = LB_KWB;
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
+// How a kernel reads worklists (and other data that other CTAs write):
+//   kLdRo     read-only path: the data is fixed for the whole launch
+//             (single-iteration launches)
+//   kLdCg     through L2 (ld.global.cg): other CTAs write it during the
+//             launch with no barrier in between (serving, small-list levels)
+//   kLdPlain  plain L1 loads: it is written during the launch, but only
+//             before a grid barrier whose acquire drops the SM's L1 lines
+//             (the persistent query kernel)
+// The visited bits and distances that the current iteration itself changes
+// are read plainly in kLdRo and kLdPlain: a stale value only costs an extra
+// atomic.
+enum : int { kLdRo = 0, kLdCg = 1, kLdPlain = 2 };
+
 // what a flush writes
 enum : int { kOutNode = 0, kOutGranule = 1, kOutEdges = 2, kOutEdgesPerEdge = 3, kOutPhys = 4 };
 
@@ -68,7 +81,7 @@ struct FlushOut {
     int32_t *elist;    // edge-id output
     unsigned long long *pack;
     uint32_t *err;               // error word (capacity overflow)
-    unsigned long long *pushes;  // push counter
+    unsigned long long *pushes;  // push counter (NULL: the caller counts list entries)
     const int32_t *child_first;  // kOutPhys: first child id of each split node
     int64_t cap;       // entries the output can hold
     int64_t tile_cap;  // tstart entries
@@ -286,6 +299,8 @@ __device__ __forceinline__ void wflush_prefix(WB &b, WS &s, uint32_t cnt, const 
     }
 }
 
+constexpr uint32_t kLaneGrains = 8;
+
 template <int KIND, bool TILED, class WB, class WS>
 __device__ __forceinline__ void wflush_write(const WB &b, const WS &s, uint32_t &cnt, const FlushOut &o,
                                              unsigned long long old, uint32_t run_u) {
@@ -312,15 +327,29 @@ __device__ __forceinline__ void wflush_write(const WB &b, const WS &s, uint32_t 
                 o.list.v[pos] = b.v[i];
                 o.list.beg[pos] = b.beg[i];
                 o.list.scan[pos] = (int32_t)S;
-                if (TILED) {
+                if (TILED && o.tile != (int32_t)kTileGrain) {
                     const int64_t E = S + d;
-                    if (o.tile == (int32_t)kTileGrain) {  // the hot path: shifts, no division
-                        for (int64_t k = (S + kTileGrain - 1) >> 8; (k << 8) < E; ++k)
-                            if (k < o.tile_cap) o.list.tstart[k] = (int32_t)pos;
-                    } else {
-                        for (int64_t k = (S + o.tile - 1) / o.tile; k * o.tile < E; ++k)
-                            if (k < o.tile_cap) o.list.tstart[k] = (int32_t)pos;
-                    }
+                    for (int64_t k = (S + o.tile - 1) / o.tile; k * o.tile < E; ++k)
+                        if (k < o.tile_cap) o.list.tstart[k] = (int32_t)pos;
+                }
+            }
+            if (TILED && o.tile == (int32_t)kTileGrain) {
+                // the hot path: 32-bit shifts.  A lane writes up to
+                // kLaneGrains starts of its entry; a longer entry (a hub
+                // covers thousands of grains) is written by the whole warp.
+                const uint32_t S = (uint32_t)ebase + re + ie - d;
+                uint32_t k0 = (S + (uint32_t)kTileGrain - 1u) >> 8;
+                const uint32_t k1 = u ? min((S + d + (uint32_t)kTileGrain - 1u) >> 8, (uint32_t)o.tile_cap) : 0u;
+                const int32_t pos = (int32_t)((uint32_t)ubase + ru + iu - u);
+                unsigned big = __ballot_sync(kFull, k1 > k0 + kLaneGrains);
+                if (k1 > k0 && k1 <= k0 + kLaneGrains)
+                    for (; k0 < k1; ++k0) o.list.tstart[k0] = pos;
+                while (big) {
+                    const int l = __ffs(big) - 1;
+                    big &= big - 1;
+                    const uint32_t kb = __shfl_sync(kFull, k0, l), ke = __shfl_sync(kFull, k1, l);
+                    const int32_t pl = __shfl_sync(kFull, pos, l);
+                    for (uint32_t k = kb + lane; k < ke; k += 32) o.list.tstart[k] = pl;
                 }
             }
             ru += __shfl_sync(kFull, iu, 31);
@@ -355,7 +384,7 @@ __device__ LB_FLUSH_INLINE void wflush(WB &b, WS &s, uint32_t &cnt, const FlushO
     unsigned long long old = 0;
     if (lane == 0) {
         old = atomicAdd(o.pack, ((unsigned long long)run_u << 32) | (unsigned long long)run_e);
-        atomicAdd(o.pushes, (unsigned long long)run_u);
+        if (o.pushes) atomicAdd(o.pushes, (unsigned long long)run_u);
     }
     old = __shfl_sync(kFull, old, 0);
     __syncwarp();
@@ -386,7 +415,7 @@ __device__ void wflush_block(WB &b, WS &s, uint32_t &cnt, const FlushOut &o) {
             sum += t;
         }
         s_base = sum ? atomicAdd(o.pack, sum) : 0ull;
-        if (sum) atomicAdd(o.pushes, sum >> 32);
+        if (sum && o.pushes) atomicAdd(o.pushes, sum >> 32);
     }
     __syncthreads();
     if (cnt) wflush_write<KIND, TILED>(b, s, cnt, o, s_base + s_tot[warp], run_u);
@@ -414,9 +443,9 @@ __device__ __forceinline__ uint32_t *queued_half(uint32_t *bitmap, int64_t words
     return bitmap + (level & 1u) * words;
 }
 
-template <bool COH>
+template <int LD>
 __device__ __forceinline__ bool is_queued(const uint32_t *q, int32_t u) {
-    const uint32_t x = COH ? __ldcg(q + ((uint32_t)u >> 5)) : q[(uint32_t)u >> 5];
+    const uint32_t x = LD == kLdCg ? __ldcg(q + ((uint32_t)u >> 5)) : q[(uint32_t)u >> 5];
     return (x >> ((uint32_t)u & 31u)) & 1u;
 }
 
@@ -445,7 +474,7 @@ __device__ __forceinline__ bool sssp_relax(uint32_t *__restrict__ status, uint32
     const uint32_t old = atomicMin(&status[v], alt);
     if (alt >= old) return false;
     if (alt == kSat) atomicOr(&ctl->error, kErrSaturated);
-    if (is_queued<false>(q, v)) return false;
+    if (is_queued<kLdRo>(q, v)) return false;
     const uint32_t bit = 1u << ((uint32_t)v & 31u);
     return !(atomicOr(&q[(uint32_t)v >> 5], bit) & bit);
 }
@@ -457,7 +486,7 @@ __device__ __forceinline__ bool sssp_relax(uint32_t *__restrict__ status, uint32
 // every relaxation from u a no-op.
 __device__ __forceinline__ uint32_t sssp_source_dist(const uint32_t *__restrict__ status, const uint32_t *q,
                                                      int32_t u) {
-    return is_queued<false>(q, u) ? kInf : status[u];
+    return is_queued<kLdRo>(q, u) ? kInf : status[u];
 }
 
 // Relaxes ITEMS loaded edges of a warp and pushes the vertices that must be
@@ -465,17 +494,15 @@ __device__ __forceinline__ uint32_t sssp_source_dist(const uint32_t *__restrict_
 // every atomic, then every offset load of a won vertex, then the pushes --
 // so the latencies of the items overlap instead of queueing behind one
 // another (a warp-synchronous push between items would serialise them).
-// Loads of data other CTAs write: plain (L1) inside a single-iteration
-// launch, L2-coherent (ld.global.cg) inside the persistent serving kernel.
 // BFS visited check through L2 (1) instead of L1 (0): sees other SMs'
 // claims sooner at the cost of L2 latency (measured 31% slower at R-MAT
 // scale 24).
 #ifndef LB_BFS_BITMAP_CG
 #define LB_BFS_BITMAP_CG 0
 #endif
-template <bool COH>
+template <int LD>
 __device__ __forceinline__ uint32_t ld_mut(const uint32_t *p) {
-    return COH ? __ldcg(p) : *p;
+    return LD == kLdCg ? __ldcg(p) : *p;
 }
 
 // Warp-uniform early exits in relax_items: after the checks when no lane
@@ -486,7 +513,7 @@ __device__ __forceinline__ uint32_t ld_mut(const uint32_t *p) {
 #endif
 // FLUSH = false: the caller flushes; then cnt + 32 * ITEMS <= capacity on entry.
 // With FlushOut::defer set (kOutNode) only the vertex is buffered.
-template <bool SSSP, int ITEMS, int KIND, bool TILED, bool COH = false, bool FLUSH = true, class WB, class WS>
+template <bool SSSP, int ITEMS, int KIND, bool TILED, int LD = kLdRo, bool FLUSH = true, class WB, class WS>
 __device__ __forceinline__ void relax_items(const bool (&ok)[ITEMS], const int32_t (&vv)[ITEMS],
                                             const uint32_t (&ww)[ITEMS], const uint32_t (&dd)[ITEMS],
                                             const int64_t *__restrict__ off, uint32_t *__restrict__ bitmap,
@@ -506,9 +533,9 @@ __device__ __forceinline__ void relax_items(const bool (&ok)[ITEMS], const int32
             // reached kSat is exactly the case of the 64-bit sum >= kSat
             const uint32_t s32 = dd[it] + ww[it];
             val[it] = (s32 < dd[it] || s32 >= kSat) ? kSat : s32;
-            cand[it] = val[it] < ld_mut<COH>(status + vv[it]);
+            cand[it] = val[it] < ld_mut<LD>(status + vv[it]);
         } else {
-            cand[it] = !(ld_mut<COH || LB_BFS_BITMAP_CG>(bitmap + ((uint32_t)vv[it] >> 5)) & (1u << ((uint32_t)vv[it] & 31u)));
+            cand[it] = !(ld_mut<LB_BFS_BITMAP_CG ? kLdCg : LD>(bitmap + ((uint32_t)vv[it] >> 5)) & (1u << ((uint32_t)vv[it] & 31u)));
         }
     }
     if (LB_EARLY_EXIT) {
@@ -540,7 +567,7 @@ __device__ __forceinline__ void relax_items(const bool (&ok)[ITEMS], const int32
         // queue only the first improvement of v in this iteration
 #pragma unroll
         for (int it = 0; it < ITEMS; ++it)
-            if (won[it] && is_queued<COH>(qcur, vv[it])) won[it] = false;
+            if (won[it] && is_queued<LD>(qcur, vv[it])) won[it] = false;
 #pragma unroll
         for (int it = 0; it < ITEMS; ++it)
             if (won[it]) prev[it] = atomicOr(&qcur[(uint32_t)vv[it] >> 5], 1u << ((uint32_t)vv[it] & 31u));
@@ -612,7 +639,7 @@ __device__ __forceinline__ void relax_items(const bool (&ok)[ITEMS], const int32
 // level writes, offset loads and one push of all won vertices with edges.
 // The push buffer is flushed only when this group's pushes would not fit,
 // so flushes carry close to a full buffer.  Requires R * 32 <= capacity.
-template <int R, bool COH, class WB, class WS>
+template <int R, int LD, class WB, class WS>
 __device__ __forceinline__ void relax_bfs_lean(const bool (&ok)[R], const int32_t (&vv)[R],
                                                const int64_t *__restrict__ off, uint32_t *__restrict__ bitmap,
                                                uint32_t *__restrict__ status, uint32_t level, WB &wb,
@@ -621,7 +648,7 @@ __device__ __forceinline__ void relax_bfs_lean(const bool (&ok)[R], const int32_
     uint32_t cand = 0;  // bit r: item r found v unvisited
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const uint32_t x = ok[r] ? ld_mut<COH || LB_BFS_BITMAP_CG>(bitmap + ((uint32_t)vv[r] >> 5)) : 0xFFFFFFFFu;
+        const uint32_t x = ok[r] ? ld_mut<LB_BFS_BITMAP_CG ? kLdCg : LD>(bitmap + ((uint32_t)vv[r] >> 5)) : 0xFFFFFFFFu;
         if (!((x >> ((uint32_t)vv[r] & 31u)) & 1u)) cand |= 1u << r;
     }
     if (!__any_sync(kFull, cand != 0u)) return;
@@ -739,7 +766,7 @@ __device__ __forceinline__ void relax_bfs_lean(const bool (&ok)[R], const int32_
 // (only if some lane found an improvement) every candidate vertex and the
 // distance it offers go into the push buffer.  The flush makes the
 // atomicMin and queued-bit claims of a whole buffer at once.
-template <int R, bool COH, class WB, class WS>
+template <int R, int LD, class WB, class WS>
 __device__ __forceinline__ void relax_sssp_defer(const bool (&ok)[R], const int32_t (&vv)[R],
                                                  const uint32_t (&ww)[R], const uint32_t (&dd)[R],
                                                  const uint32_t *__restrict__ status, WB &wb, WS &ws,
@@ -755,7 +782,7 @@ __device__ __forceinline__ void relax_sssp_defer(const bool (&ok)[R], const int3
         // reached kSat is exactly the case of the 64-bit sum >= kSat
         const uint32_t s32 = dd[r] + ww[r];
         val[r] = (s32 < dd[r] || s32 >= kSat) ? kSat : s32;
-        if (val[r] < ld_mut<COH || LB_SSSP_STATUS_CG>(status + vv[r])) cand |= 1u << r;
+        if (val[r] < ld_mut<LB_SSSP_STATUS_CG ? kLdCg : LD>(status + vv[r])) cand |= 1u << r;
     }
     if (!__any_sync(kFull, cand != 0u)) return;
     unsigned bal[R];
@@ -828,10 +855,7 @@ __device__ __forceinline__ void set_loop(const StepParams &p, Ctl *ctl, bool mor
     }
     ctl->active = more ? 1u : 0u;
     if (p.use_cond) cudaGraphSetConditional(p.cond, more ? 1u : 0u);
-    if (p.small_edges > 0) {
-        ctl->small_run = ctl->in_edges <= (uint64_t)p.small_edges ? ctl->small_run + 1u : 0u;
-        if (p.use_cond_small) cudaGraphSetConditional(p.cond_small, (more && ctl->small_run >= kSmallAfter) ? 1u : 0u);
-    }
+    if (p.small_edges > 0) ctl->small_run = ctl->in_edges <= (uint64_t)p.small_edges ? ctl->small_run + 1u : 0u;
 }
 
 // Finalise a plain (non-HP) step: the output list becomes the input list.

@@ -29,7 +29,7 @@ constexpr int kBlock = 256;             // threads per CTA of every step kernel
 constexpr int kWarps = kBlock / 32;
 constexpr int kTraceMax = 4096;
 constexpr int kHistMax = 4096;  // largest HistogramBinCount
-// The persistent small-list kernel takes over once this many consecutive
+// Host loop: the persistent small-list kernel takes over once this many consecutive
 // levels have produced lists of at most small_edges edges: a high-diameter
 // graph has thousands of such levels, a skewed graph only a few at its
 // start and end, where entering the persistent launch costs more than it
@@ -78,6 +78,22 @@ struct TraceRec {
 #else
 #define LB_CTL_ALIGN
 #endif
+// Synchronisation words of the whole-query WD kernel, each on a 128-byte
+// line of its own.  All of them must be zero when a query starts: query q
+// uses qsync[q & 1] and clears qsync[(q + 1) & 1], so a query that ended at
+// a time limit (and left its words part way) cannot disturb the next one.
+struct QuerySync {
+    alignas(128) uint32_t full_arrive;  // arrivals at the barrier of the whole grid, ever increasing
+    alignas(128) uint32_t full_release; // barriers of the whole grid completed
+    alignas(128) uint32_t team_arrive;  // arrivals at the barrier of the small-list team
+    alignas(128) uint32_t resume;       // publications of the state below (kResumeAbort: the team gave up)
+    uint32_t r_level, r_par, r_cnt, r_done;
+    uint64_t r_edges;
+    struct alignas(128) Pack {
+        unsigned long long v;  // (entries << 32) | edges; bit 63: the time limit has passed
+    } pack[3];  // output counters: level L uses pack[L % 3]
+};
+
 struct Ctl {
     // query parameters (written by the prepare kernel)
     uint32_t *status;
@@ -117,6 +133,7 @@ struct Ctl {
     LB_CTL_ALIGN unsigned long long pushes;
     uint32_t trace_len;
     uint32_t pad;
+    QuerySync qsync[2];  // whole-query kernel (query number q uses qsync[q & 1])
     TraceRec trace[kTraceMax];
     uint32_t hp_hist[kHistMax];  // HP depth > 1: histogram of a sub-list (zero between uses)
 };
@@ -166,11 +183,8 @@ struct StepParams {
     int32_t test_barrier_skip;  // test hook: CTA 1 of the small-list launch skips its first barrier
     int32_t strategy;
     int32_t use_cond;
-    int32_t small_edges;   // WD: lists of at most this many edges run in the persistent small-list kernel (0: off)
+    int32_t small_edges;   // WD: lists of at most this many edges run on a small-list team of CTAs (0: off)
     cudaGraphConditionalHandle cond;
-    cudaGraphConditionalHandle cond_small;  // device loop: run the small-list kernel on the next pass
-    int32_t use_cond_small;
-    int32_t pad2;
 };
 
 // ---- launch entry points implemented by the strategy translation units --
@@ -182,6 +196,18 @@ cudaError_t launch_init(const StepParams &p, int grid, cudaStream_t st);
 cudaError_t launch_hp_mdt(const StepParams &p, int grid, cudaStream_t st);
 cudaError_t launch_small_levels(bool sssp, const StepParams &p, int grid, cudaStream_t st);
 int small_ctas_per_sm();
+// The whole WD query in one cooperative launch (grid CTAs, of which `team`
+// run the levels with small lists).
+struct QueryArgs {
+    uint32_t *status;
+    int32_t src;
+    uint32_t max_levels;
+    uint64_t time_limit_ns;
+    uint32_t number;  // queries launched on this workspace so far
+    int32_t team;
+};
+cudaError_t launch_query_wd(bool sssp, const StepParams &p, const QueryArgs &a, int grid, cudaStream_t st);
+int query_wd_blocks_per_sm(bool sssp);
 cudaError_t launch_finish_query(const StepParams &p, cudaStream_t st);
 cudaError_t launch_coo_build(const GraphDev &g, int32_t *coo_src, cudaStream_t st);
 cudaError_t launch_mdt(const GraphDev &g, int32_t bins, unsigned long long *scratch, int64_t *result,

@@ -281,7 +281,7 @@ __device__ __forceinline__ bool sssp_relax_cg(uint32_t *status, uint32_t *q, int
     const uint32_t old = atomicMin(&status[v], alt);
     if (alt >= old) return false;
     if (alt == kSat) atomicOr(err, kErrSaturated);
-    if (is_queued<true>(q, v)) return false;
+    if (is_queued<kLdCg>(q, v)) return false;
     const uint32_t bit = 1u << ((uint32_t)v & 31u);
     return !(atomicOr(&q[(uint32_t)v >> 5], bit) & bit);
 }
@@ -495,7 +495,7 @@ __device__ void relax_tile(const Params &P, Slot *S, int64_t t, int64_t ntiles, 
     o.claim_status = st.status;
     o.claim_level = st.level;
     uint32_t cnt = 0;
-    wd_walk_tile<SSSP, ITEMS, true>(g, ws_list(st.ws, W, st.par), st.in_cnt, (int64_t)st.in_edges, q * kTileGrain,
+    wd_walk_tile<SSSP, ITEMS, kLdCg>(g, ws_list(st.ws, W, st.par), st.in_cnt, (int64_t)st.in_edges, q * kTileGrain,
                                      t, bitmap, qcur, st.status, st.level, &S->error, wb, ws, cnt, o);
 #if LB_BLOCK_FLUSH
     wflush_block<kOutNode, true>(wb, ws, cnt, o);

@@ -109,9 +109,9 @@ __host__ __device__ constexpr bool wd_run_loop() {
 #ifndef LB_WD_GRAIN_START
 #define LB_WD_GRAIN_START 1
 #endif
-template <bool SSSP, bool COH>
+template <bool SSSP, int LD>
 __host__ __device__ constexpr bool wd_grain_start() {
-    return LB_WD_GRAIN_START && (SSSP || COH);
+    return LB_WD_GRAIN_START && (SSSP || LD != 0);
 }
 // Deferred claims in the persistent small-list kernel (as in the WD step;
 // bit mask: 1 = SSSP, 2 = BFS).  Measured on the 4096^2 grid: BFS equal,
@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(kBlock) k_step_phys(StepParams p) {
                     du = sssp_source_dist(status, qcur, x);
                 } else {
                     const int32_t parent = __ldg(p.parent_of + (x - n));
-                    du = is_queued<false>(qcur, parent) ? kInf : p.child_dist[x - n];
+                    du = is_queued<kLdRo>(qcur, parent) ? kInf : p.child_dist[x - n];
                 }
             }
         }
@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(kBlock) k_step_phys(StepParams p) {
                                 const int64_t nk = ((int64_t)vd + mdt - 1) / mdt - 1;
                                 for (int64_t c = 0; c < nk; ++c) atomicMin(&p.child_dist[cf - n + c], alt);
                             }
-                            want = vd > 0 && !is_queued<false>(qcur, v) &&
+                            want = vd > 0 && !is_queued<kLdRo>(qcur, v) &&
                                    !(atomicOr(&qcur[(uint32_t)v >> 5], 1u << ((uint32_t)v & 31u)) &
                                      (1u << ((uint32_t)v & 31u)));
                         }
@@ -324,21 +324,21 @@ __global__ void __launch_bounds__(kBlock) k_step_phys(StepParams p) {
 // of starts at or before its position, and its prefix / first edge come
 // from the loading lane by shuffle.  That replaces a per-edge search by a
 // few warp-wide operations per 32 edges.
-template <bool COH, class T>
+template <int LD, class T>
 __device__ __forceinline__ T ld_list(const T *p) {
-    return COH ? __ldcg(p) : __ldg(p);
+    return LD == kLdCg ? __ldcg(p) : LD == kLdRo ? __ldg(p) : *p;
 }
 
 // The list entry holding list edge w0 within [lo, hi) (scan[lo] <= w0 <
 // scan[hi], hi may be the end): a warp-wide 32-way search, 31 probes per
 // round and a ballot, so a range of up to 32^k entries takes k rounds of
 // one load latency each instead of k * 5 dependent loads.
-template <bool COH, class IT, class KT>
+template <int LD, class IT, class KT>
 __device__ __forceinline__ KT warp_search(const int32_t *scan, KT lo, KT hi, IT w0, uint32_t lane) {
     while (hi - lo > 1) {  // warp-uniform
         const KT step = (hi - lo + 31) / 32;
         const KT p = lo + step * (KT)(lane + 1);
-        const bool le = p < hi && (IT)ld_list<COH>(scan + p) <= w0;
+        const bool le = p < hi && (IT)ld_list<LD>(scan + p) <= w0;
         const KT n = (KT)__popc(__ballot_sync(kFull, le));  // probes are increasing: a prefix of lanes
         lo += step * n;
         if (lo + step < hi) hi = lo + step;
@@ -359,7 +359,7 @@ __device__ __forceinline__ KT warp_search(const int32_t *scan, KT lo, KT hi, IT 
 // inside the step (an entry has at least one edge, so at most 32 start in
 // 32 positions) and takes its fields from the window by shuffle.  32-bit
 // list edges and edge ids (< 2^31, checked when the graph is created).
-template <bool SSSP, int R, bool COH, class WB, class WS>
+template <bool SSSP, int R, int LD, class WB, class WS>
 __device__ __forceinline__ void wd_walk_win(const GraphDev &g, const NodeList &in, int64_t in_cnt, int64_t E,
                                             int64_t T, int64_t t, uint32_t *bitmap, uint32_t *qcur,
                                             uint32_t *status, uint32_t level, uint32_t *err, WB &wb,
@@ -377,11 +377,11 @@ __device__ __forceinline__ void wd_walk_win(const GraphDev &g, const NodeList &i
     // A slice that starts on a tile-start grain (every slice of a tile of
     // a multiple of 8 x 256 edges) takes its first entry from the tile
     // starts the push recorded; the load is issued with the tile's bounds.
-    const bool on_grain = wd_grain_start<SSSP, COH>() && (w0 & (int32_t)(kTileGrain - 1)) == 0;
-    const int32_t kg = on_grain ? ld_list<COH>(in.tstart + (w0 >> 8)) : 0;
-    const int64_t i0 = ld_list<COH>(in.tstart + t * q);
+    const bool on_grain = wd_grain_start<SSSP, LD>() && (w0 & (int32_t)(kTileGrain - 1)) == 0;
+    const int32_t kg = on_grain ? ld_list<LD>(in.tstart + (w0 >> 8)) : 0;
+    const int64_t i0 = ld_list<LD>(in.tstart + t * q);
     const int64_t ihi =
-        (t + 1 < ntiles) ? min((int64_t)ld_list<COH>(in.tstart + (t + 1) * q) + 1, in_cnt) : in_cnt;
+        (t + 1 < ntiles) ? min((int64_t)ld_list<LD>(in.tstart + (t + 1) * q) + 1, in_cnt) : in_cnt;
     if (i0 < 0 || i0 >= ihi) {
         if (lane == 0) atomicOr(err, kErrBounds);
         return;
@@ -400,7 +400,7 @@ __device__ __forceinline__ void wd_walk_win(const GraphDev &g, const NodeList &i
         }
         kcur = kg;
     } else {
-        kcur = warp_search<COH, uint32_t, int32_t>(in.scan, (int32_t)i0, ihiK, (uint32_t)w0, lane);
+        kcur = warp_search<LD, uint32_t, int32_t>(in.scan, (int32_t)i0, ihiK, (uint32_t)w0, lane);
     }
     int32_t kb = kcur;
     int32_t s0 = INT32_MAX, d0 = 0, s1 = INT32_MAX, d1 = 0;
@@ -410,11 +410,11 @@ __device__ __forceinline__ void wd_walk_win(const GraphDev &g, const NodeList &i
         dj = 0;
         uj = kInf;
         if (j < ihiK) {
-            sj = ld_list<COH>(in.scan + j);
-            dj = ld_list<COH>(in.beg + j) - sj;
+            sj = ld_list<LD>(in.scan + j);
+            dj = ld_list<LD>(in.beg + j) - sj;
             if (SSSP) {
-                const int32_t u = ld_list<COH>(in.v + j);
-                if (u >= 0 && (int64_t)u < g.n) uj = is_queued<COH>(qcur, u) ? kInf : ld_mut<COH>(status + u);
+                const int32_t u = ld_list<LD>(in.v + j);
+                if (u >= 0 && (int64_t)u < g.n) uj = is_queued<LD>(qcur, u) ? kInf : ld_mut<LD>(status + u);
             }
         }
     };
@@ -585,27 +585,26 @@ __device__ __forceinline__ void wd_walk_win(const GraphDev &g, const NodeList &i
     relax_group:
         if constexpr (SSSP) {
             if (o.defer == 3) {
-                relax_sssp_defer<R, COH>(ok, vv, ww, dd, status, wb, ws, cnt, o);
+                relax_sssp_defer<R, LD>(ok, vv, ww, dd, status, wb, ws, cnt, o);
                 continue;
             }
             if (cnt > WB::kCap - 32 * R) wflush<kOutNode, true>(wb, ws, cnt, o);
-            relax_items<true, R, kOutNode, true, COH, false>(ok, vv, ww, dd, g.off, bitmap, qcur, status, level, err,
+            relax_items<true, R, kOutNode, true, LD, false>(ok, vv, ww, dd, g.off, bitmap, qcur, status, level, err,
                                                              wb, ws, cnt, o);
         } else {
-            relax_bfs_lean<R, COH>(ok, vv, g.off, bitmap, status, level, wb, ws, cnt, o);
+            relax_bfs_lean<R, LD>(ok, vv, g.off, bitmap, status, level, wb, ws, cnt, o);
         }
     }
 }
 
-// One tile of the walk.  COH selects L2-coherent loads for everything other
-// CTAs write (the persistent serving and small-list kernels); the
-// single-level launches use the read-only / L1 paths.
-template <bool SSSP, int STEPS, bool COH, class WB, class WS>
+// One tile of the walk.  LD selects how everything other CTAs write is read
+// (kLdRo, kLdCg or kLdPlain).
+template <bool SSSP, int STEPS, int LD, class WB, class WS>
 __device__ __forceinline__ void wd_walk_tile(const GraphDev &g, const NodeList &in, int64_t in_cnt, int64_t E,
                                              int64_t T, int64_t t, uint32_t *bitmap, uint32_t *qcur,
                                              uint32_t *status, uint32_t level, uint32_t *err, WB &wb,
                                              WS &ws, uint32_t &cnt, const FlushOut &o) {
-    wd_walk_win<SSSP, STEPS, COH>(g, in, in_cnt, E, T, t, bitmap, qcur, status, level, err, wb, ws, cnt, o);
+    wd_walk_win<SSSP, STEPS, LD>(g, in, in_cnt, E, T, t, bitmap, qcur, status, level, err, wb, ws, cnt, o);
 }
 
 template <bool SSSP, int STEPS, class WB, class WS>
@@ -615,7 +614,7 @@ __device__ __forceinline__ void wd_walk(const StepParams &p, Ctl *ctl, const Nod
     const int64_t T = iteration_tile(E, gridDim.x, p.tile);
     const int64_t ntiles = (E + T - 1) / T;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x)
-        wd_walk_tile<SSSP, STEPS, false>(p.g, in, in_cnt, E, T, t, p.bitmap, qcur, status, level,
+        wd_walk_tile<SSSP, STEPS, kLdRo>(p.g, in, in_cnt, E, T, t, p.bitmap, qcur, status, level,
                                          &ctl->error, wb, ws, cnt, o);
 }
 
@@ -663,7 +662,8 @@ __global__ void __launch_bounds__(kBlock, SSSP ? LB_WD_MIN_BLOCKS_SSSP : LB_WD_M
 }
 
 // ---------------------------------------------------------------------------
-// Small-list levels in one persistent launch (WD).  A high-diameter graph
+// Small-list levels in one persistent launch (WD, host loop; the device loop
+// is the whole-query kernel of lb_query_wd.cu).  A high-diameter graph
 // (a grid: thousands of levels of a few thousand edges) spends most of a
 // level on the launch and the end-of-step protocol, not on edges.  While
 // the input list has at most p.small_edges edges, this kernel (one CTA per
@@ -779,7 +779,7 @@ __global__ void __launch_bounds__(kBlock, LB_SMALL_CTAS) k_small_levels(StepPara
         const int64_t T = iteration_tile(E, gridDim.x, p.tile);
         const int64_t ntiles = (E + T - 1) / T;
         for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x)
-            wd_walk_tile<SSSP, ITEMS, true>(p.g, in, in_cnt, E, T, t, p.bitmap, qcur, status, level, &ctl->error,
+            wd_walk_tile<SSSP, ITEMS, kLdCg>(p.g, in, in_cnt, E, T, t, p.bitmap, qcur, status, level, &ctl->error,
                                             s_wb[warp], ns, cnt, o);
         wflush_block<kOutNode, true>(s_wb[warp], ns, cnt, o);
         // test hook: one CTA that never arrives makes the others' waits run out
@@ -934,7 +934,7 @@ __device__ __forceinline__ void serve_range(const StepParams &p, Ctl *ctl, int64
             dd[it] = du;
         }
         if (cnt > kWB - 32 * ITEMS) wflush<OUTK, TILED>(wb, ws, cnt, o);
-        relax_items<SSSP, ITEMS, OUTK, TILED, false, false>(ok, vv, ww, dd, p.g.off, p.bitmap, qcur, status, level,
+        relax_items<SSSP, ITEMS, OUTK, TILED, kLdRo, false>(ok, vv, ww, dd, p.g.off, p.bitmap, qcur, status, level,
                                                            &ctl->error, wb, ws, cnt, o);
     }
 }
