@@ -558,9 +558,13 @@ lb_status run_query(lb_graph *g, int kind, int s, int32_t src, void *out_dev, in
         QueryArgs a;
         a.status = (uint32_t *)out_dev;
         a.src = src;
-        a.max_levels = max_levels;
+        // with a threshold (SSSP) an interval's iterations add up to at most
+        // its vertices and one more
+        a.max_levels = sssp && max_levels < 0x7FFFFFF0u ? 2u * max_levels + 64u : max_levels;
         a.time_limit_ns = time_limit_ns;
         a.number = g->query_number;
+        a.far_shift = 7;
+        while (((g->n - 1) >> a.far_shift) >= 32 * (int64_t)kFarWords) ++a.far_shift;
         a.team = small_grid(g) < grid ? small_grid(g) : grid;
         LB_CU(launch_query_wd(sssp, p, a, grid, st));
         ++g->query_number;

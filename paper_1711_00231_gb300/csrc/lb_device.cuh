@@ -11,7 +11,7 @@
 //    direction that costs an extra atomic, never one that loses an update.
 //    In the WD kernels the atomics are deferred: the relax buffers the
 //    candidates that pass the plain test, and the flush makes the atomics
-//    of a whole buffer at once (FlushOut::defer).
+//    of a whole buffer at once (FlushOutT).
 //  * Warp push buffers: the paper pushes with one atomic per node ("work
 //    chunking", Sec. II-B / IV-D).  Here a warp collects up to kWB pushed
 //    nodes in shared memory and reserves their list slots and their edges
@@ -76,7 +76,17 @@ struct WarpScratchT {
 using WarpScratch = WarpScratchT<kWB>;
 struct NoScratch {};
 
+// SSSP with a distance threshold: a vertex improved to a distance >= T is
+// not queued; the bit of its block of 2^shift vertices is set in `bits`
+// instead (see lb_query_wd.cu).  Kept in shared memory, read at the flush.
+struct FarSet {
+    uint32_t T;
+    int32_t shift;
+    uint32_t *bits;
+};
+
 struct FlushOut {
+    static constexpr int kDefer = 0;  // see FlushOutT
     NodeList list;     // node / granule output
     int32_t *elist;    // edge-id output
     unsigned long long *pack;
@@ -87,24 +97,32 @@ struct FlushOut {
     int64_t tile_cap;  // tstart entries
     int32_t tile;      // edges between recorded tile starts (kTileGrain in the hot path)
     int32_t mdt;
-    // deferred offsets (kOutNode): the pushes buffered only the vertex, and
-    // the flush loads every buffered vertex's first edge and degree from
-    // `off` (all entries at once, so one latency per flush instead of one per
-    // relax group) and drops vertices without out-edges
-    const int64_t *off = nullptr;
-    int32_t defer = 0;
-    // defer == 3 (SSSP): the buffer holds (vertex, offered distance) pairs
-    // whose plain check passed; the flush makes their atomicMin and, for
-    // the improved vertices, the queued-bit claim.
-    // defer == 2 (BFS): the buffer holds visited-check candidates, not yet
-    // claimed; the flush claims them all at once (one atomicOr per entry,
-    // every claim of the warp in flight together), writes the new level of
-    // the vertices it won and drops the rest with the vertices that have no
-    // out-edges.  The claim then leaves each relax group's chain of
-    // dependent accesses.
+    const int64_t *off = nullptr;      // deferred offsets (see FlushOutT)
     uint32_t *claim_bitmap = nullptr;
     uint32_t *claim_status = nullptr;
     uint32_t claim_level = 0;
+    const FarSet *far = nullptr;       // kDefer == 3: the distance threshold, if any
+};
+
+// What a node flush still has to do for a buffered entry, fixed at compile
+// time (a run-time field would be one more register or load in every relax
+// group):
+//   0  nothing: the entry is complete
+//   1  deferred offsets: the pushes buffered only the vertex, and the flush
+//      loads every buffered vertex's first edge and degree from `off` (all
+//      entries at once, so one latency per flush instead of one per relax
+//      group) and drops vertices without out-edges
+//   2  (BFS) the buffer holds visited-check candidates, not yet claimed; the
+//      flush claims them all at once (one atomicOr per entry, every claim of
+//      the warp in flight together), writes the new level of the vertices it
+//      won and drops the rest with the vertices that have no out-edges.  The
+//      claim then leaves each relax group's chain of dependent accesses.
+//   3  (SSSP) the buffer holds (vertex, offered distance) pairs whose plain
+//      check passed; the flush makes their atomicMin and, for the improved
+//      vertices, the queued-bit claim.
+template <int DEFER>
+struct FlushOutT : FlushOut {
+    static constexpr int kDefer = DEFER;
 };
 
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31u; }
@@ -168,11 +186,11 @@ __device__ __forceinline__ uint32_t smem_upper(const uint32_t *a, uint32_t n, ui
 
 // Output units of buffered entry i (a node list entry; with deferred
 // offsets 0 for a node without out-edges, which is dropped).
-template <int KIND, class WB>
-__device__ __forceinline__ uint32_t entry_units(const WB &b, uint32_t i, uint32_t cnt, const FlushOut &o,
+template <int KIND, class WB, class FO>
+__device__ __forceinline__ uint32_t entry_units(const WB &b, uint32_t i, uint32_t cnt, const FO &o,
                                                 uint32_t &d) {
     d = i < cnt ? b.deg[i] : 0u;
-    return (i < cnt && !(KIND == kOutNode && o.defer && d == 0u)) ? out_units<KIND>(d, o.mdt) : 0u;
+    return (i < cnt && !(KIND == kOutNode && FO::kDefer && d == 0u)) ? out_units<KIND>(d, o.mdt) : 0u;
 }
 
 // Inclusive warp scan of (u, e) pairs.
@@ -192,13 +210,13 @@ __device__ __forceinline__ void warp_scan2(uint32_t &iu, uint32_t &ie, uint32_t 
 // position / edge prefix `old` (packed entries << 32 | edges) reserved for
 // them; a node flush recomputes its prefix there with a warp scan per 32
 // entries, so it needs no scratch.
-template <int KIND, class WB, class WS>
-__device__ __forceinline__ void wflush_prefix(WB &b, WS &s, uint32_t cnt, const FlushOut &o, uint32_t &run_u,
+template <int KIND, class WB, class WS, class FO>
+__device__ __forceinline__ void wflush_prefix(WB &b, WS &s, uint32_t cnt, const FO &o, uint32_t &run_u,
                                               uint32_t &run_e) {
     const uint32_t lane = lane_id();
     run_u = 0;
     run_e = 0;
-    if (KIND == kOutNode && o.defer == 2) {
+    if (KIND == kOutNode && FO::kDefer == 2) {
         constexpr int kPer = WB::kCap / 32;
         int32_t cv[kPer];
         uint32_t pv[kPer];
@@ -226,7 +244,7 @@ __device__ __forceinline__ void wflush_prefix(WB &b, WS &s, uint32_t cnt, const 
             }
         }
         __syncwarp();
-    } else if (KIND == kOutNode && o.defer == 3) {
+    } else if (KIND == kOutNode && FO::kDefer == 3) {
         // SSSP: entry i holds a candidate vertex and the distance it was
         // offered (in beg); the atomicMin of every entry, then the queued
         // bit of every improved vertex, all in flight together
@@ -246,7 +264,10 @@ __device__ __forceinline__ void wflush_prefix(WB &b, WS &s, uint32_t cnt, const 
             const bool improved = cv[k] >= 0 && val[k] < pv[k];
             if (improved && val[k] == kSat) atomicOr(o.err, kErrSaturated);
             pv[k] = 0xFFFFFFFFu;
-            if (improved)
+            if (o.far && improved && val[k] >= o.far->T) {
+                const uint32_t blk = (uint32_t)cv[k] >> o.far->shift, bit = 1u << (blk & 31u);
+                if (!(__ldcg(o.far->bits + (blk >> 5)) & bit)) atomicOr(o.far->bits + (blk >> 5), bit);
+            } else if (improved)
                 pv[k] = atomicOr(o.claim_bitmap + ((uint32_t)cv[k] >> 5), 1u << ((uint32_t)cv[k] & 31u));
         }
 #pragma unroll
@@ -266,7 +287,7 @@ __device__ __forceinline__ void wflush_prefix(WB &b, WS &s, uint32_t cnt, const 
             }
         }
         __syncwarp();
-    } else if (KIND == kOutNode && o.defer) {
+    } else if (KIND == kOutNode && FO::kDefer) {
         // offsets are < m < 2^31 (checked when the graph is created)
         for (uint32_t i = lane; i < cnt; i += 32) {
             const int32_t v = b.v[i];
@@ -301,8 +322,8 @@ __device__ __forceinline__ void wflush_prefix(WB &b, WS &s, uint32_t cnt, const 
 
 constexpr uint32_t kLaneGrains = 8;
 
-template <int KIND, bool TILED, class WB, class WS>
-__device__ __forceinline__ void wflush_write(const WB &b, const WS &s, uint32_t &cnt, const FlushOut &o,
+template <int KIND, bool TILED, class WB, class WS, class FO>
+__device__ __forceinline__ void wflush_write(const WB &b, const WS &s, uint32_t &cnt, const FO &o,
                                              unsigned long long old, uint32_t run_u) {
     const uint32_t lane = lane_id();
     const int64_t ubase = (int64_t)(old >> 32);
@@ -321,34 +342,35 @@ __device__ __forceinline__ void wflush_write(const WB &b, const WS &s, uint32_t 
             const uint32_t u = entry_units<KIND>(b, i, cnt, o, d);
             uint32_t iu = u, ie = d;
             warp_scan2(iu, ie, lane);
+            // list positions and edge prefixes are < 2^31: 32-bit arithmetic
+            const uint32_t pos = (uint32_t)ubase + ru + iu - u;
+            const uint32_t S = (uint32_t)ebase + re + ie - d;
             if (u) {  // a node list entry (deferred offsets: one with out-edges)
-                const int64_t pos = ubase + ru + iu - u;
-                const int64_t S = ebase + re + ie - d;
                 o.list.v[pos] = b.v[i];
                 o.list.beg[pos] = b.beg[i];
                 o.list.scan[pos] = (int32_t)S;
                 if (TILED && o.tile != (int32_t)kTileGrain) {
-                    const int64_t E = S + d;
-                    for (int64_t k = (S + o.tile - 1) / o.tile; k * o.tile < E; ++k)
+                    const int64_t E = (int64_t)S + d;
+                    for (int64_t k = ((int64_t)S + o.tile - 1) / o.tile; k * o.tile < E; ++k)
                         if (k < o.tile_cap) o.list.tstart[k] = (int32_t)pos;
                 }
             }
             if (TILED && o.tile == (int32_t)kTileGrain) {
                 // the hot path: 32-bit shifts.  A lane writes up to
                 // kLaneGrains starts of its entry; a longer entry (a hub
-                // covers thousands of grains) is written by the whole warp.
-                const uint32_t S = (uint32_t)ebase + re + ie - d;
+                // covers thousands of grains) is written by the whole warp:
+                // one lane alone took 115 us for the 19 hubs behind an R-MAT
+                // scale 24 source (20 us so).
                 uint32_t k0 = (S + (uint32_t)kTileGrain - 1u) >> 8;
                 const uint32_t k1 = u ? min((S + d + (uint32_t)kTileGrain - 1u) >> 8, (uint32_t)o.tile_cap) : 0u;
-                const int32_t pos = (int32_t)((uint32_t)ubase + ru + iu - u);
                 unsigned big = __ballot_sync(kFull, k1 > k0 + kLaneGrains);
                 if (k1 > k0 && k1 <= k0 + kLaneGrains)
-                    for (; k0 < k1; ++k0) o.list.tstart[k0] = pos;
+                    for (; k0 < k1; ++k0) o.list.tstart[k0] = (int32_t)pos;
                 while (big) {
                     const int l = __ffs(big) - 1;
                     big &= big - 1;
                     const uint32_t kb = __shfl_sync(kFull, k0, l), ke = __shfl_sync(kFull, k1, l);
-                    const int32_t pl = __shfl_sync(kFull, pos, l);
+                    const int32_t pl = (int32_t)__shfl_sync(kFull, pos, l);
                     for (uint32_t k = kb + lane; k < ke; k += 32) o.list.tstart[k] = pl;
                 }
             }
@@ -374,8 +396,8 @@ __device__ __forceinline__ void wflush_write(const WB &b, const WS &s, uint32_t 
     __syncwarp();
 }
 
-template <int KIND, bool TILED, class WB, class WS>
-__device__ LB_FLUSH_INLINE void wflush(WB &b, WS &s, uint32_t &cnt, const FlushOut &o) {
+template <int KIND, bool TILED, class WB, class WS, class FO>
+__device__ LB_FLUSH_INLINE void wflush(WB &b, WS &s, uint32_t &cnt, const FO &o) {
     if (cnt == 0) return;
     if (!LB_PUSH_SYNC) __syncwarp();
     const uint32_t lane = lane_id();
@@ -397,8 +419,8 @@ __device__ LB_FLUSH_INLINE void wflush(WB &b, WS &s, uint32_t &cnt, const FlushO
 // many small pushes (a grid's SSSP wavefront) thousands of same-address
 // atomics per iteration would queue at one L2 slice.  The packed add is
 // exact: a list's entries and its edges (< m < 2^31) each fit their half.
-template <int KIND, bool TILED, class WB, class WS>
-__device__ void wflush_block(WB &b, WS &s, uint32_t &cnt, const FlushOut &o) {
+template <int KIND, bool TILED, class WB, class WS, class FO>
+__device__ void wflush_block(WB &b, WS &s, uint32_t &cnt, const FO &o) {
     __shared__ unsigned long long s_tot[kWarps];
     __shared__ unsigned long long s_base;
     const uint32_t lane = lane_id(), warp = threadIdx.x >> 5;
@@ -512,14 +534,14 @@ __device__ __forceinline__ uint32_t ld_mut(const uint32_t *p) {
 #define LB_EARLY_EXIT 1
 #endif
 // FLUSH = false: the caller flushes; then cnt + 32 * ITEMS <= capacity on entry.
-// With FlushOut::defer set (kOutNode) only the vertex is buffered.
-template <bool SSSP, int ITEMS, int KIND, bool TILED, int LD = kLdRo, bool FLUSH = true, class WB, class WS>
+// With FlushOutT<1> (kOutNode) only the vertex is buffered.
+template <bool SSSP, int ITEMS, int KIND, bool TILED, int LD = kLdRo, bool FLUSH = true, class WB, class WS, class FO>
 __device__ __forceinline__ void relax_items(const bool (&ok)[ITEMS], const int32_t (&vv)[ITEMS],
                                             const uint32_t (&ww)[ITEMS], const uint32_t (&dd)[ITEMS],
                                             const int64_t *__restrict__ off, uint32_t *__restrict__ bitmap,
                                             uint32_t *__restrict__ qcur, uint32_t *__restrict__ status,
                                             uint32_t level, uint32_t *err, WB &wb,
-                                            WS &ws, uint32_t &cnt, const FlushOut &o) {
+                                            WS &ws, uint32_t &cnt, const FO &o) {
     bool cand[ITEMS];
     uint32_t val[ITEMS];
 #pragma unroll
@@ -581,7 +603,7 @@ __device__ __forceinline__ void relax_items(const bool (&ok)[ITEMS], const int32
         for (int it = 0; it < ITEMS; ++it) any = any || won[it];
         if (!__any_sync(kFull, any)) return;
     }
-    if (KIND == kOutNode && o.defer) {
+    if (KIND == kOutNode && FO::kDefer) {
         // deferred offsets: buffer the vertex only (the flush loads its offsets)
 #pragma unroll
         for (int it = 0; it < ITEMS; ++it) {
@@ -626,24 +648,17 @@ __device__ __forceinline__ void relax_items(const bool (&ok)[ITEMS], const int32
 #ifndef LB_LEAN_PUSH_SIMPLE
 #define LB_LEAN_PUSH_SIMPLE 0
 #endif
-// Pushes of the WD walk buffer only the vertex; the flush loads the offsets
-// (FlushOut::defer).  Measured on R-MAT scale 24: BFS 2.10 -> 1.92 ms, SSSP
-// 9.35 -> 9.01 ms per query (the offset loads leave each relax group's chain
-// of dependent memory accesses, and the walk needs fewer registers).
-#ifndef LB_DEFER_OFFSETS
-#define LB_DEFER_OFFSETS 1
-#endif
 // BFS relax of R loaded edges per lane with warp-uniform early exits: the
 // visited check for every item, then (only if some lane of the warp found
 // an unvisited vertex) the claims, then (only if some lane won one) the
 // level writes, offset loads and one push of all won vertices with edges.
 // The push buffer is flushed only when this group's pushes would not fit,
 // so flushes carry close to a full buffer.  Requires R * 32 <= capacity.
-template <int R, int LD, class WB, class WS>
+template <int R, int LD, class WB, class WS, class FO>
 __device__ __forceinline__ void relax_bfs_lean(const bool (&ok)[R], const int32_t (&vv)[R],
                                                const int64_t *__restrict__ off, uint32_t *__restrict__ bitmap,
                                                uint32_t *__restrict__ status, uint32_t level, WB &wb,
-                                               WS &ws, uint32_t &cnt, const FlushOut &o) {
+                                               WS &ws, uint32_t &cnt, const FO &o) {
     static_assert(R * 32 <= WB::kCap, "push buffer too small for one group");
     uint32_t cand = 0;  // bit r: item r found v unvisited
 #pragma unroll
@@ -652,7 +667,7 @@ __device__ __forceinline__ void relax_bfs_lean(const bool (&ok)[R], const int32_
         if (!((x >> ((uint32_t)vv[r] & 31u)) & 1u)) cand |= 1u << r;
     }
     if (!__any_sync(kFull, cand != 0u)) return;
-    if (o.defer == 2) {
+    if constexpr (FO::kDefer == 2) {
         // deferred claims: buffer the candidates; the flush claims them
         unsigned bal[R];
         uint32_t tot = 0;
@@ -680,27 +695,6 @@ __device__ __forceinline__ void relax_bfs_lean(const bool (&ok)[R], const int32_
         }
     }
     if (!__any_sync(kFull, won != 0u)) return;
-    if (o.defer) {
-        // level writes, then every won vertex is buffered; the flush loads
-        // the offsets and drops vertices without out-edges
-        unsigned bal[R];
-        uint32_t tot = 0;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            if ((won >> r) & 1u) status[vv[r]] = level + 1;
-            bal[r] = __ballot_sync(kFull, (won >> r) & 1u);
-            tot += __popc(bal[r]);
-        }
-        if (cnt + tot > (uint32_t)WB::kCap) wflush<kOutNode, true>(wb, ws, cnt, o);
-        const uint32_t lt = lanemask_lt();
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            if ((bal[r] >> lane_id()) & 1u) wb.v[cnt + __popc(bal[r] & lt)] = vv[r];
-            cnt += __popc(bal[r]);
-        }
-        __syncwarp();
-        return;
-    }
     int32_t vb[R], vd[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -762,15 +756,15 @@ __device__ __forceinline__ void relax_bfs_lean(const bool (&ok)[R], const int32_
 #define LB_SSSP_STATUS_CG 0
 #endif
 // SSSP relax of R loaded edges per lane with deferred atomics
-// (FlushOut::defer == 3): the plain distance check for every item, then
+// (FlushOutT<3>): the plain distance check for every item, then
 // (only if some lane found an improvement) every candidate vertex and the
 // distance it offers go into the push buffer.  The flush makes the
 // atomicMin and queued-bit claims of a whole buffer at once.
-template <int R, int LD, class WB, class WS>
+template <int R, int LD, class WB, class WS, class FO>
 __device__ __forceinline__ void relax_sssp_defer(const bool (&ok)[R], const int32_t (&vv)[R],
                                                  const uint32_t (&ww)[R], const uint32_t (&dd)[R],
                                                  const uint32_t *__restrict__ status, WB &wb, WS &ws,
-                                                 uint32_t &cnt, const FlushOut &o) {
+                                                 uint32_t &cnt, const FO &o) {
     static_assert(R * 32 <= WB::kCap, "push buffer too small for one group");
     uint32_t cand = 0;
     uint32_t val[R];

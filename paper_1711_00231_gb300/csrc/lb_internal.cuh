@@ -88,11 +88,20 @@ struct QuerySync {
     alignas(128) uint32_t team_arrive;  // arrivals at the barrier of the small-list team
     alignas(128) uint32_t resume;       // publications of the state below (kResumeAbort: the team gave up)
     uint32_t r_level, r_par, r_cnt, r_done;
+    uint32_t r_iters, r_pull, r_T0, r_T;
     uint64_t r_edges;
     struct alignas(128) Pack {
         unsigned long long v;  // (entries << 32) | edges; bit 63: the time limit has passed
-    } pack[3];  // output counters: level L uses pack[L % 3]
+        uint32_t far_min;      // pull step: smallest distance left in the far set
+        uint32_t T;            // distance threshold from this step on
+        uint32_t delta;        // width of the next distance interval
+        uint32_t pull_size;    // expected edges a pull makes (whether the team runs it)
+    } pack[3];  // step L counts its output in pack[L % 3]
 };
+
+// Blocks of the far set's bitmap (SSSP with a distance threshold): at most
+// 32 * kFarWords blocks of 2^s >= 128 vertices.
+constexpr int32_t kFarWords = 4096;
 
 struct Ctl {
     // query parameters (written by the prepare kernel)
@@ -134,6 +143,7 @@ struct Ctl {
     uint32_t trace_len;
     uint32_t pad;
     QuerySync qsync[2];  // whole-query kernel (query number q uses qsync[q & 1])
+    uint32_t far_bits[kFarWords];  // whole-query kernel: blocks that may hold far vertices
     TraceRec trace[kTraceMax];
     uint32_t hp_hist[kHistMax];  // HP depth > 1: histogram of a sub-list (zero between uses)
 };
@@ -205,6 +215,7 @@ struct QueryArgs {
     uint64_t time_limit_ns;
     uint32_t number;  // queries launched on this workspace so far
     int32_t team;
+    int32_t far_shift;  // SSSP: blocks of 2^far_shift vertices in Ctl::far_bits
 };
 cudaError_t launch_query_wd(bool sssp, const StepParams &p, const QueryArgs &a, int grid, cudaStream_t st);
 int query_wd_blocks_per_sm(bool sssp);

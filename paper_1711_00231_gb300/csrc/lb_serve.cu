@@ -45,12 +45,6 @@ constexpr int64_t kInitChunk = 1 << 16;      // vertices reset per INIT tile
 // CTAs per SM the kernel is compiled for (the register budget); the edges
 // per thread per round in a RELAX tile (2 or 3) are a server option, one
 // kernel instance each
-// Deferred claims in the serving kernel's relax tiles (as in the WD step).
-// Measured on the 32-graph serving mix: 746 -> 904 queries/s batched, p99
-// at the Poisson rate 239 -> 208 ms.
-#ifndef LB_SERVE_DEFER_CLAIM
-#define LB_SERVE_DEFER_CLAIM 1
-#endif
 #ifndef LB_SERVE_MIN_BLOCKS
 #define LB_SERVE_MIN_BLOCKS 4
 #endif
@@ -478,7 +472,9 @@ __device__ void relax_tile(const Params &P, Slot *S, int64_t t, int64_t ntiles, 
             if (u >= 0 && (int64_t)u < g.n) atomicAnd(&qn[(uint32_t)u >> 5], ~(1u << ((uint32_t)u & 31u)));
         }
     }
-    FlushOut o;
+    // deferred claims, as in the WD step: 746 -> 904 queries/s on the 32-graph
+    // serving mix, p99 at the Poisson rate 239 -> 208 ms
+    FlushOutT<SSSP ? 3 : 2> o;
     o.list = ws_list(st.ws, W, st.par ^ 1u);
     o.elist = nullptr;
     o.pack = &S->out_pack;
@@ -490,13 +486,12 @@ __device__ void relax_tile(const Params &P, Slot *S, int64_t t, int64_t ntiles, 
     o.pushes = &S->pushes;
     o.child_first = nullptr;
     o.off = g.off;
-    o.defer = SSSP ? (LB_SERVE_DEFER_CLAIM ? 3 : LB_DEFER_OFFSETS) : (LB_SERVE_DEFER_CLAIM ? 2 : LB_DEFER_OFFSETS);
     o.claim_bitmap = SSSP ? qcur : bitmap;
     o.claim_status = st.status;
     o.claim_level = st.level;
     uint32_t cnt = 0;
-    wd_walk_tile<SSSP, ITEMS, kLdCg>(g, ws_list(st.ws, W, st.par), st.in_cnt, (int64_t)st.in_edges, q * kTileGrain,
-                                     t, bitmap, qcur, st.status, st.level, &S->error, wb, ws, cnt, o);
+    wd_walk_tile<SSSP, ITEMS, kLdCg>(g, ws_list(st.ws, W, st.par), (int32_t)st.in_cnt, (uint32_t)st.in_edges,
+                                     (uint32_t)(q * kTileGrain), (uint32_t)t, bitmap, qcur, st.status, st.level, &S->error, wb, ws, cnt, o);
 #if LB_BLOCK_FLUSH
     wflush_block<kOutNode, true>(wb, ws, cnt, o);
 #else

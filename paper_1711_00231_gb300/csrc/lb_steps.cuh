@@ -70,17 +70,11 @@ __device__ __forceinline__ uint32_t u4_get(const uint4 &x, int r) {
 #endif
 // Deferred claims in the WD step kernel: the relax only buffers the
 // candidates that pass the plain check, and the flush makes their atomics
-// for a whole buffer at once (BFS: the visited-bit claim, FlushOut::defer
-// == 2; SSSP: the atomicMin and the queued-bit claim, defer == 3).  The
+// for a whole buffer at once (BFS: the visited-bit claim, FlushOutT<2>;
+// SSSP: the atomicMin and the queued-bit claim, FlushOutT<3>).  The
 // atomics then leave each relax group's chain of dependent accesses.
 // Measured on R-MAT scale 24, 8 sources: BFS 1.93 -> 1.80 ms, SSSP 8.47
 // -> 7.69 ms per query.
-#ifndef LB_BFS_DEFER_CLAIM
-#define LB_BFS_DEFER_CLAIM 1
-#endif
-#ifndef LB_SSSP_DEFER_CLAIM
-#define LB_SSSP_DEFER_CLAIM 1
-#endif
 
 // Runs through long adjacency lists: after the first group of a run, the
 // following groups of the same entry skip the window and bounds work, and
@@ -113,13 +107,6 @@ template <bool SSSP, int LD>
 __host__ __device__ constexpr bool wd_grain_start() {
     return LB_WD_GRAIN_START && (SSSP || LD != 0);
 }
-// Deferred claims in the persistent small-list kernel (as in the WD step;
-// bit mask: 1 = SSSP, 2 = BFS).  Measured on the 4096^2 grid: BFS equal,
-// SSSP 2% slower with them (408 -> 416 ms), so BFS only.
-#ifndef LB_SMALL_DEFER_CLAIM
-#define LB_SMALL_DEFER_CLAIM 2
-#endif
-
 // The final flush of a WD iteration (and of a serving RELAX tile) as one
 // list reservation per CTA (wflush_block) instead of one per warp.
 #ifndef LB_BLOCK_FLUSH
@@ -359,48 +346,46 @@ __device__ __forceinline__ KT warp_search(const int32_t *scan, KT lo, KT hi, IT 
 // inside the step (an entry has at least one edge, so at most 32 start in
 // 32 positions) and takes its fields from the window by shuffle.  32-bit
 // list edges and edge ids (< 2^31, checked when the graph is created).
-template <bool SSSP, int R, int LD, class WB, class WS>
-__device__ __forceinline__ void wd_walk_win(const GraphDev &g, const NodeList &in, int64_t in_cnt, int64_t E,
-                                            int64_t T, int64_t t, uint32_t *bitmap, uint32_t *qcur,
+template <bool SSSP, int R, int LD, class WB, class WS, class FO>
+__device__ __forceinline__ void wd_walk_win(const GraphDev &g, const NodeList &in, int32_t in_cnt, uint32_t E,
+                                            uint32_t T, uint32_t t, uint32_t *bitmap, uint32_t *qcur,
                                             uint32_t *status, uint32_t level, uint32_t *err, WB &wb,
-                                            WS &ws, uint32_t &cnt, const FlushOut &o) {
-    const int64_t q = T / kTileGrain;
-    const int64_t W = T / kWarps;  // edges per warp and tile (a multiple of 32)
-    const int64_t ntiles = (E + T - 1) / T;
+                                            WS &ws, uint32_t &cnt, const FO &o) {
+    // 32-bit tile arithmetic: a list has < 2^31 edges and a tile <= 32768
+    const uint32_t q = T / (uint32_t)kTileGrain;
+    const uint32_t W = T / kWarps;  // edges per warp and tile (a multiple of 32)
     const uint32_t lane = lane_id();
     const uint32_t warp = threadIdx.x >> 5;
-    const int64_t e0 = t * T;
-    const int64_t e1 = min(e0 + T, E);
-    const int64_t w064 = e0 + (int64_t)warp * W;
-    if (w064 >= e1) return;  // warp-uniform
-    const int32_t w0 = (int32_t)w064;
+    const uint32_t e0 = t * T;
+    const uint32_t e1 = min(e0 + T, E);
+    const uint32_t w0u = e0 + warp * W;
+    if (w0u >= e1) return;  // warp-uniform
+    const int32_t w0 = (int32_t)w0u;
     // A slice that starts on a tile-start grain (every slice of a tile of
     // a multiple of 8 x 256 edges) takes its first entry from the tile
     // starts the push recorded; the load is issued with the tile's bounds.
     const bool on_grain = wd_grain_start<SSSP, LD>() && (w0 & (int32_t)(kTileGrain - 1)) == 0;
     const int32_t kg = on_grain ? ld_list<LD>(in.tstart + (w0 >> 8)) : 0;
-    const int64_t i0 = ld_list<LD>(in.tstart + t * q);
-    const int64_t ihi =
-        (t + 1 < ntiles) ? min((int64_t)ld_list<LD>(in.tstart + (t + 1) * q) + 1, in_cnt) : in_cnt;
-    if (i0 < 0 || i0 >= ihi) {
+    const int32_t i0 = ld_list<LD>(in.tstart + t * q);
+    const int32_t ihiK = e0 + T < E ? min(ld_list<LD>(in.tstart + (t + 1u) * q) + 1, in_cnt) : in_cnt;
+    if (i0 < 0 || i0 >= ihiK) {
         if (lane == 0) atomicOr(err, kErrBounds);
         return;
     }
-    const int32_t w1 = (int32_t)min(w064 + W, e1);
-    const int32_t ihiK = (int32_t)ihi;
+    const int32_t w1 = (int32_t)min(w0u + W, e1);
     const int32_t m = (int32_t)g.m;
     const bool vec_ok = wd_vec<SSSP, R>() &&
                         ((reinterpret_cast<uintptr_t>(g.col) | (SSSP ? reinterpret_cast<uintptr_t>(g.w) : 0u)) &
                          15u) == 0;
     int32_t kcur;
     if (on_grain) {
-        if (kg < (int32_t)i0 || kg >= ihiK) {
+        if (kg < i0 || kg >= ihiK) {
             if (lane == 0) atomicOr(err, kErrBounds);
             return;
         }
         kcur = kg;
     } else {
-        kcur = warp_search<LD, uint32_t, int32_t>(in.scan, (int32_t)i0, ihiK, (uint32_t)w0, lane);
+        kcur = warp_search<LD, uint32_t, int32_t>(in.scan, i0, ihiK, (uint32_t)w0, lane);
     }
     int32_t kb = kcur;
     int32_t s0 = INT32_MAX, d0 = 0, s1 = INT32_MAX, d1 = 0;
@@ -583,14 +568,12 @@ __device__ __forceinline__ void wd_walk_win(const GraphDev &g, const NodeList &i
         }
         }
     relax_group:
-        if constexpr (SSSP) {
-            if (o.defer == 3) {
-                relax_sssp_defer<R, LD>(ok, vv, ww, dd, status, wb, ws, cnt, o);
-                continue;
-            }
+        if constexpr (SSSP && FO::kDefer == 3) {
+            relax_sssp_defer<R, LD>(ok, vv, ww, dd, status, wb, ws, cnt, o);
+        } else if constexpr (SSSP) {
             if (cnt > WB::kCap - 32 * R) wflush<kOutNode, true>(wb, ws, cnt, o);
             relax_items<true, R, kOutNode, true, LD, false>(ok, vv, ww, dd, g.off, bitmap, qcur, status, level, err,
-                                                             wb, ws, cnt, o);
+                                                            wb, ws, cnt, o);
         } else {
             relax_bfs_lean<R, LD>(ok, vv, g.off, bitmap, status, level, wb, ws, cnt, o);
         }
@@ -599,22 +582,22 @@ __device__ __forceinline__ void wd_walk_win(const GraphDev &g, const NodeList &i
 
 // One tile of the walk.  LD selects how everything other CTAs write is read
 // (kLdRo, kLdCg or kLdPlain).
-template <bool SSSP, int STEPS, int LD, class WB, class WS>
-__device__ __forceinline__ void wd_walk_tile(const GraphDev &g, const NodeList &in, int64_t in_cnt, int64_t E,
-                                             int64_t T, int64_t t, uint32_t *bitmap, uint32_t *qcur,
+template <bool SSSP, int STEPS, int LD, class WB, class WS, class FO>
+__device__ __forceinline__ void wd_walk_tile(const GraphDev &g, const NodeList &in, int32_t in_cnt, uint32_t E,
+                                             uint32_t T, uint32_t t, uint32_t *bitmap, uint32_t *qcur,
                                              uint32_t *status, uint32_t level, uint32_t *err, WB &wb,
-                                             WS &ws, uint32_t &cnt, const FlushOut &o) {
+                                             WS &ws, uint32_t &cnt, const FO &o) {
     wd_walk_win<SSSP, STEPS, LD>(g, in, in_cnt, E, T, t, bitmap, qcur, status, level, err, wb, ws, cnt, o);
 }
 
-template <bool SSSP, int STEPS, class WB, class WS>
+template <bool SSSP, int STEPS, class WB, class WS, class FO>
 __device__ __forceinline__ void wd_walk(const StepParams &p, Ctl *ctl, const NodeList &in, int64_t in_cnt, int64_t E,
-                                        WB &wb, WS &ws, uint32_t &cnt, const FlushOut &o,
+                                        WB &wb, WS &ws, uint32_t &cnt, const FO &o,
                                         uint32_t *status, uint32_t level, uint32_t *qcur) {
-    const int64_t T = iteration_tile(E, gridDim.x, p.tile);
-    const int64_t ntiles = (E + T - 1) / T;
-    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x)
-        wd_walk_tile<SSSP, STEPS, kLdRo>(p.g, in, in_cnt, E, T, t, p.bitmap, qcur, status, level,
+    const uint32_t T = (uint32_t)iteration_tile(E, gridDim.x, p.tile);
+    const uint32_t ntiles = ((uint32_t)E + T - 1u) / T;
+    for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x)
+        wd_walk_tile<SSSP, STEPS, kLdRo>(p.g, in, (int32_t)in_cnt, (uint32_t)E, T, t, p.bitmap, qcur, status, level,
                                          &ctl->error, wb, ws, cnt, o);
 }
 
@@ -635,7 +618,7 @@ __global__ void __launch_bounds__(kBlock, SSSP ? LB_WD_MIN_BLOCKS_SSSP : LB_WD_M
     if (SSSP) clear_next_queued(p.bitmap, p.bm_words, level);
     uint32_t *status = ctl->status;
     const NodeList in = p.lists[par];
-    FlushOut o;
+    FlushOutT<SSSP ? 3 : 2> o;
     o.list = p.lists[par ^ 1u];
     o.elist = nullptr;
     o.pack = &ctl->out_pack;
@@ -646,7 +629,6 @@ __global__ void __launch_bounds__(kBlock, SSSP ? LB_WD_MIN_BLOCKS_SSSP : LB_WD_M
     o.err = &ctl->error;
     o.pushes = &ctl->pushes;
     o.off = p.g.off;
-    o.defer = SSSP ? (LB_SSSP_DEFER_CLAIM ? 3 : LB_DEFER_OFFSETS) : (LB_BFS_DEFER_CLAIM ? 2 : LB_DEFER_OFFSETS);
     o.claim_bitmap = SSSP ? qcur : p.bitmap;
     o.claim_status = status;
     o.claim_level = level;
@@ -758,7 +740,9 @@ __global__ void __launch_bounds__(kBlock, LB_SMALL_CTAS) k_small_levels(StepPara
             }
         }
         if (blockIdx.x == 0 && threadIdx.x == 0) ctl->small_pack[(level + 1u) % 3u] = 0ull;
-        FlushOut o;
+        // deferred claims: BFS equal, SSSP 2% slower with them on the 4096^2
+        // grid (408 -> 416 ms), so SSSP defers only the offsets
+        FlushOutT<SSSP ? 1 : 2> o;
         o.list = p.lists[par ^ 1u];
         o.elist = nullptr;
         o.pack = &ctl->small_pack[level % 3u];
@@ -770,16 +754,14 @@ __global__ void __launch_bounds__(kBlock, LB_SMALL_CTAS) k_small_levels(StepPara
         o.pushes = &ctl->pushes;
         o.child_first = nullptr;
         o.off = p.g.off;
-        o.defer = SSSP ? ((LB_SMALL_DEFER_CLAIM & 1) ? 3 : LB_DEFER_OFFSETS)
-                       : ((LB_SMALL_DEFER_CLAIM & 2) ? 2 : LB_DEFER_OFFSETS);
         o.claim_bitmap = SSSP ? qcur : p.bitmap;
         o.claim_status = status;
         o.claim_level = level;
         uint32_t cnt = 0;
-        const int64_t T = iteration_tile(E, gridDim.x, p.tile);
-        const int64_t ntiles = (E + T - 1) / T;
-        for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x)
-            wd_walk_tile<SSSP, ITEMS, kLdCg>(p.g, in, in_cnt, E, T, t, p.bitmap, qcur, status, level, &ctl->error,
+        const uint32_t T = (uint32_t)iteration_tile(E, gridDim.x, p.tile);
+        const uint32_t ntiles = ((uint32_t)E + T - 1u) / T;
+        for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x)
+            wd_walk_tile<SSSP, ITEMS, kLdCg>(p.g, in, (int32_t)in_cnt, (uint32_t)E, T, t, p.bitmap, qcur, status, level, &ctl->error,
                                             s_wb[warp], ns, cnt, o);
         wflush_block<kOutNode, true>(s_wb[warp], ns, cnt, o);
         // test hook: one CTA that never arrives makes the others' waits run out
@@ -916,10 +898,10 @@ __global__ void __launch_bounds__(kBlock) k_step_ep(StepParams p) {
 // Edges first + lane + k * stride (< last) of one node, relaxed ITEMS per
 // lane at a time from source distance du (the warp and CTA bins of the
 // degree-binned HP step).  first, last and stride are warp-uniform.
-template <bool SSSP, int ITEMS, int OUTK = kOutNode, bool TILED = true>
+template <bool SSSP, int ITEMS, int OUTK = kOutNode, bool TILED = true, class FO>
 __device__ __forceinline__ void serve_range(const StepParams &p, Ctl *ctl, int64_t first, int64_t last, int64_t stride,
                                             uint32_t du, uint32_t *status, uint32_t level, uint32_t *qcur,
-                                            WarpBuf &wb, WarpScratch &ws, uint32_t &cnt, const FlushOut &o) {
+                                            WarpBuf &wb, WarpScratch &ws, uint32_t &cnt, const FO &o) {
     const uint32_t lane = lane_id();
     for (int64_t e0 = first; e0 < last; e0 += stride * ITEMS) {
         bool ok[ITEMS];
@@ -947,10 +929,10 @@ __device__ __forceinline__ void serve_range(const StepParams &p, Ctl *ctl, int64
 // (the CTA bin is a block-local list; when it is full the warp serves the
 // entry instead).  OUTK / TILED: what the pushes write (nodes with tile
 // starts for HP, granules for NS).  Every thread of the block calls it.
-template <bool SSSP, int ITEMS, int OUTK, bool TILED>
+template <bool SSSP, int ITEMS, int OUTK, bool TILED, class FO>
 __device__ __forceinline__ void binned_step(const StepParams &p, Ctl *ctl, const NodeList &in, int64_t in_cnt,
                                             int64_t tmax, uint32_t *status, uint32_t level, uint32_t *qcur,
-                                            WarpBuf &wb, WarpScratch &ws, uint32_t &cnt, const FlushOut &o) {
+                                            WarpBuf &wb, WarpScratch &ws, uint32_t &cnt, const FO &o) {
     constexpr int kBigCap = 256;
     __shared__ int32_t s_big[kBigCap];
     __shared__ uint32_t s_nbig;

@@ -70,3 +70,59 @@ def test_grid_and_team_sizes(opts):
             check(G, g, src)
         finally:
             G.close()
+
+
+def far_graph(kind):
+    # uniform random graphs whose lists grow past the threshold rule's size
+    # early; n is not a multiple of the far set's 128-vertex blocks
+    g = gg.erdos_renyi(300001, 1200000, seed=6)
+    r = np.random.default_rng(4)
+    if kind == "zero":
+        g.weights[:] = r.integers(0, 9, g.m)
+    elif kind == "gaps":
+        g.weights[:] = np.where(r.random(g.m) < 0.5, 1, 1 << 20)
+    elif kind == "equal":
+        g.weights[:] = 1
+    elif kind == "overflow":
+        g.weights[:] = r.integers(1 << 28, 1 << 31, g.m)
+    return g
+
+
+@pytest.mark.parametrize("kind", ["uniform", "zero", "gaps", "equal", "overflow"])
+def test_sssp_distance_threshold(kind):
+    import torch
+    g = far_graph(kind)
+    G = lb.Graph.from_csr(g)
+    try:
+        src = int(gg.pick_sources(g, 1, seed=3)[0])
+        ref, ov = oracle.dijkstra(g, src)
+        d, rc = G.sssp(src, "WD")
+        assert rc == (lb.LB_ERR_OVERFLOW if ov else lb.LB_OK) and np.array_equal(d, ref)
+        assert ov == (kind == "overflow")
+        relaxed = G.stats()["edges_relaxed"]
+        # any 4-byte alignment of the caller's buffer
+        buf = torch.empty(g.n + 1, dtype=torch.int32, device="cuda")
+        G.sssp_dev(src, "WD", buf[1:], None, torch.cuda.current_stream())
+        torch.cuda.synchronize()
+        assert np.array_equal(buf[1:].cpu().numpy().view(np.uint32), ref)
+        if kind == "uniform":
+            # the host loop keeps the plain order: the threshold was in force
+            G.set_options(loop_mode=1)
+            G.sssp(src, "WD")
+            assert relaxed < 0.8 * G.stats()["edges_relaxed"]
+    finally:
+        G.close()
+
+
+def test_sssp_distance_threshold_on_a_grid():
+    # high diameter: the threshold comes in after 32 iterations, the intervals
+    # widen, and lists move between the team and the whole grid
+    g = gg.grid(900, 1100, seed=2)
+    G = lb.Graph.from_csr(g)
+    try:
+        for opts in (dict(), dict(small_edges=0), dict(small_edges=2000, ctas_per_sm=1)):
+            G.set_options(**opts)
+            d, rc = G.sssp(450 * 1100 + 7, "WD")
+            assert rc == lb.LB_OK and np.array_equal(d, oracle.dijkstra(g, 450 * 1100 + 7)[0])
+    finally:
+        G.close()
