@@ -163,7 +163,8 @@ typedef struct lb_mem_stats {
                               cols/weights arrays, not duplicated) */
     int64_t edge_lists;    /* EP: edge worklists (two buffers of m ids) */
     int64_t sub_lists;     /* HP: sub-worklists (two buffers) */
-    int64_t control;       /* counters, step trace */
+    int64_t control;       /* counters, step trace; WD: list segments of the
+                              small-list team (2 MiB) */
     int64_t extra_total;   /* sum of the fields from status to control */
     int64_t base_total;    /* csr_offsets + csr_cols + csr_weights */
     int64_t resident;      /* bytes this graph holds on the device now */

@@ -79,6 +79,11 @@ struct DeviceGuard {
 };
 
 constexpr int kStrategies = 7;
+// WD, fast levels: entries per CTA segment (lists of small graphs are short:
+// less to allocate in the first query), and 16-byte list entries in all, one
+// of them to align the rest (a custom allocator may return any address)
+int32_t fast_seg_cap(int64_t n) { return n <= 32768 ? 256 : kFastSeg; }
+int64_t fast_entries(int64_t n) { return 2 * (int64_t)kFastTeam * fast_seg_cap(n) + 1; }
 
 // Default small_edges.
 #ifndef LB_SMALL_EDGES_DEFAULT
@@ -131,10 +136,12 @@ struct lb_graph {
     // workspace (lazily allocated)
     Ctl *ctl = nullptr;
     uint32_t *bitmap = nullptr;  // bitmap_alloc_words(n): two halves (BFS visited bits / SSSP queued bits) + placement slack
+    int4 *fast_seg = nullptr;    // WD: list segments of the fast levels (fast_entries)
     uint32_t *out_internal = nullptr;  // result buffer of host-output queries
     int32_t *par_internal = nullptr;
     NodeList lists[2]{};
     NodeList subs[2]{};
+    int64_t lists_bytes = 0, subs_bytes = 0;  // of the two pairs' allocations
     int64_t list_cap = 0;
     int64_t tile_cap = 0;
     bool have_tiles = false;
@@ -262,40 +269,46 @@ void drop_execs(lb_graph *g) {
             }
 }
 
-void free_lists(lb_graph *g, NodeList *L, int64_t cap, int64_t tcap) {
-    for (int b = 0; b < 2; ++b) {
-        g->release(L[b].v, cap);
-        g->release(L[b].beg, cap);
-        g->release(L[b].scan, cap + 1);
-        g->release(L[b].tstart, tcap);
-    }
+// Both buffers of a worklist live in one allocation, each piece on a
+// 256-byte step of it: cudaMalloc takes about 30 us from 1 MiB up, and a
+// first query would make eight of them per pair.
+int64_t step256(int64_t bytes) { return (bytes + 255) / 256 * 256; }
+
+void free_lists(lb_graph *g, NodeList *L, int64_t &bytes) {
+    unsigned char *block = (unsigned char *)L[0].v;
+    g->release(block, bytes);
+    L[0] = L[1] = NodeList{};
+    bytes = 0;
 }
 
-// On a failed allocation the lists allocated so far are released, so the
-// next attempt starts from nothing.
-lb_status alloc_lists(lb_graph *g, NodeList *L, int64_t cap, int64_t tcap, bool tiles) {
-    lb_status st = LB_OK;
-    for (int b = 0; b < 2 && st == LB_OK; ++b) {
-        st = g->alloc(&L[b].v, cap);
-        if (st == LB_OK) st = g->alloc(&L[b].beg, cap);
-        if (st == LB_OK) st = g->alloc(&L[b].scan, cap + 1);
-        if (st == LB_OK && tiles) st = g->alloc(&L[b].tstart, tcap);
+lb_status alloc_lists(lb_graph *g, NodeList *L, int64_t &bytes, int64_t cap, int64_t tcap, bool tiles) {
+    const int64_t entry = step256(4 * (cap > 0 ? cap : 1)), scan = step256(4 * (cap + 1));
+    const int64_t ts = tiles ? step256(4 * tcap) : 0, one = 2 * entry + scan + ts;
+    unsigned char *block = nullptr;
+    LB_TRY(g->alloc(&block, 2 * one));
+    bytes = 2 * one;
+    for (int b = 0; b < 2; ++b) {
+        unsigned char *q = block + b * one;
+        L[b].v = (int32_t *)q;
+        L[b].beg = (int32_t *)(q + entry);
+        L[b].scan = (int32_t *)(q + 2 * entry);
+        L[b].tstart = tiles ? (int32_t *)(q + 2 * entry + scan) : nullptr;
     }
-    if (st != LB_OK) free_lists(g, L, cap, tcap);
-    return st;
+    return LB_OK;
 }
 
 void free_workspace(lb_graph *g) {
     drop_execs(g);
     g->release(g->ctl, 1);
     g->release(g->bitmap, bitmap_alloc_words(g->n));
+    g->release(g->fast_seg, fast_entries(g->n));
     g->release(g->out_internal, g->n);
     g->release(g->out_internal2, g->n);
     g->release(g->batch_err, g->batch_err_cap);
     g->batch_err_cap = 0;
     g->release(g->par_internal, g->n);
-    free_lists(g, g->lists, g->list_cap, g->tile_cap);
-    free_lists(g, g->subs, g->n, g->tile_cap);
+    free_lists(g, g->lists, g->lists_bytes);
+    free_lists(g, g->subs, g->subs_bytes);
     g->list_cap = 0;
     g->have_tiles = false;
     g->have_subs = false;
@@ -352,6 +365,7 @@ lb_status ensure_workspace(lb_graph *g, int s) {
     if (!g->ctl) {
         LB_TRY(g->alloc(&g->ctl, 1));
         LB_CU(cudaMemsetAsync(g->ctl, 0, sizeof(Ctl), g->stream));
+        LB_CU(launch_team_pick(g->ctl, g->sms, g->stream));
     }
     if (!g->bitmap) LB_TRY(g->alloc(&g->bitmap, bitmap_alloc_words(g->n)));
     if (s == LB_NS || s == LB_NS_PHYS || s == LB_HP) LB_TRY(ensure_mdt(g));
@@ -391,25 +405,26 @@ lb_status ensure_workspace(lb_graph *g, int s) {
     if (g->list_cap < cap || (tiles && (!g->have_tiles || g->tile_cap != tcap))) {
         quiesce(g);
         drop_execs(g);
-        free_lists(g, g->lists, g->list_cap, g->tile_cap);
+        free_lists(g, g->lists, g->lists_bytes);
         const int64_t newcap = cap > g->list_cap ? cap : g->list_cap;
         const bool want_tiles = tiles || g->have_tiles;
         if (g->have_subs) {
-            free_lists(g, g->subs, g->n, g->tile_cap);
+            free_lists(g, g->subs, g->subs_bytes);
             g->have_subs = false;
         }
         g->list_cap = 0;
         g->have_tiles = false;
         g->tile_cap = tcap;
-        LB_TRY(alloc_lists(g, g->lists, newcap, tcap, want_tiles));
+        LB_TRY(alloc_lists(g, g->lists, g->lists_bytes, newcap, tcap, want_tiles));
         g->list_cap = newcap;
         g->have_tiles = want_tiles;
     }
+    if (s == LB_WD && !g->fast_seg) LB_TRY(g->alloc(&g->fast_seg, fast_entries(g->n)));
     if (s == LB_HP && !g->have_subs) {
         quiesce(g);
         drop_execs(g);
-        free_lists(g, g->subs, g->n, g->tile_cap);
-        LB_TRY(alloc_lists(g, g->subs, g->n, g->tile_cap, true));
+        free_lists(g, g->subs, g->subs_bytes);
+        LB_TRY(alloc_lists(g, g->subs, g->subs_bytes, g->n, g->tile_cap, true));
         g->have_subs = true;
     }
     return LB_OK;
@@ -563,9 +578,11 @@ lb_status run_query(lb_graph *g, int kind, int s, int32_t src, void *out_dev, in
         a.max_levels = sssp && max_levels < 0x7FFFFFF0u ? 2u * max_levels + 64u : max_levels;
         a.time_limit_ns = time_limit_ns;
         a.number = g->query_number;
-        a.far_shift = 7;
+        a.seg_cap = fast_seg_cap(g->n);
+        a.far_shift = 5;
         while (((g->n - 1) >> a.far_shift) >= 32 * (int64_t)kFarWords) ++a.far_shift;
-        a.team = small_grid(g) < grid ? small_grid(g) : grid;
+        a.team = kFastTeam < grid ? kFastTeam : grid;
+        a.fast_seg = a.team == kFastTeam ? (int4 *)(((uintptr_t)g->fast_seg + 15u) & ~(uintptr_t)15u) : nullptr;
         LB_CU(launch_query_wd(sssp, p, a, grid, st));
         ++g->query_number;
         if (parents_dev) LB_CU(launch_parents(p, sssp, parents_dev, st));
@@ -986,7 +1003,7 @@ lb_status lb_mem_report(lb_graph *g, lb_strategy s, lb_mem_stats *out) {
         if (s == LB_WD || s == LB_HP) out->tile_starts = 2 * 4 * tcap;
         if (s == LB_HP) out->sub_lists = 2 * (4 * n + 4 * n + 4 * (n + 1) + 4 * tcap);
     }
-    out->control = (int64_t)sizeof(Ctl);
+    out->control = (int64_t)sizeof(Ctl) + (s == LB_WD ? fast_entries(n) * (int64_t)sizeof(int4) : 0);
     out->extra_total = out->status + out->visited + out->node_lists + out->tile_starts + out->coo_src +
                        out->edge_lists + out->sub_lists + out->control + out->ns_split;
     out->resident = g->resident;

@@ -101,6 +101,9 @@ struct FlushOut {
     uint32_t *claim_bitmap = nullptr;
     uint32_t *claim_status = nullptr;
     uint32_t claim_level = 0;
+    // node output: if set (shared memory), takes the largest degree of what
+    // the block flush writes, or kInf when a warp flushed before (a long list)
+    uint32_t *maxdeg = nullptr;
     const FarSet *far = nullptr;       // kDefer == 3: the distance threshold, if any
 };
 
@@ -409,6 +412,7 @@ __device__ LB_FLUSH_INLINE void wflush(WB &b, WS &s, uint32_t &cnt, const FO &o)
         if (o.pushes) atomicAdd(o.pushes, (unsigned long long)run_u);
     }
     old = __shfl_sync(kFull, old, 0);
+    if (KIND == kOutNode && o.maxdeg && lane == 0) atomicMax(o.maxdeg, kInf);
     __syncwarp();
     wflush_write<KIND, TILED>(b, s, cnt, o, old, run_u);
 }
@@ -427,6 +431,12 @@ __device__ void wflush_block(WB &b, WS &s, uint32_t &cnt, const FO &o) {
     __syncwarp();
     uint32_t run_u = 0, run_e = 0;
     if (cnt) wflush_prefix<KIND>(b, s, cnt, o, run_u, run_e);
+    if (KIND == kOutNode && o.maxdeg) {
+        uint32_t md = 0;
+        for (uint32_t i = lane; i < cnt; i += 32) md = max(md, b.deg[i]);
+        md = __reduce_max_sync(kFull, md);
+        if (lane == 0) atomicMax(o.maxdeg, md);
+    }
     if (lane == 0) s_tot[warp] = ((unsigned long long)run_u << 32) | (unsigned long long)run_e;
     __syncthreads();
     if (threadIdx.x == 0) {

@@ -78,6 +78,31 @@ struct TraceRec {
 #else
 #define LB_CTL_ALIGN
 #endif
+#ifndef LB_FAST_TEAM
+#define LB_FAST_TEAM 64
+#endif
+#ifndef LB_FAST_SEG
+#define LB_FAST_SEG 2048
+#endif
+constexpr int kFastTeam = LB_FAST_TEAM;  // CTAs of the small-list team (a multiple of 32)
+constexpr int kFastSeg = LB_FAST_SEG;    // entries per CTA segment of a fast level's list (two buffers)
+
+constexpr uint32_t kMaxSms = 512;
+constexpr uint32_t kNoRank = 0xFFFFFFFFu;
+
+// Loop state of the whole-query WD kernel, the same in every CTA of a step.
+struct QueryLoop {
+    uint32_t level, par;      // step index (picks counters and queued bits); input list
+    uint32_t cnt, edges;      // the input list's entries and edges
+    uint32_t maxdeg;          // its largest entry (0: not known)
+    uint32_t done, iters;     // iterations so far (pull steps do not count)
+    // SSSP threshold (lb_query_wd.cu): in force, from where a pull step
+    // starts, whether the next step is one, width of the next interval
+    uint32_t T, T0, pull, delta, delta_min, engaged;
+    uint32_t int_lists, int_max;       // the current interval's lists, largest list
+    uint64_t relaxed, int_edges;       // edges listed, in all and in this interval
+};
+
 // Synchronisation words of the whole-query WD kernel, each on a 128-byte
 // line of its own.  All of them must be zero when a query starts: query q
 // uses qsync[q & 1] and clears qsync[(q + 1) & 1], so a query that ended at
@@ -86,22 +111,22 @@ struct QuerySync {
     alignas(128) uint32_t full_arrive;  // arrivals at the barrier of the whole grid, ever increasing
     alignas(128) uint32_t full_release; // barriers of the whole grid completed
     alignas(128) uint32_t team_arrive;  // arrivals at the barrier of the small-list team
-    alignas(128) uint32_t resume;       // publications of the state below (kResumeAbort: the team gave up)
-    uint32_t r_level, r_par, r_cnt, r_done;
-    uint32_t r_iters, r_pull, r_T0, r_T;
-    uint64_t r_edges;
+    alignas(128) uint32_t resume;       // publications of `loop` (kResumeAbort: a wait ran out)
+    alignas(128) QueryLoop loop;
+    uint32_t delta0;                    // SSSP: first interval width
     struct alignas(128) Pack {
         unsigned long long v;  // (entries << 32) | edges; bit 63: the time limit has passed
         uint32_t far_min;      // pull step: smallest distance left in the far set
-        uint32_t T;            // distance threshold from this step on
-        uint32_t delta;        // width of the next distance interval
-        uint32_t pull_size;    // expected edges a pull makes (whether the team runs it)
+        uint32_t maxdeg;       // largest degree listed
     } pack[3];  // step L counts its output in pack[L % 3]
+    alignas(128) unsigned long long fast_pack[2];  // fast levels: list counter of the way back
+    alignas(128) uint32_t team_here;  // team ranks taken
+    uint32_t sm_ctas[kMaxSms];        // CTAs per SM
 };
 
 // Blocks of the far set's bitmap (SSSP with a distance threshold): at most
-// 32 * kFarWords blocks of 2^s >= 128 vertices.
-constexpr int32_t kFarWords = 4096;
+// 32 * kFarWords blocks of 2^s >= 32 vertices.
+constexpr int32_t kFarWords = 16384;
 
 struct Ctl {
     // query parameters (written by the prepare kernel)
@@ -143,10 +168,24 @@ struct Ctl {
     uint32_t trace_len;
     uint32_t pad;
     QuerySync qsync[2];  // whole-query kernel (query number q uses qsync[q & 1])
+    // fast levels: a word per CTA and exchange (one set: a query clears it
+    // before its first barrier), each SM's rank in the team.  The words lie
+    // in one 4 KiB page (fast_words), which one half of the L2 holds.
+    unsigned long long fast_area[4 * kFastTeam];
+    uint32_t sm_rank[kMaxSms];
+    uint32_t team_done;
     uint32_t far_bits[kFarWords];  // whole-query kernel: blocks that may hold far vertices
     TraceRec trace[kTraceMax];
     uint32_t hp_hist[kHistMax];  // HP depth > 1: histogram of a sub-list (zero between uses)
 };
+
+// The 2 x kFastTeam words of the fast levels, on a boundary of their size.
+__host__ __device__ inline unsigned long long *fast_words(Ctl *c) {
+    constexpr uintptr_t kBytes = 2 * kFastTeam * sizeof(unsigned long long);
+    static_assert(kBytes <= 4096 && (kBytes & (kBytes - 1)) == 0, "one page");
+    return reinterpret_cast<unsigned long long *>((reinterpret_cast<uintptr_t>(c->fast_area) + kBytes - 1) &
+                                                  ~(kBytes - 1));
+}
 
 struct GraphDev {
     const int64_t *off;
@@ -215,10 +254,13 @@ struct QueryArgs {
     uint64_t time_limit_ns;
     uint32_t number;  // queries launched on this workspace so far
     int32_t team;
+    int4 *fast_seg;     // 2 * kFastTeam * seg_cap entries (NULL: no fast levels)
+    int32_t seg_cap;    // entries per CTA segment, at most kFastSeg
     int32_t far_shift;  // SSSP: blocks of 2^far_shift vertices in Ctl::far_bits
 };
 cudaError_t launch_query_wd(bool sssp, const StepParams &p, const QueryArgs &a, int grid, cudaStream_t st);
 int query_wd_blocks_per_sm(bool sssp);
+cudaError_t launch_team_pick(Ctl *ctl, int sms, cudaStream_t st);  // once per zeroed Ctl
 cudaError_t launch_finish_query(const StepParams &p, cudaStream_t st);
 cudaError_t launch_coo_build(const GraphDev &g, int32_t *coo_src, cudaStream_t st);
 cudaError_t launch_mdt(const GraphDev &g, int32_t bins, unsigned long long *scratch, int64_t *result,

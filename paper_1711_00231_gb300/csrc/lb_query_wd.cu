@@ -57,16 +57,19 @@ __device__ __forceinline__ uint32_t add_acq_rel(uint32_t *p, uint32_t v) {
 __device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
 // Waits until *p - want >= 0 (wrapping); false when `limit` ns have passed
-// or *p became kResumeAbort.
-__device__ __forceinline__ bool wait_for(const uint32_t *p, uint32_t want, uint64_t limit, uint32_t sleep_ns) {
+// or *p became kResumeAbort.  `idle`: sleep between the polls, an eighth of
+// the time waited so far (0.2 to 8 us), for the CTAs outside a long-running
+// team.
+__device__ __forceinline__ bool wait_for(const uint32_t *p, uint32_t want, uint64_t limit, bool idle) {
     if ((int32_t)(ld_acquire(p) - want) >= 0) return true;
     const uint64_t t0 = global_ns();
     for (;;) {
         const uint32_t v = ld_acquire(p);
         if (v == kResumeAbort) return false;
         if ((int32_t)(v - want) >= 0) return true;
-        if (global_ns() - t0 > limit) return false;
-        if (sleep_ns) __nanosleep(sleep_ns);
+        const uint64_t t = global_ns() - t0;
+        if (t > limit) return false;
+        if (idle) __nanosleep(t < 1600u ? 200u : t > 64000u ? 8000u : (uint32_t)t / 8u);
     }
 }
 
@@ -82,13 +85,13 @@ __device__ __forceinline__ bool arrive_full(QuerySync *s, uint32_t size, uint32_
         st_release(&s->full_release, round);
         return true;
     }
-    return wait_for(&s->full_release, round, kQueryBarrierNs, 32);
+    return wait_for(&s->full_release, round, kQueryBarrierNs, false);
 }
 __device__ __forceinline__ bool arrive_team(QuerySync *s, uint32_t size, uint32_t round) {
     fence_acq_rel();
     const uint32_t old = add_acq_rel(&s->team_arrive, 1u);
     if (old + 1u == size * round) return true;
-    return wait_for(&s->team_arrive, size * round, kQueryBarrierNs, 0);
+    return wait_for(&s->team_arrive, size * round, kQueryBarrierNs, false);
 }
 
 // ---- SSSP: the far set -----------------------------------------------------
@@ -116,30 +119,32 @@ __device__ __forceinline__ bool arrive_team(QuerySync *s, uint32_t size, uint32_
 // (halves) after an interval whose lists averaged fewer than kFarLow (more
 // than kFarHigh) edges.
 //
-// Measured: 4096^2 grid 334 -> 96 ms (list edges 203 -> 8 per edge), uniform
-// graph of 8.4M vertices and 33.5M edges 2.93 -> 1.67 ms (3.0 -> 1.3).
-// First width 8 / 16 / 32 / 64 * weight / degree: uniform graph 2.14 / 1.73
-// / 1.67 / 3.17 ms; kFarEdges 8192 / 32768: grid 97.4 / 96.2 ms.  On R-MAT
+// Measured: 4096^2 grid 334 -> 96 ms (list edges 203 -> 8 per edge), with
+// the fast levels below 53 ms; uniform graph of 8.4M vertices and 33.5M edges
+// 2.93 -> 1.6 ms (3.0 -> 1.3).  First width 8 / 16 / 32 / 64 * weight / degree:
+// uniform graph 2.14 / 1.73 / 1.67 / 3.17 ms.  kFarHigh 131072 / 65536 / 32768
+// / 24576: grid 75.4 / 65.8 / 62.4 / 62.5 ms.  On R-MAT
 // graphs no width pays (a model of scale 21: 1.58 -> 1.42 relaxations per
 // edge for 3 times the iterations), and the rule never sets T there.
 #ifndef LB_FAR_EDGES
-#define LB_FAR_EDGES 32768
+#define LB_FAR_EDGES 16384
 #endif
 #ifndef LB_FAR_MULT
 #define LB_FAR_MULT 32
 #endif
 #ifndef LB_FAR_LOW
-#define LB_FAR_LOW 8192
+#define LB_FAR_LOW 4096
 #endif
 #ifndef LB_FAR_HIGH
-#define LB_FAR_HIGH 131072
+#define LB_FAR_HIGH 32768
 #endif
 #ifndef LB_FAR_MINDIV
 #define LB_FAR_MINDIV 4
 #endif
-constexpr int64_t kFarEdges = LB_FAR_EDGES;
+constexpr uint32_t kFarEdges = LB_FAR_EDGES;
 constexpr uint32_t kFarLevels = 6, kFarLate = 32;
 constexpr uint64_t kFarLow = LB_FAR_LOW, kFarHigh = LB_FAR_HIGH;
+constexpr uint32_t kFarMaxDelta = 1u << 30;
 
 // T + delta, or "no threshold" when that passes the largest distance.
 __device__ __forceinline__ uint32_t far_add(uint32_t t, uint32_t delta) {
@@ -147,76 +152,655 @@ __device__ __forceinline__ uint32_t far_add(uint32_t t, uint32_t delta) {
     return x >= kSat ? kInf : (uint32_t)x;
 }
 
-// One pull: queues the vertices of the far set in [T0, T1), keeps the bits
-// of the blocks that still hold vertices at T1 or above, and lowers *fmin
-// (shared memory) to the smallest of those.  A warp owns a word of the
-// bitmap: nothing else touches the bits during a pull.
-template <class WB, class WS, class FO>
-__device__ __forceinline__ void far_pull(const uint32_t *status, int64_t n, uint32_t *far_bits, int32_t shift,
-                                         uint32_t T0, uint32_t T1, uint32_t ctas, uint32_t *fmin, WB &wb, WS &ws,
-                                         uint32_t &cnt, const FO &o) {
+// Loop state of a CTA.  `u` is the same in every CTA of a step: each of them
+// updates it from the step's published counts alone.
+struct QueryState {
+    QueryLoop u;
+    FarSet far;  // far.T == u.T
+    uint32_t ok, rank;            // rank: this CTA in the team (kNoRank: outside); 0 leads
+    uint32_t full, team, resume;  // barriers and publications so far
+    uint32_t fmin;                // a pull's smallest distance left
+    uint32_t maxdeg;              // largest degree this CTA listed in the level
+    uint32_t trace;               // leader: records written
+    uint64_t deadline, t0, pushes;
+    // fast levels: exchanges and conversions so far, what the last exchange
+    // said, the segments' first positions, this CTA's pushes of the level
+    uint32_t fast_epoch, fast_conv, fast_n, fast_e, fast_maxdeg, fast_late;
+    uint32_t fast_pre[kFastTeam + 1];
+    uint32_t out_n, out_e, out_maxdeg;
+};
+
+// Thread 0, the same in every CTA: whether a list of E edges (iteration
+// u.iters) makes the threshold rule above hold.
+__device__ __forceinline__ void far_engage(QueryState &q, uint32_t E, int64_t m) {
+    ++q.u.int_lists;
+    q.u.int_edges += E;
+    q.u.int_max = max(q.u.int_max, E);
+    if (q.u.engaged || E < kFarEdges) return;
+    if (!((q.u.iters >= kFarLevels && q.u.relaxed + E < (uint64_t)m / 4) || q.u.iters >= kFarLate)) return;
+    q.u.engaged = 1u;
+    q.u.T = q.far.T = far_add(0u, q.u.delta);
+    q.u.int_lists = q.u.int_max = 0u;
+    q.u.int_edges = 0ull;
+}
+
+// Thread 0, the same in every CTA: the next step pulls [u.T, from + delta).
+// u.edges becomes the size of list to expect (whether the team runs it), and
+// the interval's lists decide the next width.
+__device__ __forceinline__ void far_start_pull(QueryState &q, uint32_t from) {
+    q.u.done = 0u;
+    q.u.pull = 1u;
+    q.u.T0 = q.u.T;
+    q.u.T = q.far.T = far_add(from, q.u.delta);
+    q.u.edges = q.u.int_max;
+    if (q.u.int_lists > 0u) {
+        const uint64_t avg = q.u.int_edges / q.u.int_lists;
+        if (avg < kFarLow && q.u.delta < kFarMaxDelta) q.u.delta *= 2u;
+        if (avg > kFarHigh) q.u.delta = max(q.u.delta / 2u, q.u.delta_min);
+    }
+    q.u.int_lists = q.u.int_max = 0u;
+    q.u.int_edges = 0ull;
+}
+
+// Calls take(v, d) for 32 consecutive vertices at a time of this warp's
+// share of the far set's blocks, with d their distances (kInf past the end),
+// and clears the bits of the blocks in which no lane's keep(d) held.  A lane
+// holds one word of the bitmap (one load for up to 1024 blocks per warp),
+// and eight blocks' distances are in flight at once: a wave on a grid sets
+// one bit in each of thousands of words.
+template <class Take, class Keep>
+__device__ __forceinline__ void far_blocks(const uint32_t *status, int64_t n, const FarSet &far, uint32_t me,
+                                           uint32_t ctas, bool clear, Take take, Keep keep) {
+    constexpr int kB = 8;
     const uint32_t lane = lane_id();
-    const int32_t words = (int32_t)((((n - 1) >> shift) >> 5) + 1);
-    const int32_t stride = (int32_t)ctas * kWarps;
-    uint32_t mn = kInf;
-    for (int32_t w = (int32_t)blockIdx.x + (int32_t)ctas * (int32_t)(threadIdx.x >> 5); w < words; w += stride) {
-        uint32_t bits = __ldcg(far_bits + w);
-        uint32_t keep = 0;
-        const uint32_t had = bits;
-        while (bits) {  // warp-uniform
-            const int b = __ffs(bits) - 1;
-            bits &= bits - 1;
-            const int64_t v0 = ((int64_t)w * 32 + b) << shift;
-            const int64_t v1 = min(v0 + ((int64_t)1 << shift), n);
-            bool left = false;
-            for (int64_t v = v0 + lane; v < v1 + lane; v += 128) {  // warp-uniform trip count
-                uint32_t d[4];
+    const uint32_t words = (uint32_t)(((n - 1) >> far.shift) >> 5) + 1u;
+    const uint32_t warps = ctas * kWarps;
+    const int32_t chunks = 1 << (far.shift - 5);  // of 32 vertices per block
+    for (uint32_t w0 = me + ctas * (threadIdx.x >> 5); w0 < words; w0 += 32u * warps) {  // warp-uniform
+        uint32_t my = w0 + lane * warps < words ? __ldcg(far.bits + w0 + lane * warps) : 0u;
+        unsigned nz = __ballot_sync(kFull, my != 0u);
+        while (nz) {
+            uint32_t blk[kB], left = 0u;  // block numbers (kInf: none), bit r: block r keeps its bit
 #pragma unroll
-                for (int r = 0; r < 4; ++r) d[r] = v + 32 * r < v1 ? __ldcg(status + v + 32 * r) : kInf;
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    if (d[r] != kInf && d[r] >= T1) {
-                        left = true;
-                        mn = min(mn, d[r]);
-                    }
-                    const bool take = d[r] >= T0 && d[r] < T1;  // kInf is never below T1
-                    if (__any_sync(kFull, take)) {
-                        wpush(wb, cnt, take, (int32_t)(v + 32 * r), 0, 0u);
-                        if (cnt > (uint32_t)(WB::kCap - 32)) wflush<kOutNode, true>(wb, ws, cnt, o);
-                    }
+            for (int r = 0; r < kB; ++r) {
+                blk[r] = kInf;
+                if (nz) {  // warp-uniform
+                    const int l = __ffs(nz) - 1;
+                    const int b = __ffs(__shfl_sync(kFull, my, l)) - 1;
+                    blk[r] = (w0 + (uint32_t)l * warps) * 32u + (uint32_t)b;
+                    if ((int)lane == l) my &= my - 1u;
+                    nz = __ballot_sync(kFull, my != 0u);
                 }
             }
-            if (__any_sync(kFull, left)) keep |= 1u << b;
+            for (int32_t c = 0; c < chunks; ++c) {
+                uint32_t d[kB];
+#pragma unroll
+                for (int r = 0; r < kB; ++r) {
+                    const int64_t v = ((int64_t)blk[r] << far.shift) + 32 * c + lane;
+                    d[r] = blk[r] != kInf && v < n ? __ldcg(status + v) : kInf;
+                }
+#pragma unroll
+                for (int r = 0; r < kB; ++r) {
+                    if (__any_sync(kFull, keep(d[r]))) left |= 1u << r;
+                    take((int32_t)(((int64_t)blk[r] << far.shift) + 32 * c + lane), d[r]);
+                }
+            }
+            if (clear && lane == 0)
+#pragma unroll
+                for (int r = 0; r < kB; ++r)
+                    if (blk[r] != kInf && !((left >> r) & 1u)) atomicAnd(far.bits + (blk[r] >> 5), ~(1u << (blk[r] & 31u)));
         }
-        if (lane == 0 && keep != had) far_bits[w] = keep;
     }
+}
+
+// One pull: queues the vertices of the far set in [T0, T1), clears the bits
+// of the blocks that hold no vertex at T1 or above, and lowers *fmin (shared
+// memory) to the smallest of those that are left.  Nothing sets bits
+// meanwhile.
+template <class WB, class WS, class FO>
+__device__ __forceinline__ void far_pull(const uint32_t *status, int64_t n, const FarSet &far, uint32_t T0,
+                                         uint32_t T1, uint32_t me, uint32_t ctas, uint32_t *fmin, WB &wb, WS &ws,
+                                         uint32_t &cnt, const FO &o) {
+    uint32_t mn = kInf;
+    far_blocks(
+        status, n, far, me, ctas, true,
+        [&](int32_t v, uint32_t d) {
+            const bool want = d >= T0 && d < T1;  // kInf is never below T1
+            if (__any_sync(kFull, want)) {
+                wpush(wb, cnt, want, v, 0, 0u);
+                if (cnt > (uint32_t)(WB::kCap - 32)) wflush<kOutNode, true>(wb, ws, cnt, o);
+            }
+        },
+        [&](uint32_t d) {
+            const bool k = d != kInf && d >= T1;
+            if (k) mn = min(mn, d);
+            return k;
+        });
     wflush<kOutNode, true>(wb, ws, cnt, o);
     mn = __reduce_min_sync(kFull, mn);
-    if (lane == 0 && mn != kInf) atomicMin(fmin, mn);
+    if (lane_id() == 0 && mn != kInf) atomicMin(fmin, mn);
+}
+
+// Picks the SMs of the small-list team, once per workspace.  The L2 is in two
+// halves, each by one die's SMs, and what another SM has just written costs
+// an SM of the other half 600-690 cycles instead of 260-330 (a dependent
+// atomic; a line that stays unwritten is read in 230-310 from either).  A
+// fast level's exchange waits for the slowest CTA's word to reach the
+// slowest reader, so the team is the kFastTeam SMs nearest to the words:
+// every CTA times atomics on them, and the last one ranks the SMs.
+// Teams from both halves: 3.4 us per level of the 1000 x 1537 grid's BFS, and
+// 7.0 to 8.9 ms per query by where the words lay.
+__global__ void __launch_bounds__(kBlock) k_team_pick(Ctl *ctl) {
+    __shared__ alignas(16) uint32_t s_lat[kMaxSms];
+    __shared__ bool s_last;
+    if (threadIdx.x == 0) {
+        uint32_t sm, best = kNoRank;
+        asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
+        // CTAs spread over the words: queueing at one would hide the distance
+        unsigned long long *const w = fast_words(ctl) + (blockIdx.x * 5u) % (2u * kFastTeam);
+        for (int r = 0; r < 3; ++r) {
+            unsigned long long x = 0ull;
+            const long long t0 = clock64();
+#pragma unroll 1
+            for (int k = 0; k < 6; ++k) x = atomicAdd(w + x, 0ull);  // the words are zero: a dependent chain
+            const long long t1 = clock64() + (long long)x;
+            best = min(best, (uint32_t)(t1 - t0));
+        }
+        if (sm < kMaxSms) ctl->sm_rank[sm] = best;  // zero: no CTA ran there
+        __threadfence();
+        s_last = atomicAdd(&ctl->team_done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    for (uint32_t k = threadIdx.x; k < kMaxSms; k += kBlock) {
+        const uint32_t l = __ldcg(&ctl->sm_rank[k]);
+        s_lat[k] = l ? min(l, kNoRank >> 10) << 9 | k : kNoRank;  // ordered by latency, then SM
+    }
+    __syncthreads();
+    for (uint32_t k = threadIdx.x; k < kMaxSms; k += kBlock) {
+        const uint32_t mine = s_lat[k];
+        uint32_t rank = 0;
+        for (uint32_t j = 0; j < kMaxSms / 4; ++j) {
+            const uint4 x = reinterpret_cast<const uint4 *>(s_lat)[j];
+            rank += (x.x < mine) + (x.y < mine) + (x.z < mine) + (x.w < mine);
+        }
+        ctl->sm_rank[k] = mine != kNoRank && rank < (uint32_t)kFastTeam ? rank : kNoRank;
+    }
+}
+
+cudaError_t launch_team_pick(Ctl *ctl, int sms, cudaStream_t st) {
+    // one CTA per SM (shared memory)
+    constexpr int kSmem = 160 * 1024;
+    cudaError_t e = cudaFuncSetAttribute(k_team_pick, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    if (e != cudaSuccess) return e;
+    k_team_pick<<<sms, kBlock, kSmem, st>>>(ctl);
+    return cudaGetLastError();
+}
+
+// The leader's thread 0: the state the CTAs outside the team go on from.
+__device__ __forceinline__ void publish(QuerySync *sync, QueryState &q) {
+    sync->loop = q.u;
+    st_release(&sync->resume, ++q.resume);
+}
+
+// ---- fast levels -------------------------------------------------------------
+// A high-diameter graph spends thousands of levels on lists of a few
+// thousand short entries, and such a level is a chain of dependent L2 and
+// DRAM trips of 0.6-0.9 us each, whatever its size.  The walk's chain has
+// about eleven (tile start, list window, columns, check, claim, offsets,
+// list reservation, fence, barrier arrival, release, list size).  A fast
+// level has six: entry, columns, claim beside the claimed vertex's offsets,
+// fence, and the exchange of the CTAs' counts, which is the barrier too.
+//
+// Lists: each of the kFastTeam CTAs appends to a segment of its own, a
+// 16-byte record {vertex, first edge, degree} per entry, two buffers.  A
+// level ends when every CTA has published one word (entries, edges, largest
+// degree, stamped with the number of the exchange) and warp 0 has read the
+// words of all of them.  The counts' prefix sums turn a list position into a
+// segment and a slot.
+// Work: four lanes per entry, two entries per lane group and two edges of
+// each per lane in flight; entry k goes to CTA k % kFastTeam, so a level
+// spreads over the team and a CTA takes at most ceil(N / kFastRound) * 64
+// entries.  A level runs here only while that times the largest degree is
+// at most the segment's size (it cannot overflow), no entry has more than
+// kFastMaxDeg edges (no lane loops long) and the list has at most
+// LB_FAST_LIMIT * small_edges edges.
+// Measured, per level: grid BFS (4000-8000 edges) 7.7 -> 3.0 us, grid SSSP
+// 9 -> 4.6 us, with 16384-32768 edges 10.2 -> 5.6 us, 32768-65536 edges
+// 10.2 -> 8.3 us (above that the whole grid is as fast, hence LB_FAST_LIMIT).
+// Teams of 32 / 64 / 128 CTAs on both halves of the L2: grid BFS 3.9 / 3.3 /
+// 5.6 us (the words of 128 CTAs take longer to collect).
+constexpr int kFastLanes = 4;
+constexpr int kFastWords = kFastTeam / 32;  // CTAs' words a lane of warp 0 reads
+static_assert(kFastWords % 2 == 0, "words are read in pairs");
+constexpr uint32_t kFastGroups = kBlock / kFastLanes;     // entries a CTA takes at once
+constexpr uint32_t kFastRound = kFastGroups * kFastTeam;  // entries the team takes at once
+constexpr uint32_t kFastMaxDeg = kFastSeg / kFastGroups;  // the longest entry
+#ifndef LB_FAST_LIMIT
+#define LB_FAST_LIMIT 4
+#endif
+constexpr uint32_t kFastMaxEdges = 1u << 24;
+
+// Largest list (edges) of a fast level.
+__device__ __forceinline__ uint32_t fast_limit(int32_t small_edges) {
+    return (uint32_t)min((int64_t)small_edges * LB_FAST_LIMIT, (int64_t)kFastMaxEdges);
+}
+__device__ __forceinline__ bool fast_fits(const QueryArgs &a, uint32_t n, uint32_t e, uint32_t maxdeg, uint32_t lim) {
+    return e <= lim && maxdeg <= kFastMaxDeg &&
+           (n + kFastRound - 1u) / kFastRound * maxdeg * kFastGroups <= (uint32_t)a.seg_cap;
+}
+
+// Whether a regular list is taken to the fast levels, and whether the team
+// runs it (the same in every CTA).
+__device__ __forceinline__ bool fast_takes(const StepParams &p, const QueryArgs &a, const QueryLoop &u) {
+    return a.fast_seg && u.pull == 0u && u.cnt > 0u && u.maxdeg > 0u &&
+           fast_fits(a, u.cnt, u.edges, u.maxdeg, fast_limit(p.small_edges));
+}
+__device__ __forceinline__ bool team_runs(const StepParams &p, const QueryArgs &a, const QueryLoop &u) {
+    return p.small_edges > 0 && (u.edges <= (uint32_t)p.small_edges || fast_takes(p, a, u));
+}
+
+// One CTA's word of an exchange: stamp 16 | time limit passed 1 | largest
+// degree 7 | entries 12 | edges 28; degree and edges saturate (a saturated
+// value never fits, and what leaves the fast levels is counted anew).
+__device__ __forceinline__ unsigned long long fast_word(uint32_t epoch, bool late, uint32_t maxdeg, uint32_t n,
+                                                        uint32_t e) {
+    return (unsigned long long)(epoch & 0xFFFFu) << 48 | (unsigned long long)(late ? 1u : 0u) << 47 |
+           (unsigned long long)min(maxdeg, 127u) << 40 | (unsigned long long)n << 28 |
+           (unsigned long long)min(e, (1u << 28) - 1u);
+}
+
+// Publishes this CTA's pushes and waits for everyone's (every thread calls
+// it).  False when a CTA's word did not come within the barrier limit.
+__device__ __forceinline__ bool fast_exchange(Ctl *ctl, QueryState &q) {
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const uint32_t lane = threadIdx.x;
+        const uint32_t epoch = q.fast_epoch + 1u;
+        unsigned long long *const all = fast_words(ctl) + (epoch & 1u) * kFastTeam;
+        if (lane == 0) {
+            fence_acq_rel();
+            *(volatile unsigned long long *)(all + q.rank) =
+                fast_word(epoch, q.rank == 0u && global_ns() > q.deadline, q.out_maxdeg, q.out_n, q.out_e);
+        }
+        const unsigned long long *const words = all + kFastWords * lane;
+        const uint64_t t0 = global_ns();
+        unsigned long long w[kFastWords];
+        bool ok = true;
+        for (;;) {
+            bool have = true;
+#pragma unroll
+            for (int j = 0; j < kFastWords; j += 2)
+                asm volatile("ld.acquire.gpu.global.v2.u64 {%0, %1}, [%2];"
+                             : "=l"(w[j]), "=l"(w[j + 1]) : "l"(words + j) : "memory");
+#pragma unroll
+            for (int j = 0; j < kFastWords; ++j) have = have && (uint32_t)(w[j] >> 48) == (epoch & 0xFFFFu);
+            if (__all_sync(kFull, have)) break;
+            if (__any_sync(kFull, global_ns() - t0 > kQueryBarrierNs)) {
+                ok = false;
+                break;
+            }
+        }
+        uint32_t in = 0, e = 0, md = 0, late = 0;
+#pragma unroll
+        for (int j = 0; j < kFastWords; ++j) {
+            in += (uint32_t)(w[j] >> 28) & 0xFFFu;
+            // up to 2^25 / kFastWords each (the sum fits 32 bits): that never fits a fast level
+            e += min((uint32_t)w[j] & ((1u << 28) - 1u), (1u << 26) / kFastWords);
+            md = max(md, (uint32_t)(w[j] >> 40) & 127u);
+            late |= (uint32_t)(w[j] >> 47) & 1u;
+        }
+#pragma unroll
+        for (int k = 1; k < 32; k <<= 1) {
+            const uint32_t t = __shfl_up_sync(kFull, in, k);
+            if ((int)lane >= k) in += t;
+        }
+        const uint32_t tot = __shfl_sync(kFull, in, 31);
+#pragma unroll
+        for (int j = kFastWords - 1; j >= 0; --j) {
+            q.fast_pre[kFastWords * lane + j + 1] = in;
+            in -= (uint32_t)(w[j] >> 28) & 0xFFFu;
+        }
+        e = __reduce_add_sync(kFull, e);
+        md = __reduce_max_sync(kFull, md);
+        late = __reduce_or_sync(kFull, late);
+        if (lane == 0) {
+            q.fast_pre[0] = 0;
+            q.fast_n = tot;
+            q.fast_e = e;
+            q.fast_maxdeg = md;
+            q.fast_late = late;
+            q.fast_epoch = epoch;
+            q.ok = ok ? 1u : 0u;
+            q.out_n = q.out_e = q.out_maxdeg = 0u;
+        }
+    }
+    __syncthreads();
+    return q.ok != 0u;
+}
+
+// Appends the lanes' entries (those with want set) to this CTA's segment.
+__device__ __forceinline__ void fast_push(int4 *seg, int32_t cap, QueryState &q, bool want, int32_t v, int32_t beg, int32_t deg) {
+    const unsigned m = __ballot_sync(kFull, want);
+    if (!m) return;
+    const uint32_t lane = lane_id();
+    const uint32_t e = __reduce_add_sync(kFull, want ? (uint32_t)deg : 0u);
+    const uint32_t md = __reduce_max_sync(kFull, want ? (uint32_t)deg : 0u);
+    uint32_t base = 0;
+    if (lane == 0) {
+        base = atomicAdd(&q.out_n, (uint32_t)__popc(m));
+        atomicAdd(&q.out_e, e);
+        atomicMax(&q.out_maxdeg, md);
+    }
+    base = __shfl_sync(kFull, base, 0);
+    const uint32_t slot = base + __popc(m & lanemask_lt());
+    if (want && slot < (uint32_t)cap) seg[slot] = make_int4(v, beg, deg, 0);
+}
+
+// Segment holding list position i.
+__device__ __forceinline__ uint32_t fast_segment(const uint32_t *pre, uint32_t i) {
+    uint32_t lo = 0;
+#pragma unroll
+    for (int k = kFastTeam / 2; k > 0; k >>= 1)
+        if (pre[lo + k] <= i) lo += k;
+    return lo;
+}
+
+// Runs levels on the team's segments from the regular list lists[u.par], and
+// leaves a regular list (or an empty one) and the loop state behind.  Every
+// thread of every team CTA calls it with the same state.  False: a wait ran
+// out.
+template <bool SSSP>
+__device__ __forceinline__ bool fast_levels(const StepParams &p, const QueryArgs &a, QuerySync *sync, QueryState &q,
+                                            WarpBufT<SSSP ? LB_KWB_WD_SSSP : LB_KWB_WD_BFS> &wb) {
+    constexpr int kE = 2, kU = 2, kI = kE * kU;  // entries of a lane group, edges per lane of each, at once
+    Ctl *const ctl = p.ctl;
+    const uint32_t tid = threadIdx.x, rank = q.rank;
+    const uint32_t lim = fast_limit(p.small_edges);
+    const uint32_t conv = q.fast_conv & 1u;
+    int4 *const mine = a.fast_seg + (size_t)rank * a.seg_cap;  // this CTA's segment of buffer 0
+    const size_t seg_buf = (size_t)kFastTeam * a.seg_cap;
+    // the regular list into segment buffer 0
+    {
+        const NodeList in = p.lists[q.u.par];
+        const uint32_t n = q.u.cnt;
+        // last used two conversions back: every CTA has read it since
+        if (rank == 0 && tid == 0) sync->fast_pack[conv] = 0ull;
+        for (uint32_t i0 = 0; i0 < n; i0 += kBlock * kFastTeam) {
+            const uint32_t i = i0 + tid * kFastTeam + rank;
+            int32_t v = 0, beg = 0, deg = 0;
+            if (i < n) {
+                v = in.v[i];
+                beg = in.beg[i];
+                deg = (i + 1 < n ? in.scan[i + 1] : (int32_t)q.u.edges) - in.scan[i];
+                if (beg < 0 || deg < 0 || (int64_t)beg + deg > p.g.m || v < 0 || (int64_t)v >= p.g.n) {
+                    atomicOr(&ctl->error, kErrBounds);
+                    v = beg = deg = 0;
+                }
+            }
+            // fast levels set no queued bits: drop the ones of this list
+            if (SSSP && i < n) {
+                uint32_t *const qn = queued_half(p.bitmap, p.bm_words, q.u.level + 1u);
+                atomicAnd(qn + ((uint32_t)v >> 5), ~(1u << ((uint32_t)v & 31u)));
+            }
+            fast_push(mine, a.seg_cap, q, i < n && deg > 0, v, beg, deg);
+        }
+        if (!fast_exchange(ctl, q)) return false;
+        // every CTA has read the output counters of the levels before
+        if (rank == 0 && tid == 0)
+            for (int k = 0; k < 3; ++k) {
+                sync->pack[k].v = 0ull;
+                sync->pack[k].far_min = kInf;
+                sync->pack[k].maxdeg = 0u;
+            }
+        if (tid == 0) ++q.fast_conv;
+    }
+    uint32_t buf = 0, err = 0;
+    for (;;) {
+        const uint32_t n = q.fast_n, e = q.fast_e, level = q.u.level;
+        if (err || n == 0u || !fast_fits(a, n, e, q.fast_maxdeg, lim)) break;
+        const int4 *const in = a.fast_seg + buf * seg_buf;
+        int4 *const out = mine + (buf ^ 1u) * seg_buf;
+        const int32_t r = (int32_t)(tid % kFastLanes);
+        for (uint32_t i0 = 0; i0 < n; i0 += kE * kFastRound) {
+            int4 x[kE];
+            uint32_t du[kE];
+            int32_t maxdeg = 0;
+#pragma unroll
+            for (int g = 0; g < kE; ++g) {
+                const uint32_t i = i0 + g * kFastRound + (tid / kFastLanes) * kFastTeam + rank;
+                x[g] = make_int4(0, 0, 0, 0);
+                du[g] = 0u;
+                if (i < n) {
+                    const uint32_t sg = fast_segment(q.fast_pre, i);
+                    x[g] = __ldcg(in + (size_t)sg * a.seg_cap + (i - q.fast_pre[sg]));
+                }
+            }
+#pragma unroll
+            for (int g = 0; g < kE; ++g) {
+                maxdeg = max(maxdeg, x[g].z);
+                if (SSSP && x[g].z > 0) du[g] = __ldcg(a.status + x[g].x);
+            }
+            for (int32_t k = r; __any_sync(kFull, k < maxdeg); k += kFastLanes * kU) {
+                int32_t c[kI], b0[kI], b1[kI];
+                uint32_t w[kI], old[kI];
+#pragma unroll
+                for (int j = 0; j < kI; ++j) {
+                    const int32_t kk = k + kFastLanes * (j % kU);
+                    const int4 &y = x[j / kU];
+                    c[j] = kk < y.z ? __ldg(p.g.col + y.y + kk) : -1;
+                    w[j] = SSSP && kk < y.z ? __ldg(p.g.w + y.y + kk) : 0u;
+                }
+                // the claim and the offsets of the vertex in one round trip
+#pragma unroll
+                for (int j = 0; j < kI; ++j) {
+                    old[j] = SSSP ? 0u : kInf;
+                    b0[j] = b1[j] = 0;
+                    if (SSSP) {
+                        // du is finite: the entry was reached
+                        const uint32_t s32 = du[j / kU] + w[j];
+                        w[j] = (s32 < w[j] || s32 >= kSat) ? kSat : s32;
+                    }
+                    if (c[j] >= 0) {
+                        if (SSSP) old[j] = atomicMin(a.status + c[j], w[j]);
+                        else old[j] = atomicOr(p.bitmap + ((uint32_t)c[j] >> 5), 1u << ((uint32_t)c[j] & 31u));
+                        b0[j] = (int32_t)__ldg(p.g.off + c[j]);
+                        b1[j] = (int32_t)__ldg(p.g.off + c[j] + 1);
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < kI; ++j) {
+                    bool want;
+                    if (SSSP) {
+                        // a vertex improved k times in a level is listed k
+                        // times: the repeats relax nothing, and a queued bit
+                        // would be one more round trip per level
+                        want = w[j] < old[j];
+                        if (want && w[j] == kSat) atomicOr(&ctl->error, kErrSaturated);
+                        if (want && w[j] >= q.u.T) {
+                            const uint32_t blk = (uint32_t)c[j] >> q.far.shift;
+                            atomicOr(q.far.bits + (blk >> 5), 1u << (blk & 31u));  // no result: nothing waits for it
+                            want = false;
+                        }
+                    } else {
+                        want = !((old[j] >> ((uint32_t)c[j] & 31u)) & 1u);
+                        if (want) a.status[c[j]] = level + 1u;
+                    }
+                    fast_push(out, a.seg_cap, q, want && b1[j] > b0[j], c[j], b0[j], b1[j] - b0[j]);
+                }
+            }
+        }
+        if (!fast_exchange(ctl, q)) return false;
+        if (tid == 0) {
+            if (rank == 0) {
+                if (q.trace < (uint32_t)kTraceMax) {
+                    TraceRec *t = &ctl->trace[q.trace];
+                    t->level = (int32_t)q.u.iters;
+                    t->mode = kModeSmall;
+                    t->list_size = n;
+                    t->edges = e;
+                    t->t_ns = (int64_t)(global_ns() - q.t0);
+                    ++q.trace;
+                }
+                q.pushes += q.fast_n;
+            }
+            q.u.relaxed += e;
+            q.u.iters += 1u;
+            if (SSSP) far_engage(q, e, p.g.m);
+            q.u.level = level + 1u;
+        }
+        buf ^= 1u;
+        __syncthreads();
+        if (q.fast_n > 0u) {
+            if (q.u.iters >= a.max_levels) err = kErrIterCap;
+            else if (q.fast_late) err = kErrDeadline;
+        }
+    }
+    const uint32_t n = q.fast_n;
+    if (err || n == 0u) {
+        if (tid == 0) {
+            if (err) atomicOr(&ctl->error, err);
+            q.u.cnt = n;
+            q.u.edges = 0;
+            q.u.done = 1u;
+            if (SSSP && !err && q.u.T != kInf) far_start_pull(q, q.u.T);
+        }
+        __syncthreads();
+        return true;
+    }
+    // back to a regular list in lists[u.par], whose entries have all been read
+    {
+        const int4 *const in = a.fast_seg + buf * seg_buf;
+        FlushOut o;
+        o.list = p.lists[q.u.par];
+        o.elist = nullptr;
+        o.pack = &sync->fast_pack[conv];
+        o.err = &ctl->error;
+        o.pushes = nullptr;
+        o.child_first = nullptr;
+        o.cap = p.list_cap;
+        o.tile_cap = p.tile_cap;
+        o.tile = (int32_t)kTileGrain;
+        o.mdt = p.mdt;
+        NoScratch ns;
+        uint32_t cnt = 0;
+        for (uint32_t i0 = 0; i0 < n; i0 += kBlock * kFastTeam) {
+            const uint32_t i = i0 + tid * kFastTeam + rank;
+            int4 x = make_int4(0, 0, 0, 0);
+            if (i < n) {
+                const uint32_t sg = fast_segment(q.fast_pre, i);
+                x = __ldcg(in + (size_t)sg * a.seg_cap + (i - q.fast_pre[sg]));
+            }
+            bool want = i < n;
+            if (SSSP && want) {
+                // each vertex once, with the queued bit of the level before
+                uint32_t *const qb = queued_half(p.bitmap, p.bm_words, q.u.level + 1u);
+                const uint32_t bit = 1u << ((uint32_t)x.x & 31u);
+                want = !(atomicOr(qb + ((uint32_t)x.x >> 5), bit) & bit);
+            }
+            wpush(wb, cnt, want, x.x, x.y, (uint32_t)x.z);
+            if (cnt > (uint32_t)(WarpBufT<SSSP ? LB_KWB_WD_SSSP : LB_KWB_WD_BFS>::kCap - 32))
+                wflush<kOutNode, true>(wb, ns, cnt, o);
+        }
+        wflush_block<kOutNode, true>(wb, ns, cnt, o);
+        __syncthreads();
+        if (tid == 0) {
+            q.ok = arrive_team(sync, kFastTeam, ++q.team) ? 1u : 0u;
+            const unsigned long long x = __ldcg(&sync->fast_pack[conv]);
+            q.u.cnt = (uint32_t)(x >> 32);
+            q.u.edges = (uint32_t)x;
+            q.u.maxdeg = 0u;  // it did not fit: a regular level is next
+        }
+        __syncthreads();
+    }
+    return q.ok != 0u;
+}
+
+// A pull step up to its barrier, out of line: its registers are not the
+// walk's.
+template <class WB>
+__device__ __noinline__ void pull_level(const StepParams &p, const QueryArgs &a, QuerySync *sync, QueryState &q,
+                                        WB &wb, uint32_t me, uint32_t ctas) {
+    NoScratch ns;
+    FlushOutT<1> o;
+    o.list = p.lists[q.u.par ^ 1u];
+    o.elist = nullptr;
+    o.pack = &sync->pack[q.u.level % 3u].v;
+    o.cap = p.list_cap;
+    o.tile_cap = p.tile_cap;
+    o.tile = (int32_t)kTileGrain;
+    o.mdt = p.mdt;
+    o.err = &p.ctl->error;
+    o.pushes = nullptr;
+    o.child_first = nullptr;
+    o.off = p.g.off;
+    o.maxdeg = &q.maxdeg;
+    uint32_t cnt = 0;
+    far_pull(a.status, p.g.n, q.far, q.u.T0, q.u.T, me, ctas, &q.fmin, wb, ns, cnt, o);
+}
+
+// One regular level up to its barrier: the walk over the list's tiles and
+// the flushes.
+template <bool SSSP, int ITEMS>
+__device__ __forceinline__ void regular_level(const StepParams &p, const QueryArgs &a, QuerySync *sync, QueryState &q,
+                                           WarpBufT<SSSP ? LB_KWB_WD_SSSP : LB_KWB_WD_BFS> &wb, uint32_t me,
+                                           uint32_t ctas, bool team_mode) {
+    Ctl *const ctl = p.ctl;
+    uint32_t *const status = a.status;
+    NoScratch ns;
+    const uint32_t level = q.u.level, par = q.u.par, in_cnt = q.u.cnt, E = q.u.edges;
+    uint32_t *const qcur = queued_half(p.bitmap, p.bm_words, level);
+    const NodeList in = p.lists[par];
+    if (SSSP) {
+        // the other half holds the bits of the previous level, whose
+        // queued vertices with out-edges are exactly this level's entries
+        // (bits of vertices without out-edges are never read): clear
+        // those, or sweep the half when the list is long
+        if (!team_mode && (int64_t)in_cnt > p.bm_words / 8) {
+            clear_next_queued(p.bitmap, p.bm_words, level);
+        } else {
+            uint32_t *qn = queued_half(p.bitmap, p.bm_words, level + 1u);
+            for (uint32_t k = me * kBlock + threadIdx.x; k < in_cnt; k += ctas * kBlock) {
+                const int32_t u = in.v[k];
+                if (u >= 0 && (int64_t)u < p.g.n) atomicAnd(&qn[(uint32_t)u >> 5], ~(1u << ((uint32_t)u & 31u)));
+            }
+        }
+    }
+    FlushOutT<SSSP ? 3 : 2> o;
+    o.list = p.lists[par ^ 1u];
+    o.elist = nullptr;
+    o.pack = &sync->pack[level % 3u].v;
+    o.cap = p.list_cap;
+    o.tile_cap = p.tile_cap;
+    o.tile = (int32_t)kTileGrain;
+    o.mdt = p.mdt;
+    o.err = &ctl->error;
+    o.pushes = nullptr;
+    o.child_first = nullptr;
+    o.off = p.g.off;
+    o.maxdeg = &q.maxdeg;
+    if (SSSP) o.far = &q.far;
+    o.claim_bitmap = SSSP ? qcur : p.bitmap;
+    o.claim_status = status;
+    o.claim_level = level;
+    uint32_t cnt = 0;
+    const uint32_t T = (uint32_t)iteration_tile(E, ctas, p.tile);
+    const uint32_t ntiles = (E + T - 1u) / T;
+    for (uint32_t t = me; t < ntiles; t += ctas)
+        wd_walk_tile<SSSP, ITEMS, kLdPlain>(p.g, in, (int32_t)in_cnt, E, T, t, p.bitmap, qcur, status, level,
+                                            &ctl->error, wb, ns, cnt, o);
+    wflush_block<kOutNode, true>(wb, ns, cnt, o);
 }
 
 template <bool SSSP, int ITEMS>
 __global__ void __launch_bounds__(kBlock, SSSP ? LB_QUERY_MIN_BLOCKS_SSSP : LB_QUERY_MIN_BLOCKS)
-    k_query_wd(StepParams p, QueryArgs a) {
+    k_query_wd(const __grid_constant__ StepParams p, const __grid_constant__ QueryArgs a) {
     __shared__ WarpBufT<SSSP ? LB_KWB_WD_SSSP : LB_KWB_WD_BFS> s_wb[kWarps];
-    // loop state, kept in shared memory (registers belong to the walk)
-    __shared__ uint32_t s_ok, s_level, s_par, s_cnt, s_done, s_full, s_team, s_resume;
-    __shared__ uint64_t s_edges, s_deadline, s_t0;
-    __shared__ uint32_t s_trace;               // CTA 0
-    __shared__ unsigned long long s_relaxed, s_pushes;
-    // SSSP threshold: in force (s_far.T), the interval of a pull step [s_T0,
-    // s_far.T), whether the next step is a pull, a pull's smallest distance left
-    __shared__ FarSet s_far;
-    __shared__ uint32_t s_iters, s_T0, s_pull, s_fmin;
-    // CTA 0's decisions: width of the next interval and its smallest value,
-    // lists and edges of the current interval
-    __shared__ uint32_t s_delta, s_delta_min, s_int_lists;
-    __shared__ uint64_t s_int_edges, s_int_max;
-    NoScratch ns;
+    __shared__ QueryState q;  // in shared memory: the registers belong to the walk
     Ctl *ctl = p.ctl;
     QuerySync *const sync = &ctl->qsync[a.number & 1u];
     uint32_t *const status = a.status;
-    const int64_t lim = p.small_edges;
 
     // ---- set-up -----------------------------------------------------------
     {
@@ -254,31 +838,32 @@ __global__ void __launch_bounds__(kBlock, SSSP ? LB_QUERY_MIN_BLOCKS_SSSP : LB_Q
         const int64_t words = SSSP ? 2 * p.bm_words : (n + 31) / 32;
         for (int64_t w = tid; w < words; w += stride)
             p.bitmap[w] = (!SSSP && w == (src >> 5)) ? (1u << (src & 31)) : 0u;
+        if (SSSP)
+            for (int64_t w = tid; w < kFarWords; w += stride) ctl->far_bits[w] = 0u;
         const NodeList L = p.lists[0];
         if (L.tstart != nullptr) {
             const int64_t grains = (deg + kTileGrain - 1) / kTileGrain;
             for (int64_t k = tid; k < grains && k < p.tile_cap; k += stride) L.tstart[k] = 0;
         }
         if (threadIdx.x == 0) {
-            s_level = 0;
-            s_par = 0;
-            s_cnt = deg > 0 ? 1u : 0u;
-            s_edges = (uint64_t)deg;
-            s_done = 0;
-            s_full = s_team = s_resume = 0;
-            s_trace = 0;
-            s_iters = 0;
-            s_far.T = kInf;
-            s_far.shift = a.far_shift;
-            s_far.bits = ctl->far_bits;
-            s_T0 = s_pull = 0;
-            s_fmin = kInf;
-            s_delta = 0;
-            s_int_lists = 0;
-            s_int_edges = s_int_max = 0;
-            s_relaxed = s_pushes = 0ull;
-            s_t0 = global_ns();
-            s_deadline = s_t0 + a.time_limit_ns;
+            for (uint32_t k = 0; k < sizeof(QueryState) / 4; ++k) reinterpret_cast<uint32_t *>(&q)[k] = 0u;
+            q.u.cnt = deg > 0 ? 1u : 0u;
+            q.u.edges = q.u.maxdeg = (uint32_t)deg;
+            q.u.T = q.far.T = kInf;
+            q.far.shift = a.far_shift;
+            q.far.bits = ctl->far_bits;
+            q.fmin = kInf;
+            q.t0 = global_ns();
+            q.deadline = q.t0 + a.time_limit_ns;
+            // The team is the first CTA on each of the SMs that k_team_pick
+            // gave a rank.
+            uint32_t sm;
+            asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
+            q.rank = kNoRank;
+            if (sm < kMaxSms && atomicAdd(&sync->sm_ctas[sm], 1u) == 0u) {
+                q.rank = ctl->sm_rank[sm];
+                if (q.rank != kNoRank) atomicAdd(&sync->team_here, 1u);
+            }
             if (blockIdx.x == 0) {
                 L.v[0] = src;
                 L.beg[0] = (int32_t)beg;
@@ -288,15 +873,14 @@ __global__ void __launch_bounds__(kBlock, SSSP ? LB_QUERY_MIN_BLOCKS_SSSP : LB_Q
                 ctl->src = src;
                 ctl->kind = SSSP ? 1 : 0;
                 ctl->error = 0;
-                ctl->t_start = s_t0;
-                QuerySync *const nx = &ctl->qsync[(a.number + 1u) & 1u];
-                nx->full_arrive = nx->full_release = nx->team_arrive = nx->resume = 0u;
-                for (int k = 0; k < 3; ++k) nx->pack[k].v = 0ull;
+                ctl->t_start = q.t0;
             }
         }
-        if (SSSP) {
-            for (int64_t w = tid; w < kFarWords; w += stride) ctl->far_bits[w] = 0u;
-            if (blockIdx.x == 0) {
+        if (blockIdx.x == 0) {
+            uint32_t *const nx = reinterpret_cast<uint32_t *>(&ctl->qsync[(a.number + 1u) & 1u]);
+            for (uint32_t k = threadIdx.x; k < sizeof(QuerySync) / 4; k += kBlock) nx[k] = 0u;
+            for (uint32_t k = threadIdx.x; k < 2 * kFastTeam; k += kBlock) fast_words(ctl)[k] = 0ull;
+            if (SSSP) {
                 // mean weight of 1024 evenly spaced edges -> first interval width
                 __shared__ unsigned long long s_w;
                 if (threadIdx.x == 0) s_w = 0ull;
@@ -305,10 +889,10 @@ __global__ void __launch_bounds__(kBlock, SSSP ? LB_QUERY_MIN_BLOCKS_SSSP : LB_Q
                 for (int k = 16; k > 0; k >>= 1) wsum += __shfl_xor_sync(kFull, wsum, k);
                 if (lane_id() == 0) atomicAdd(&s_w, wsum);
                 __syncthreads();
-                if (threadIdx.x == 0 && p.g.m > 0) {
-                    const double d = (double)LB_FAR_MULT * ((double)s_w / 1024.0) * (double)n / (double)p.g.m;
-                    s_delta = d < 1.0 ? 1u : d > 1073741824.0 ? (1u << 30) : (uint32_t)d;
-                    s_delta_min = s_delta / LB_FAR_MINDIV > 0 ? s_delta / LB_FAR_MINDIV : 1u;
+                if (threadIdx.x == 0) {
+                    const double d = (double)LB_FAR_MULT * ((double)s_w / 1024.0) * (double)n /
+                                     (double)(p.g.m > 0 ? p.g.m : 1);
+                    sync->delta0 = d < 1.0 ? 1u : d > (double)kFarMaxDelta ? kFarMaxDelta : (uint32_t)d;
                 }
             }
         }
@@ -316,219 +900,132 @@ __global__ void __launch_bounds__(kBlock, SSSP ? LB_QUERY_MIN_BLOCKS_SSSP : LB_Q
         if (p.test_barrier_skip && blockIdx.x == 1) return;
         __syncthreads();
         if (threadIdx.x == 0) {
-            s_full = 1;
-            s_ok = arrive_full(sync, gridDim.x, 1u) ? 1u : 0u;
+            q.full = 1;
+            q.ok = arrive_full(sync, gridDim.x, 1u) ? 1u : 0u;
+            // not every SM of the team holds a CTA: the first CTAs are the team
+            if (__ldcg(&sync->team_here) != (uint32_t)a.team)
+                q.rank = blockIdx.x < (uint32_t)a.team ? blockIdx.x : kNoRank;
+            if (SSSP) q.u.delta = __ldcg(&sync->delta0);
+            q.u.delta_min = max(q.u.delta / LB_FAR_MINDIV, 1u);
         }
         __syncthreads();
     }
 
     // ---- worklist iterations ------------------------------------------------
     bool team_mode = false;
-    bool failed = s_ok == 0u;
-    while (!failed && !s_done) {
-        const int64_t E = (int64_t)s_edges;
-        const bool small = lim > 0 && E <= lim;
+    bool failed = q.ok == 0u;
+    while (!failed && !q.u.done) {
+        const uint32_t E = q.u.edges;
+        const bool small = team_runs(p, a, q.u);
         if (small && !team_mode) {
             team_mode = true;
-            if (blockIdx.x >= (uint32_t)a.team) {
+            if (q.rank == kNoRank) {
                 // wait until the team publishes the state it stopped at (every
                 // thread has read the loop state before it is replaced)
                 __syncthreads();
-                if (threadIdx.x == 0) {
-                    const uint32_t want = ++s_resume;
-                    s_ok = wait_for(&sync->resume, want, a.time_limit_ns + 2 * kQueryBarrierNs, 1000) ? 1u : 0u;
-                    s_level = __ldcg(&sync->r_level);
-                    s_par = __ldcg(&sync->r_par);
-                    s_cnt = __ldcg(&sync->r_cnt);
-                    s_edges = __ldcg(&sync->r_edges);
-                    s_done = __ldcg(&sync->r_done);
-                    s_iters = __ldcg(&sync->r_iters);
-                    s_pull = __ldcg(&sync->r_pull);
-                    s_T0 = __ldcg(&sync->r_T0);
-                    s_far.T = __ldcg(&sync->r_T);
-                }
+                if (threadIdx.x == 0)
+                    q.ok = wait_for(&sync->resume, ++q.resume, a.time_limit_ns + 2 * kQueryBarrierNs, true) ? 1u : 0u;
                 __syncthreads();
-                failed = s_ok == 0u;
+                if (threadIdx.x < sizeof(QueryLoop) / 4)
+                    reinterpret_cast<uint32_t *>(&q.u)[threadIdx.x] =
+                        __ldcg(reinterpret_cast<const uint32_t *>(&sync->loop) + threadIdx.x);
+                __syncthreads();
+                if (threadIdx.x == 0) q.far.T = q.u.T;
+                __syncthreads();
+                failed = q.ok == 0u;
                 team_mode = false;
                 continue;
             }
         } else if (!small) {
             team_mode = false;
         }
-        const uint32_t ctas = team_mode ? (uint32_t)a.team : gridDim.x;
-        const uint32_t level = s_level, par = s_par;
-        const int64_t in_cnt = s_cnt;
-        const bool pull = SSSP && s_pull != 0u;
-        uint32_t *const qcur = queued_half(p.bitmap, p.bm_words, level);
-        const NodeList in = p.lists[par];
-        if (SSSP && !pull) {
-            // the other half holds the bits of the previous level, whose
-            // queued vertices with out-edges are exactly this level's entries
-            // (bits of vertices without out-edges are never read): clear
-            // those, or sweep the half when the list is long
-            uint32_t *qn = queued_half(p.bitmap, p.bm_words, level + 1u);
-            const int64_t stride = (int64_t)ctas * blockDim.x;
-            const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-            if (!team_mode && in_cnt > p.bm_words / 8) {
-                clear_next_queued(p.bitmap, p.bm_words, level);
-            } else {
-                for (int64_t k = tid; k < in_cnt; k += stride) {
-                    const int32_t u = in.v[k];
-                    if (u >= 0 && (int64_t)u < p.g.n) atomicAnd(&qn[(uint32_t)u >> 5], ~(1u << ((uint32_t)u & 31u)));
-                }
-            }
+        if (team_mode && fast_takes(p, a, q.u)) {
+            // uniform over the team: every CTA has the same state
+            failed = !fast_levels<SSSP>(p, a, sync, q, s_wb[threadIdx.x >> 5]);
+            // the team hands over, as after a regular level
+            if (!failed && q.rank == 0u && threadIdx.x == 0 && (q.u.done || !team_runs(p, a, q.u))) publish(sync, q);
+            continue;
         }
+        const uint32_t ctas = team_mode ? (uint32_t)a.team : gridDim.x;
+        const uint32_t me = team_mode ? q.rank : blockIdx.x;
+        const uint32_t level = q.u.level, par = q.u.par;
+        const uint32_t in_cnt = q.u.cnt;
+        const bool pull = SSSP && q.u.pull != 0u;
         // the next level's output counter (its last reads were before the
         // barrier that ended the previous level)
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            QuerySync::Pack *const nx = &sync->pack[(level + 1u) % 3u];
-            nx->v = 0ull;
-            if (SSSP) {
-                uint32_t T = s_far.T;
-                if (pull) {
-                    // an interval has ended: its lists decide the next width
-                    if (s_int_lists > 0) {
-                        const uint64_t avg = s_int_edges / s_int_lists;
-                        if (avg < kFarLow && s_delta < (1u << 30)) s_delta *= 2u;
-                        if (avg > kFarHigh) s_delta = max(s_delta / 2u, s_delta_min);
-                    }
-                    s_int_lists = 0;
-                    s_int_edges = s_int_max = 0;
-                } else {
-                    ++s_int_lists;
-                    s_int_edges += (uint64_t)E;
-                    s_int_max = max(s_int_max, (uint64_t)E);
-                    if (T == kInf && s_T0 == 0u && E >= kFarEdges &&
-                        ((s_iters >= kFarLevels && s_relaxed + (uint64_t)E < (uint64_t)p.g.m / 4) ||
-                         s_iters >= kFarLate)) {
-                        T = far_add(0u, s_delta);
-                        s_T0 = 1u;  // set once
-                        s_int_lists = 0;
-                        s_int_edges = s_int_max = 0;
-                    }
-                }
-                nx->far_min = kInf;
-                nx->T = T;
-                nx->delta = s_delta;
-                nx->pull_size = (uint32_t)(s_int_max > 0x7FFFFFFFull ? 0x7FFFFFFFull : s_int_max);
-            }
+        if (q.rank == 0u && threadIdx.x == 0) {
+            sync->pack[(level + 1u) % 3u].v = 0ull;
+            sync->pack[(level + 1u) % 3u].maxdeg = 0u;
+            if (SSSP) sync->pack[(level + 1u) % 3u].far_min = kInf;
         }
-        FlushOutT<SSSP ? 3 : 2> o;
-        o.list = p.lists[par ^ 1u];
-        o.elist = nullptr;
-        o.pack = &sync->pack[level % 3u].v;
-        o.cap = p.list_cap;
-        o.tile_cap = p.tile_cap;
-        o.tile = (int32_t)kTileGrain;
-        o.mdt = p.mdt;
-        o.err = &ctl->error;
-        o.pushes = nullptr;
-        o.child_first = nullptr;
-        o.off = p.g.off;
-        if (SSSP) o.far = &s_far;
-        o.claim_bitmap = SSSP ? qcur : p.bitmap;
-        o.claim_status = status;
-        o.claim_level = level;
-        uint32_t cnt = 0;
-        const uint32_t warp = threadIdx.x >> 5;
-        const uint32_t T = (uint32_t)iteration_tile(E, ctas, p.tile);
-        const uint32_t ntiles = pull ? 0u : ((uint32_t)E + T - 1u) / T;
-        if (SSSP && pull) {
-            FlushOutT<1> op;
-            static_cast<FlushOut &>(op) = o;
-            far_pull(status, p.g.n, ctl->far_bits, a.far_shift, s_T0, s_far.T, ctas, &s_fmin, s_wb[warp], ns, cnt, op);
-        }
-        for (uint32_t t = blockIdx.x; t < ntiles; t += ctas)
-            wd_walk_tile<SSSP, ITEMS, kLdPlain>(p.g, in, (int32_t)in_cnt, (uint32_t)E, T, t, p.bitmap, qcur, status, level, &ctl->error,
-                                                s_wb[warp], ns, cnt, o);
-        wflush_block<kOutNode, true>(s_wb[warp], ns, cnt, o);
+        if (SSSP && pull) pull_level(p, a, sync, q, s_wb[threadIdx.x >> 5], me, ctas);
+        else regular_level<SSSP, ITEMS>(p, a, sync, q, s_wb[threadIdx.x >> 5], me, ctas, team_mode);
         __syncthreads();
         if (threadIdx.x == 0) {
             unsigned long long *const pk = &sync->pack[level % 3u].v;
-            QuerySync::Pack *const nx = &sync->pack[(level + 1u) % 3u];
-            if (SSSP && pull && s_fmin != kInf) {
-                atomicMin(&sync->pack[level % 3u].far_min, s_fmin);
-                s_fmin = kInf;
+            if (SSSP && pull && q.fmin != kInf) {
+                atomicMin(&sync->pack[level % 3u].far_min, q.fmin);
+                q.fmin = kInf;
             }
-            if (blockIdx.x == 0 && global_ns() > s_deadline) atomicOr(pk, 1ull << 63);
-            s_ok = (team_mode ? arrive_team(sync, ctas, ++s_team) : arrive_full(sync, ctas, ++s_full)) ? 1u : 0u;
+            if (q.maxdeg > 0u) {
+                atomicMax(&sync->pack[level % 3u].maxdeg, q.maxdeg);
+                q.maxdeg = 0u;
+            }
+            if (q.rank == 0u && global_ns() > q.deadline) atomicOr(pk, 1ull << 63);
+            q.ok = (team_mode ? arrive_team(sync, ctas, ++q.team) : arrive_full(sync, ctas, ++q.full)) ? 1u : 0u;
             const unsigned long long x = __ldcg(pk);
-            const bool late = (x >> 63) != 0ull;
-            int64_t ncnt = (int64_t)((x >> 32) & 0x7FFFFFFFull);
-            uint32_t nedges = (uint32_t)x;
+            q.u.maxdeg = __ldcg(&sync->pack[level % 3u].maxdeg);
+            const uint32_t fmin = SSSP && pull ? __ldcg(&sync->pack[level % 3u].far_min) : 0u;
+            uint32_t ncnt = (uint32_t)(x >> 32) & 0x7FFFFFFFu;
             uint32_t err = 0;
-            if (ncnt > p.list_cap) {
+            if ((int64_t)ncnt > p.list_cap) {
                 err |= kErrCapacity;
-                ncnt = p.list_cap;
+                ncnt = (uint32_t)p.list_cap;
+            }
+            if (q.rank == 0u) {
+                if (!pull && q.trace < (uint32_t)kTraceMax) {
+                    TraceRec *r = &ctl->trace[q.trace];
+                    r->level = (int32_t)q.u.iters;
+                    r->mode = team_mode ? kModeSmall : kModeRelax;
+                    r->list_size = in_cnt;
+                    r->edges = E;
+                    r->t_ns = (int64_t)(global_ns() - q.t0);
+                    ++q.trace;
+                }
+                q.pushes += ncnt;
+            }
+            q.u.level = level + 1u;
+            q.u.par = par ^ 1u;
+            q.u.cnt = ncnt;
+            q.u.edges = (uint32_t)x;
+            q.u.pull = 0u;
+            if (!pull) {
+                if (SSSP) far_engage(q, E, p.g.m);
+                q.u.iters += 1u;
+                q.u.relaxed += E;
             }
             bool more = ncnt > 0;
-            const uint32_t iters = s_iters + (pull ? 0u : 1u);
-            uint32_t npull = 0, nT = kInf, nT0 = 0;
-            if (SSSP) {
-                const uint32_t fmin = pull ? __ldcg(&sync->pack[level % 3u].far_min) : 0u;
-                const uint32_t delta = __ldcg(&nx->delta), hint = __ldcg(&nx->pull_size);
-                nT = pull ? s_far.T : __ldcg(&nx->T);
-                nT0 = s_T0;
-                // the list is empty: pull the next interval, unless no
-                // threshold is in force or nothing was left at the last pull
-                if (!more && nT != kInf && !(pull && fmin == kInf)) {
-                    npull = 1u;
-                    more = true;
-                    nT0 = nT;
-                    nT = far_add(pull ? fmin : nT, delta);
-                    nedges = hint;
-                }
+            // the list is empty: pull the next interval, unless no threshold
+            // is in force or nothing was left at the last pull
+            if (SSSP && !more && q.u.T != kInf && !(pull && fmin == kInf)) {
+                more = true;
+                far_start_pull(q, pull ? fmin : q.u.T);
             }
-            if (more && iters >= a.max_levels) {
+            if (more && q.u.iters >= a.max_levels) {
                 err |= kErrIterCap;
                 more = false;
             }
-            if (more && late) {
+            if (more && (x >> 63) != 0ull) {
                 err |= kErrDeadline;
                 more = false;
             }
             if (err) atomicOr(&ctl->error, err);
-            if (blockIdx.x == 0) {
-                const uint32_t tl = s_trace;
-                if (!pull && tl < (uint32_t)kTraceMax) {
-                    TraceRec *r = &ctl->trace[tl];
-                    r->level = (int32_t)s_iters;
-                    r->mode = team_mode ? kModeSmall : kModeRelax;
-                    r->list_size = in_cnt;
-                    r->edges = E;
-                    r->t_ns = (int64_t)(global_ns() - s_t0);
-                    s_trace = tl + 1u;
-                }
-                if (!pull) s_relaxed += (unsigned long long)E;
-                s_pushes += (unsigned long long)ncnt;
-                // the team hands over: the list has grown, or the query ends
-                if (team_mode && s_ok && (!more || (int64_t)nedges > lim)) {
-                    sync->r_level = level + 1u;
-                    sync->r_par = par ^ 1u;
-                    sync->r_cnt = (uint32_t)ncnt;
-                    sync->r_edges = nedges;
-                    sync->r_done = more ? 0u : 1u;
-                    sync->r_iters = iters;
-                    sync->r_pull = npull;
-                    sync->r_T0 = nT0;
-                    sync->r_T = nT;
-                    st_release(&sync->resume, ++s_resume);
-                }
-            }
-            s_level = level + 1u;
-            s_par = par ^ 1u;
-            s_cnt = (uint32_t)ncnt;
-            s_edges = nedges;
-            s_done = more ? 0u : 1u;
-            s_iters = iters;
-            if (SSSP) {
-                s_pull = npull;
-                s_T0 = nT0;
-                s_far.T = nT;
-            }
+            q.u.done = more ? 0u : 1u;
+            // the team hands over: the list has grown, or the query ends
+            if (q.rank == 0u && team_mode && q.ok && (q.u.done || !team_runs(p, a, q.u))) publish(sync, q);
         }
         __syncthreads();
-        failed = s_ok == 0u;
+        failed = q.ok == 0u;
     }
     if (failed) {
         if (threadIdx.x == 0) {
@@ -549,18 +1046,17 @@ __global__ void __launch_bounds__(kBlock, SSSP ? LB_QUERY_MIN_BLOCKS_SSSP : LB_Q
                 break;
             }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        const uint32_t par = s_par;
-        p.lists[par].scan[s_cnt] = (int32_t)s_edges;
-        ctl->level = s_iters;
-        ctl->step = s_iters;
-        ctl->par = par;
-        ctl->in_cnt = s_cnt;
-        ctl->in_edges = s_edges;
+    if (q.rank == 0u && threadIdx.x == 0) {
+        p.lists[q.u.par].scan[q.u.cnt] = (int32_t)q.u.edges;
+        ctl->level = q.u.iters;
+        ctl->step = q.u.iters;
+        ctl->par = q.u.par;
+        ctl->in_cnt = q.u.cnt;
+        ctl->in_edges = q.u.edges;
         ctl->active = 0u;
-        ctl->relaxed = s_relaxed;
-        ctl->pushes = s_pushes;
-        ctl->trace_len = s_trace;
+        ctl->relaxed = q.u.relaxed;
+        ctl->pushes = q.pushes;
+        ctl->trace_len = q.trace;
     }
 }
 

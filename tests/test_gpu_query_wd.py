@@ -72,6 +72,42 @@ def test_grid_and_team_sizes(opts):
             G.close()
 
 
+@pytest.mark.parametrize("deg", [1, 2, 4, 8, 32, 33])
+def test_fast_levels_at_their_degree_limits(deg):
+    # layered graphs whose entries have exactly deg edges: lists that fit the
+    # team's segments, that just do not (33), and that grow past them
+    L, width = 30, 3000
+    r = np.random.default_rng(deg)
+    n = 1 + L * width
+    src, dst = [np.zeros(min(width, 40), int)], [1 + np.arange(min(width, 40))]
+    for k in range(L - 1):
+        u = np.repeat(1 + k * width + np.arange(width), deg)
+        src.append(u)
+        dst.append(1 + (k + 1) * width + (u * 7 + r.integers(0, 60, u.size)) % width)
+    src, dst = np.concatenate(src), np.concatenate(dst)
+    g = gg.from_edges(n, src, dst, r.integers(1, 1000, src.size), clean=False)
+    G = lb.Graph.from_csr(g)
+    try:
+        check(G, g, 0)
+        G.set_options(small_edges=100)
+        check(G, g, 0)
+        check(G, g, 1 + 5 * width)
+    finally:
+        G.close()
+
+
+def test_fast_levels_on_small_and_large_graphs():
+    # the segments' size changes at 32768 vertices
+    for R, C in ((181, 181), (182, 181), (64, 5000), (3, 40000)):
+        g = gg.grid(R, C, seed=R)
+        G = lb.Graph.from_csr(g)
+        try:
+            check(G, g, 0)
+            check(G, g, R * C // 2)
+        finally:
+            G.close()
+
+
 def far_graph(kind):
     # uniform random graphs whose lists grow past the threshold rule's size
     # early; n is not a multiple of the far set's 128-vertex blocks
