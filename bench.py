@@ -171,17 +171,17 @@ def measured_peak():
         return 6800.0, "fallback"
 
 
-def kernel_launches(trace, whole_query: bool = False):
+def kernel_launches(trace, kind: str, whole_query: bool = False):
     """Kernels one query launches: one when the whole query is a single
-    cooperative launch (WD's device loop); else set-up (prepare, init), one
+    cooperative launch (WD's device loop); else set-up, one
     per step of the trace except the levels that ran inside one persistent
     small-list launch (trace mode 4; one launch per run of such levels), and
-    the overflow check."""
+    the overflow check (SSSP)."""
     if whole_query:
         return 1
     modes = [int(m) for m in trace["mode"]]
     small_runs = sum(1 for i, m in enumerate(modes) if m == 4 and (i == 0 or modes[i - 1] != 4))
-    return 2 + sum(1 for m in modes if m != 4) + small_runs + 1
+    return 1 + sum(1 for m in modes if m != 4) + small_runs + (kind == "sssp")
 
 
 def m_reached_torch(out, deg_t):
@@ -562,7 +562,7 @@ def main():
             if st["status"] != 0:
                 raise SystemExit(f"query failed: {kind} src={s} status={st['status']}")
             work[(kind, int(s))] = m_reached_torch(out, deg_t) + (
-                kernel_launches(G.trace(), args.loop_mode == 0 and args.strategy.upper() in ("WD", "AUTO")),
+                kernel_launches(G.trace(), kind, args.loop_mode == 0 and args.strategy.upper() in ("WD", "AUTO")),
                 st["iterations"], st["edges_relaxed"])
 
     ev = {k: [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in srcs]

@@ -593,8 +593,7 @@ lb_status run_query(lb_graph *g, int kind, int s, int32_t src, void *out_dev, in
         g->last_strategy = s;
         return LB_OK;
     }
-    LB_CU(launch_prepare(p, src, (uint32_t *)out_dev, kind, max_levels, max_steps, time_limit_ns, st));
-    LB_CU(launch_init(p, grid, st));
+    LB_CU(launch_init(p, src, (uint32_t *)out_dev, kind, max_levels, max_steps, time_limit_ns, grid, st));
     if (g->opt.loop_mode == 0) {
         cudaGraphExec_t &ex = g->exec[s][sssp ? 1 : 0];
         if (!ex) LB_TRY(build_exec(g, s, sssp, &ex));
@@ -609,7 +608,7 @@ lb_status run_query(lb_graph *g, int kind, int s, int32_t src, void *out_dev, in
             if (!*g->hflag) break;
         }
     }
-    LB_CU(launch_finish_query(p, st));
+    if (sssp) LB_CU(launch_finish_query(p, st));
     if (parents_dev) LB_CU(launch_parents(p, sssp, parents_dev, st));
     LB_CU(cudaEventRecord(g->ev_stop, st));
     LB_CU(cudaEventRecord(g->ev_done, st));

@@ -324,6 +324,16 @@ __device__ __forceinline__ void wflush_prefix(WB &b, WS &s, uint32_t cnt, const 
 }
 
 constexpr uint32_t kLaneGrains = 8;
+// Edge-id output: a flush whose entries average at least this many edges
+// writes entry by entry; below, lanes search each id's entry (7 dependent
+// shared-memory reads per id, but no idle lanes).  Measured on R-MAT scale
+// 20, highest-degree source: EP SSSP 4.10 -> 0.83 ms (its first step, 39460
+// edges that list 9.6M, 2276 -> 109 us); 4 / 8 / 16 / 32: 0.83 / 0.83 / 0.83 /
+// 0.86 ms.
+#ifndef LB_RUN_EDGES
+#define LB_RUN_EDGES 16
+#endif
+constexpr uint32_t kRunEdges = LB_RUN_EDGES;
 
 template <int KIND, bool TILED, class WB, class WS, class FO>
 __device__ __forceinline__ void wflush_write(const WB &b, const WS &s, uint32_t &cnt, const FO &o,
@@ -379,6 +389,25 @@ __device__ __forceinline__ void wflush_write(const WB &b, const WS &s, uint32_t 
             }
             ru += __shfl_sync(kFull, iu, 31);
             re += __shfl_sync(kFull, ie, 31);
+        }
+    } else if (KIND == kOutEdges && run_u >= kRunEdges * cnt) {
+        // long entries: the warp writes one entry's edge ids after another,
+        // 16 bytes per lane, instead of searching every id's entry
+        for (uint32_t i = 0; i < cnt; ++i) {
+            int32_t e = b.beg[i];
+            uint32_t d = b.deg[i];
+            int32_t *q = o.elist + ubase + s.pu[i];
+            const uint32_t head = min((uint32_t)((16u - ((uintptr_t)q & 15u)) & 15u) / 4u, d);
+            if (lane < head) q[lane] = e + (int32_t)lane;
+            q += head;
+            e += (int32_t)head;
+            d -= head;
+            for (uint32_t k = lane; k < d / 4u; k += 32) {
+                const int32_t x = e + 4 * (int32_t)k;
+                reinterpret_cast<int4 *>(q)[k] = make_int4(x, x + 1, x + 2, x + 3);
+            }
+            const uint32_t tail = d & ~3u;
+            if (tail + lane < d) q[tail + lane] = e + (int32_t)(tail + lane);
         }
     } else {
         for (uint32_t j = lane; j < run_u; j += 32) {
@@ -836,53 +865,96 @@ __device__ __forceinline__ uint64_t global_ns() {
     return t;
 }
 
-__device__ __forceinline__ void trace_append(Ctl *ctl, int32_t mode, int64_t list_size, int64_t edges) {
-    const uint32_t t = ctl->trace_len;
+// The loop state a step's last CTA needs, read in one go: read field by
+// field between the stores, each would be an L2 round trip of its own on the
+// path of every launch-per-level iteration.
+struct CtlSnap {
+    unsigned long long out_pack, sub_pack, relaxed;
+    uint64_t in_edges, step, max_steps, t_start, t_deadline;
+    uint32_t level, par, in_cnt, max_levels, error, trace_len, small_run;
+    uint32_t hp_kind, hp_from, hp_sub, hp_lvl, sub_in;
+};
+__device__ __forceinline__ CtlSnap ctl_snap(const Ctl *ctl) {
+    const volatile Ctl *c = ctl;
+    CtlSnap s;
+    s.out_pack = c->out_pack;
+    s.sub_pack = c->sub_pack;
+    s.relaxed = c->relaxed;
+    s.in_edges = c->in_edges;
+    s.step = c->step;
+    s.max_steps = c->max_steps;
+    s.t_start = c->t_start;
+    s.t_deadline = c->t_deadline;
+    s.level = c->level;
+    s.par = c->par;
+    s.in_cnt = c->in_cnt;
+    s.max_levels = c->max_levels;
+    s.error = c->error;
+    s.trace_len = c->trace_len;
+    s.small_run = c->small_run;
+    s.hp_kind = c->hp_kind;
+    s.hp_from = c->hp_from;
+    s.hp_sub = c->hp_sub;
+    s.hp_lvl = c->hp_lvl;
+    s.sub_in = c->sub_in;
+    return s;
+}
+
+__device__ __forceinline__ void trace_append(Ctl *ctl, const CtlSnap &s, int32_t mode, int64_t list_size,
+                                             int64_t edges) {
+    const uint32_t t = s.trace_len;
     if (t < (uint32_t)kTraceMax) {
-        ctl->trace[t].level = (int32_t)ctl->level;
+        ctl->trace[t].level = (int32_t)s.level;
         ctl->trace[t].mode = mode;
         ctl->trace[t].list_size = list_size;
         ctl->trace[t].edges = edges;
-        ctl->trace[t].t_ns = (int64_t)(global_ns() - ctl->t_start);
+        ctl->trace[t].t_ns = (int64_t)(global_ns() - s.t_start);
         ctl->trace_len = t + 1;
     }
 }
 
-__device__ __forceinline__ void set_loop(const StepParams &p, Ctl *ctl, bool more) {
-    if (ctl->level >= ctl->max_levels || ctl->step >= ctl->max_steps) {
-        if (more) ctl->error |= kErrIterCap;
+// level, step and in_edges: of the next step; err: error bits so far.
+__device__ __forceinline__ void set_loop(const StepParams &p, Ctl *ctl, const CtlSnap &s, uint32_t level,
+                                         uint64_t step, uint64_t in_edges, uint32_t err, bool more) {
+    const uint32_t err0 = err;
+    if (level >= s.max_levels || step >= s.max_steps) {
+        if (more) err |= kErrIterCap;
         more = false;
     }
-    if (more && global_ns() > ctl->t_deadline) {
-        ctl->error |= kErrDeadline;
+    if (more && global_ns() > s.t_deadline) {
+        err |= kErrDeadline;
         more = false;
     }
+    if (err != err0) atomicOr(&ctl->error, err);
     ctl->active = more ? 1u : 0u;
     if (p.use_cond) cudaGraphSetConditional(p.cond, more ? 1u : 0u);
-    if (p.small_edges > 0) ctl->small_run = ctl->in_edges <= (uint64_t)p.small_edges ? ctl->small_run + 1u : 0u;
+    if (p.small_edges > 0) ctl->small_run = in_edges <= (uint64_t)p.small_edges ? s.small_run + 1u : 0u;
 }
 
 // Finalise a plain (non-HP) step: the output list becomes the input list.
 // node_list: the output is a node / granule list needing a scan sentinel.
 __device__ __forceinline__ void finish_plain_step(const StepParams &p, Ctl *ctl, bool node_list, int64_t cap) {
     __threadfence();
-    const unsigned long long pk = ld_volatile(&ctl->out_pack);
-    int64_t cnt = (int64_t)(pk >> 32);
-    const int64_t edges = (int64_t)(pk & 0xFFFFFFFFull);
-    if (cnt > cap) { ctl->error |= kErrCapacity; cnt = cap; }
-    const int64_t step_edges = node_list ? (int64_t)ctl->in_edges : (int64_t)ctl->in_cnt;
-    trace_append(ctl, kModeRelax, ctl->in_cnt, step_edges);
-    ctl->relaxed += (unsigned long long)step_edges;
-    const uint32_t out = ctl->par ^ 1u;
+    const CtlSnap s = ctl_snap(ctl);
+    int64_t cnt = (int64_t)(s.out_pack >> 32);
+    const int64_t edges = (int64_t)(s.out_pack & 0xFFFFFFFFull);
+    if (cnt > cap) {
+        atomicOr(&ctl->error, kErrCapacity);
+        cnt = cap;
+    }
+    const int64_t step_edges = node_list ? (int64_t)s.in_edges : (int64_t)s.in_cnt;
+    trace_append(ctl, s, kModeRelax, s.in_cnt, step_edges);
+    ctl->relaxed = s.relaxed + (unsigned long long)step_edges;
+    const uint32_t out = s.par ^ 1u;
     if (node_list) p.lists[out].scan[cnt] = (int32_t)edges;
     ctl->par = out;
     ctl->in_cnt = (uint32_t)cnt;
     ctl->in_edges = (uint64_t)edges;
     ctl->out_pack = 0ull;
-    ctl->level += 1;
-    ctl->step += 1;
+    ctl->level = s.level + 1;
+    ctl->step = s.step + 1;
     ctl->blocks_done = 0;
-    set_loop(p, ctl, cnt > 0);
+    set_loop(p, ctl, s, s.level + 1, s.step + 1, (uint64_t)edges, 0u, cnt > 0);
     __threadfence();
 }
 

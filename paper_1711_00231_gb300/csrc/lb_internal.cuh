@@ -129,7 +129,7 @@ struct QuerySync {
 constexpr int32_t kFarWords = 16384;
 
 struct Ctl {
-    // query parameters (written by the prepare kernel)
+    // query parameters (written by the set-up kernel)
     uint32_t *status;
     int32_t src;
     int32_t kind;  // 0 BFS, 1 SSSP
@@ -162,7 +162,7 @@ struct Ctl {
     uint64_t max_steps;
     uint64_t step;
     uint64_t t_deadline;  // %globaltimer (ns) after which the loop stops
-    uint64_t t_start;     // %globaltimer (ns) when the query was prepared
+    uint64_t t_start;     // %globaltimer (ns) when the query was set up
     unsigned long long relaxed;
     LB_CTL_ALIGN unsigned long long pushes;
     uint32_t trace_len;
@@ -239,9 +239,8 @@ struct StepParams {
 // ---- launch entry points implemented by the strategy translation units --
 cudaError_t launch_step(int strategy, bool sssp, const StepParams &p, int grid, cudaStream_t st);
 int step_blocks_per_sm(int strategy, bool sssp, int ns_mode);
-cudaError_t launch_prepare(const StepParams &p, int32_t src, uint32_t *status, int kind, uint32_t max_levels,
-                           uint64_t max_steps, uint64_t time_limit_ns, cudaStream_t st);
-cudaError_t launch_init(const StepParams &p, int grid, cudaStream_t st);
+cudaError_t launch_init(const StepParams &p, int32_t src, uint32_t *status, int kind, uint32_t max_levels,
+                        uint64_t max_steps, uint64_t time_limit_ns, int grid, cudaStream_t st);
 cudaError_t launch_hp_mdt(const StepParams &p, int grid, cudaStream_t st);
 cudaError_t launch_small_levels(bool sssp, const StepParams &p, int grid, cudaStream_t st);
 int small_ctas_per_sm();

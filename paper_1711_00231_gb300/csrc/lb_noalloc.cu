@@ -132,9 +132,8 @@ extern "C" lb_status lb_bfs_wd_noalloc(const int64_t *offsets_dev, const int32_t
     if (vword & kErrShape)
         return na_fail(LB_ERR_ARG, "malformed CSR (offsets not 0..m and non-decreasing, or a column outside [0, n))");
     const uint32_t max_levels = (uint32_t)(n + 1);
-    e = launch_prepare(p, src, (uint32_t *)levels_dev, LB_KIND_BFS, max_levels, (uint64_t)1 << 40,
-                       (uint64_t)60 * 1000000000ull, st);
-    if (e == cudaSuccess) e = launch_init(p, grid, st);
+    e = launch_init(p, src, (uint32_t *)levels_dev, LB_KIND_BFS, max_levels, (uint64_t)1 << 40,
+                    (uint64_t)60 * 1000000000ull, grid, st);
     if (e != cudaSuccess) return na_fail(LB_ERR_CUDA, "launch", e);
     for (;;) {
         e = launch_step(LB_WD, false, p, grid, st);

@@ -817,7 +817,7 @@ __global__ void __launch_bounds__(kBlock, LB_SMALL_CTAS) k_small_levels(StepPara
         ctl->in_edges = (uint64_t)E;
         ctl->out_pack = 0ull;
         ctl->step = step0 + steps;
-        set_loop(p, ctl, in_cnt > 0);
+        set_loop(p, ctl, ctl_snap(ctl), level, step0 + steps, (uint64_t)E, 0u, in_cnt > 0);
         __threadfence();
     }
 }
@@ -890,8 +890,8 @@ __global__ void __launch_bounds__(kBlock) k_step_ep(StepParams p) {
 // ---------------------------------------------------------------------------
 // Hierarchical processing (Sec. III-C).  One launch is one step of the
 // super-iteration: either a sub-iteration over the current list (each entry
-// relaxes at most MDT edges; entries with edges left are pushed, with their
-// remaining range, to the next sub-list) or, when the list is shorter than
+// relaxes at most MDT edges, by a thread, a warp or the CTA; entries with
+// edges left are pushed, with their remaining range, to the next sub-list) or, when the list is shorter than
 // the threshold, one workload-decomposition step over everything left.
 // Nodes updated in any step go to the next super worklist.
 // ---------------------------------------------------------------------------
@@ -921,17 +921,23 @@ __device__ __forceinline__ void serve_range(const StepParams &p, Ctl *ctl, int64
     }
 }
 
-// The degree-binned step (HP's hp_mode 1 and NS's ns_mode 1): every entry
+// The degree-binned service (HP's sub-iterations and hp_mode 1, NS's ns_mode
+// 1): every entry
 // of the list is served in this one step at its own granularity -- an
 // entry of at most tmax edges by its own thread, one of at most
 // hp_warp_max edges by its warp (the warp takes its warp-class entries one
 // after another), a larger one by the whole CTA after the block's batches
 // (the CTA bin is a block-local list; when it is full the warp serves the
-// entry instead).  OUTK / TILED: what the pushes write (nodes with tile
+// entry instead).  cap: at most this many edges of an entry are served; the
+// warp calls rest(i, left?, first edge left, edges left) for its 32 entries.  OUTK / TILED: what the pushes write (nodes with tile
 // starts for HP, granules for NS).  Every thread of the block calls it.
-template <bool SSSP, int ITEMS, int OUTK, bool TILED, class FO>
+#ifndef LB_SPREAD_EDGES
+#define LB_SPREAD_EDGES 16
+#endif
+constexpr int64_t kSpreadEdges = LB_SPREAD_EDGES;
+template <bool SSSP, int ITEMS, int OUTK, bool TILED, class FO, class Rest>
 __device__ __forceinline__ void binned_step(const StepParams &p, Ctl *ctl, const NodeList &in, int64_t in_cnt,
-                                            int64_t tmax, uint32_t *status, uint32_t level, uint32_t *qcur,
+                                            int64_t cap, int64_t tmax, Rest rest, uint32_t *status, uint32_t level, uint32_t *qcur,
                                             WarpBuf &wb, WarpScratch &ws, uint32_t &cnt, const FO &o) {
     constexpr int kBigCap = 256;
     __shared__ int32_t s_big[kBigCap];
@@ -941,9 +947,16 @@ __device__ __forceinline__ void binned_step(const StepParams &p, Ctl *ctl, const
     __syncthreads();
     const int64_t wmax = p.hp_warp_max;
     const int64_t stride = (int64_t)gridDim.x * kBlock;
-    for (int64_t base = (int64_t)blockIdx.x * kBlock + warp * 32; base < in_cnt; base += stride) {
-        const int64_t i = base + lane;
-        int64_t cur = 0, len = 0;
+    // A warp's 32 entries are neighbours in the list, or, when entries are
+    // long, spread over it: neighbours have alike degrees (a hub's list holds
+    // the other hubs first), and a warp with 32 of them is what the whole
+    // step waits for.  Measured on R-MAT scale 20: HP BFS 1.06 -> 0.36 ms; from
+    // 8 / 16 / 64 edges per entry on: 0.360 / 0.360 / 0.393 ms.
+    const bool spread = (int64_t)ctl->in_edges >= kSpreadEdges * in_cnt;
+    const int64_t gw = (int64_t)blockIdx.x * kWarps + warp, warps = (int64_t)gridDim.x * kWarps;
+    for (int64_t base = spread ? 0 : gw * 32; base < in_cnt; base += stride) {
+        const int64_t i = spread ? base + (int64_t)lane * warps + gw : base + lane;
+        int64_t cur = 0, len = 0, left = 0;
         uint32_t du = 0;
         int cls = -1;  // -1 nothing to do, 0 thread, 1 warp, 2 CTA
         if (i < in_cnt) {
@@ -953,9 +966,13 @@ __device__ __forceinline__ void binned_step(const StepParams &p, Ctl *ctl, const
                 atomicOr(&ctl->error, kErrBounds);
             } else {
                 if (SSSP) du = sssp_source_dist(status, qcur, __ldg(in.v + i));
-                if (!SSSP || du != kInf) cls = len <= tmax ? 0 : (len <= wmax ? 1 : 2);
+                const int64_t take = len < cap ? len : cap;
+                if (!SSSP || du != kInf) cls = take <= tmax ? 0 : (take <= wmax ? 1 : 2);
+                left = len - take;
+                len = take;
             }
         }
+        rest(i, cls >= 0 && left > 0, cur + len, left);
         if (cls == 2) {
             const uint32_t slot = atomicAdd(&s_nbig, 1u);
             if (slot < (uint32_t)kBigCap) s_big[slot] = (int32_t)i;
@@ -970,25 +987,24 @@ __device__ __forceinline__ void binned_step(const StepParams &p, Ctl *ctl, const
             const uint32_t d0 = __shfl_sync(kFull, du, l);
             serve_range<SSSP, ITEMS, OUTK, TILED>(p, ctl, c0, c0 + n0, 32, d0, status, level, qcur, wb, ws, cnt, o);
         }
-        int64_t end = cls == 0 ? cur + len : cur;
+        // a thread takes ITEMS edges of its entry at a time, staged as in
+        // relax_items, so that their latencies overlap
+        const int64_t end = cls == 0 ? cur + len : cur;
         while (__any_sync(kFull, cur < end)) {
-            bool want = false;
-            int32_t v = 0;
-            int64_t vb = 0;
-            uint32_t vd = 0;
-            if (cur < end) {
-                v = __ldg(p.g.col + cur);
-                const bool hit = SSSP ? sssp_relax(status, qcur, v, du, __ldg(p.g.w + cur), ctl)
-                                      : bfs_claim(p.bitmap, status, v, level + 1);
-                if (hit) {
-                    vb = __ldg(p.g.off + v);
-                    vd = (uint32_t)(__ldg(p.g.off + v + 1) - vb);
-                    want = vd > 0;
-                }
-                ++cur;
+            bool ok[ITEMS];
+            int32_t vv[ITEMS];
+            uint32_t ww[ITEMS], dd[ITEMS];
+#pragma unroll
+            for (int it = 0; it < ITEMS; ++it) {
+                ok[it] = cur + it < end;
+                vv[it] = ok[it] ? __ldg(p.g.col + cur + it) : 0;
+                ww[it] = (SSSP && ok[it]) ? __ldg(p.g.w + cur + it) : 0u;
+                dd[it] = du;
             }
-            wpush(wb, cnt, want, v, vb, vd);
-            if (cnt > kWB - 32) wflush<OUTK, TILED>(wb, ws, cnt, o);
+            cur += ITEMS;
+            if (cnt > kWB - 32 * ITEMS) wflush<OUTK, TILED>(wb, ws, cnt, o);
+            relax_items<SSSP, ITEMS, OUTK, TILED, kLdRo, false>(ok, vv, ww, dd, p.g.off, p.bitmap, qcur, status, level,
+                                                               &ctl->error, wb, ws, cnt, o);
         }
     }
     __syncthreads();
@@ -996,7 +1012,8 @@ __device__ __forceinline__ void binned_step(const StepParams &p, Ctl *ctl, const
     for (uint32_t k = 0; k < nbig; ++k) {
         const int64_t i = s_big[k];
         const int64_t c0 = __ldg(in.beg + i);
-        const int64_t n0 = __ldg(in.scan + i + 1) - __ldg(in.scan + i);
+        const int64_t all = __ldg(in.scan + i + 1) - __ldg(in.scan + i);
+        const int64_t n0 = all < cap ? all : cap;
         const uint32_t d0 = SSSP ? sssp_source_dist(status, qcur, __ldg(in.v + i)) : 0u;
         // warp w takes the 32-edge stripes w, w + 8, w + 16, ... of the entry
         serve_range<SSSP, ITEMS, OUTK, TILED>(p, ctl, c0 + 32 * (int64_t)warp, c0 + n0, kBlock, d0, status, level,
@@ -1006,46 +1023,51 @@ __device__ __forceinline__ void binned_step(const StepParams &p, Ctl *ctl, const
 
 __device__ __forceinline__ void finish_hp_step(const StepParams &p, Ctl *ctl) {
     __threadfence();
-    const unsigned long long pk = ld_volatile(&ctl->out_pack);
-    const unsigned long long spk = ld_volatile(&ctl->sub_pack);
-    int64_t sub_cnt = (int64_t)(spk >> 32);
-    const int64_t sub_edges = (int64_t)(spk & 0xFFFFFFFFull);
-    if (sub_cnt > p.list_cap) { ctl->error |= kErrCapacity; sub_cnt = p.list_cap; }
-    const uint32_t kind = ctl->hp_kind;
-    const int64_t step_edges = kind == 1u ? (int64_t)ctl->in_edges - sub_edges : (int64_t)ctl->in_edges;
-    trace_append(ctl, kind == 1u ? kModeHpSub : (kind == 3u ? kModeHpBin : kModeHpWd), ctl->in_cnt, step_edges);
-    ctl->relaxed += (unsigned long long)step_edges;
-    ctl->step += 1;
+    const CtlSnap s = ctl_snap(ctl);
+    int64_t sub_cnt = (int64_t)(s.sub_pack >> 32);
+    const int64_t sub_edges = (int64_t)(s.sub_pack & 0xFFFFFFFFull);
+    if (sub_cnt > p.list_cap) {
+        atomicOr(&ctl->error, kErrCapacity);
+        sub_cnt = p.list_cap;
+    }
+    const uint32_t kind = s.hp_kind;
+    const int64_t step_edges = kind == 1u ? (int64_t)s.in_edges - sub_edges : (int64_t)s.in_edges;
+    trace_append(ctl, s, kind == 1u ? kModeHpSub : (kind == 3u ? kModeHpBin : kModeHpWd), s.in_cnt, step_edges);
+    ctl->relaxed = s.relaxed + (unsigned long long)step_edges;
+    ctl->step = s.step + 1;
     ctl->blocks_done = 0;
     const int64_t thr = p.hp_threshold;
     if (kind == 1u && sub_cnt > 0) {
-        const uint32_t so = ctl->hp_from == kHpFromSuper ? 0u : (ctl->sub_in ^ 1u);
+        const uint32_t so = s.hp_from == kHpFromSuper ? 0u : (s.sub_in ^ 1u);
         const bool sub_next = !(thr > 0 && sub_cnt < thr);
-        ctl->hp_lvl += 1;
+        ctl->hp_lvl = s.hp_lvl + 1;
         // a list within the first hp_depth of the chain gets its own MDT
         // (k_hp_mdt, before the next sub-iteration); later ones keep it
-        if (p.hp_depth > 1 && ctl->hp_lvl < (uint32_t)p.hp_depth && sub_next) ctl->hp_mdt_pending = 1;
+        if (p.hp_depth > 1 && s.hp_lvl + 1 < (uint32_t)p.hp_depth && sub_next) ctl->hp_mdt_pending = 1;
         p.subs[so].scan[sub_cnt] = (int32_t)sub_edges;
         ctl->hp_from = kHpFromSub;
         ctl->sub_in = so;
         ctl->in_cnt = (uint32_t)sub_cnt;
         ctl->in_edges = (uint64_t)sub_edges;
         ctl->sub_pack = 0ull;
-        ctl->hp_sub += 1;
+        ctl->hp_sub = s.hp_sub + 1;
         ctl->hp_kind = (thr > 0 && sub_cnt < thr) ? 2u : 1u;
-        set_loop(p, ctl, true);
+        set_loop(p, ctl, s, s.level, s.step + 1, (uint64_t)sub_edges, 0u, true);
     } else {
-        int64_t cnt = (int64_t)(pk >> 32);
-        const int64_t edges = (int64_t)(pk & 0xFFFFFFFFull);
-        if (cnt > p.list_cap) { ctl->error |= kErrCapacity; cnt = p.list_cap; }
-        const uint32_t out = ctl->par ^ 1u;
+        int64_t cnt = (int64_t)(s.out_pack >> 32);
+        const int64_t edges = (int64_t)(s.out_pack & 0xFFFFFFFFull);
+        if (cnt > p.list_cap) {
+            atomicOr(&ctl->error, kErrCapacity);
+            cnt = p.list_cap;
+        }
+        const uint32_t out = s.par ^ 1u;
         p.lists[out].scan[cnt] = (int32_t)edges;
         ctl->par = out;
         ctl->in_cnt = (uint32_t)cnt;
         ctl->in_edges = (uint64_t)edges;
         ctl->out_pack = 0ull;
         ctl->sub_pack = 0ull;
-        ctl->level += 1;
+        ctl->level = s.level + 1;
         ctl->hp_from = kHpFromSuper;
         ctl->hp_sub = 0;
         ctl->hp_mdt = (uint32_t)p.mdt;
@@ -1053,7 +1075,7 @@ __device__ __forceinline__ void finish_hp_step(const StepParams &p, Ctl *ctl) {
         ctl->hp_mdt_pending = 0;
         ctl->sub_maxdeg = 0ull;
         ctl->hp_kind = (thr > 0 && cnt < thr) ? 2u : (p.hp_mode == 1 ? 3u : 1u);
-        set_loop(p, ctl, cnt > 0);
+        set_loop(p, ctl, s, s.level + 1, s.step + 1, (uint64_t)edges, 0u, cnt > 0);
     }
     __threadfence();
 }
@@ -1087,7 +1109,8 @@ __global__ void __launch_bounds__(kBlock) k_step_ns_binned(StepParams p) {
     o.child_first = nullptr;
     const uint32_t warp = threadIdx.x >> 5;
     uint32_t cnt = 0;
-    binned_step<SSSP, ITEMS, kOutGranule, false>(p, ctl, p.lists[par], in_cnt, p.thread_max, status, level, qcur,
+    binned_step<SSSP, ITEMS, kOutGranule, false>(p, ctl, p.lists[par], in_cnt, INT64_MAX, p.thread_max,
+                                                 [](int64_t, bool, int64_t, int64_t) {}, status, level, qcur,
                                                  s_wb[warp], s_ws[warp], cnt, o);
     wflush<kOutGranule, false>(s_wb[warp], s_ws[warp], cnt, o);
     if (block_is_last(ctl) && threadIdx.x == 0) finish_plain_step(p, ctl, true, p.list_cap);
@@ -1130,63 +1153,32 @@ __global__ void __launch_bounds__(kBlock) k_step_hp(StepParams p) {
     uint32_t cnt = 0, scnt = 0;
     if (kind == 2u) {
         wd_walk<SSSP, ITEMS>(p, ctl, in, in_cnt, E, wb, ws, cnt, osup, status, level, qcur);
-    } else if (kind == 3u) {
-        // a thread serves at most min(MDT, thread_max) edges: on a skewed
-        // graph the histogram MDT runs into the thousands
-        const int64_t tmax = p.mdt < p.thread_max ? (int64_t)p.mdt : (int64_t)p.thread_max;
-        binned_step<SSSP, ITEMS, kOutNode, true>(p, ctl, in, in_cnt, tmax, status, level, qcur, wb, ws, cnt, osup);
     } else {
-        const int64_t mdt = (int64_t)ctl->hp_mdt;
+        // A sub-iteration (kind 1) relaxes at most MDT edges per entry and
+        // pushes what is left to the sub-list; the degree-binned step (kind
+        // 3) takes whole entries.  Either way an entry's edges go to a
+        // thread, its warp or the CTA by their number: a thread serves at
+        // most min(MDT, thread_max) edges, as on a skewed graph the
+        // histogram MDT runs into the thousands (R-MAT scale 20: 3946, and a
+        // thread per entry took 2.1 of the 3.2 ms of a BFS in one
+        // sub-iteration; binned and spread the sub-iteration takes 0.13 ms).
+        const int64_t cap = kind == 1u ? (int64_t)ctl->hp_mdt : INT64_MAX;
+        const int64_t mdt = kind == 1u ? cap : (int64_t)p.mdt;
+        const int64_t tmax = mdt < p.thread_max ? mdt : (int64_t)p.thread_max;
         const bool track = p.hp_depth > 1;  // the sub-list's largest remaining degree, for k_hp_mdt
-        const int64_t stride = (int64_t)gridDim.x * kBlock;
-        for (int64_t base = (int64_t)blockIdx.x * kBlock + warp * 32; base < in_cnt; base += stride) {
-            const int64_t i = base + lane;
-            int64_t cur = 0, end = 0, rest = 0;
-            uint32_t du = 0;
-            int32_t u = 0;
-            if (i < in_cnt) {
-                cur = __ldg(in.beg + i);
-                const int64_t len = __ldg(in.scan + i + 1) - __ldg(in.scan + i);
-                if (cur < 0 || len < 0 || cur + len > p.g.m) {
-                    atomicOr(&ctl->error, kErrBounds);
-                    cur = 0;
-                } else {
-                    const int64_t take = len < mdt ? len : mdt;
-                    end = cur + take;
-                    rest = len - take;
-                    u = __ldg(in.v + i);
-                    if (SSSP) du = sssp_source_dist(status, qcur, u);
+        binned_step<SSSP, ITEMS, kOutNode, true>(
+            p, ctl, in, in_cnt, cap, tmax,
+            [&](int64_t i, bool keep, int64_t first, int64_t left) {
+                // an entry skipped as redundant (SSSP, see sssp_source_dist) leaves no remainder
+                if (!__any_sync(kFull, keep)) return;
+                if (track) {
+                    const uint32_t mx = __reduce_max_sync(kFull, keep ? (uint32_t)left : 0u);
+                    if (lane == 0) atomicMax(&ctl->sub_maxdeg, (unsigned long long)mx);
                 }
-            }
-            // an entry skipped as redundant (SSSP, see sssp_source_dist) leaves no remainder
-            const bool keep = rest > 0 && (!SSSP || du != kInf);
-            if (track) {
-                const uint32_t mx = __reduce_max_sync(kFull, keep ? (uint32_t)rest : 0u);
-                if (lane == 0 && mx > 0) atomicMax(&ctl->sub_maxdeg, (unsigned long long)mx);
-            }
-            if (SSSP && du == kInf) end = cur;
-            wpush(sb, scnt, keep, u, end, (uint32_t)rest);
-            if (scnt > kWB - 32) wflush<kOutNode, true>(sb, ws, scnt, osub);
-            while (__any_sync(kFull, cur < end)) {
-                bool want = false;
-                int32_t v = 0;
-                int64_t vb = 0;
-                uint32_t vd = 0;
-                if (cur < end) {
-                    v = __ldg(p.g.col + cur);
-                    const bool hit = SSSP ? sssp_relax(status, qcur, v, du, __ldg(p.g.w + cur), ctl)
-                                          : bfs_claim(p.bitmap, status, v, level + 1);
-                    if (hit) {
-                        vb = __ldg(p.g.off + v);
-                        vd = (uint32_t)(__ldg(p.g.off + v + 1) - vb);
-                        want = vd > 0;
-                    }
-                    ++cur;
-                }
-                wpush(wb, cnt, want, v, vb, vd);
-                if (cnt > kWB - 32) wflush<kOutNode, true>(wb, ws, cnt, osup);
-            }
-        }
+                wpush(sb, scnt, keep, keep ? __ldg(in.v + i) : 0, first, (uint32_t)left);
+                if (scnt > kWB - 32) wflush<kOutNode, true>(sb, ws, scnt, osub);
+            },
+            status, level, qcur, wb, ws, cnt, osup);
     }
     wflush<kOutNode, true>(wb, ws, cnt, osup);
     wflush<kOutNode, true>(sb, ws, scnt, osub);

@@ -47,50 +47,49 @@ __device__ __forceinline__ int64_t source_units(int strategy, int64_t deg, int32
     return 1;
 }
 
-__global__ void k_prepare(StepParams p, int32_t src, uint32_t *status, int kind, uint32_t max_levels,
-                          uint64_t max_steps, uint64_t time_limit_ns) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    Ctl *c = p.ctl;
-    const int64_t deg = p.g.off[src + 1] - p.g.off[src];
-    c->status = status;
-    c->src = src;
-    c->kind = kind;
-    c->level = 0;
-    c->par = 0;
-    c->in_cnt = (uint32_t)source_units(p.strategy, deg, p.mdt);
-    c->in_edges = (uint64_t)deg;
-    c->out_pack = 0ull;
-    c->sub_pack = 0ull;
-    c->hp_from = kHpFromSuper;
-    c->hp_sub = 0;
-    c->sub_in = 0;
-    c->hp_kind = (p.hp_threshold > 0 && (int64_t)c->in_cnt < p.hp_threshold) ? 2u : (p.hp_mode == 1 ? 3u : 1u);
-    c->hp_mdt = (uint32_t)p.mdt;
-    c->small_pack[0] = c->small_pack[1] = c->small_pack[2] = 0ull;
-    c->bar_count = 0u;
-    c->bar_stop = 0u;
-    c->small_run = 0u;
-    c->hp_lvl = 0;
-    c->hp_mdt_pending = 0;
-    c->sub_maxdeg = 0ull;
-    c->blocks_done = 0;
-    c->active = 1;
-    c->error = 0;
-    c->max_levels = max_levels;
-    c->max_steps = max_steps;
-    c->t_start = global_ns();
-    c->t_deadline = c->t_start + time_limit_ns;
-    c->step = 0;
-    c->relaxed = 0ull;
-    c->pushes = 0ull;
-    c->trace_len = 0;
-}
-
-__global__ void k_init(StepParams p) {
-    const Ctl *c = p.ctl;
-    const int32_t src = c->src;
-    const bool sssp = c->kind == 1;
-    uint32_t *status = c->status;
+// Query set-up in one launch: the loop state (one thread), the output and the
+// bitmaps, the source's worklist.
+__global__ void k_init(StepParams p, int32_t src, uint32_t *status, int kind, uint32_t max_levels, uint64_t max_steps,
+                       uint64_t time_limit_ns) {
+    const bool sssp = kind == 1;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        Ctl *c = p.ctl;
+        const int64_t deg = p.g.off[src + 1] - p.g.off[src];
+        const uint32_t in_cnt = (uint32_t)source_units(p.strategy, deg, p.mdt);
+        const uint64_t t0 = global_ns();
+        c->status = status;
+        c->src = src;
+        c->kind = kind;
+        c->level = 0;
+        c->par = 0;
+        c->in_cnt = in_cnt;
+        c->in_edges = (uint64_t)deg;
+        c->out_pack = 0ull;
+        c->sub_pack = 0ull;
+        c->hp_from = kHpFromSuper;
+        c->hp_sub = 0;
+        c->sub_in = 0;
+        c->hp_kind = (p.hp_threshold > 0 && (int64_t)in_cnt < p.hp_threshold) ? 2u : (p.hp_mode == 1 ? 3u : 1u);
+        c->hp_mdt = (uint32_t)p.mdt;
+        c->small_pack[0] = c->small_pack[1] = c->small_pack[2] = 0ull;
+        c->bar_count = 0u;
+        c->bar_stop = 0u;
+        c->small_run = 0u;
+        c->hp_lvl = 0;
+        c->hp_mdt_pending = 0;
+        c->sub_maxdeg = 0ull;
+        c->blocks_done = 0;
+        c->active = 1;
+        c->error = 0;
+        c->max_levels = max_levels;
+        c->max_steps = max_steps;
+        c->t_start = t0;
+        c->t_deadline = t0 + time_limit_ns;
+        c->step = 0;
+        c->relaxed = 0ull;
+        c->pushes = 0ull;
+        c->trace_len = 0;
+    }
     const int64_t n = p.g.n;
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -223,14 +222,9 @@ cudaError_t launch_hp_mdt(const StepParams &p, int grid, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_prepare(const StepParams &p, int32_t src, uint32_t *status, int kind, uint32_t max_levels,
-                           uint64_t max_steps, uint64_t time_limit_ns, cudaStream_t st) {
-    k_prepare<<<1, 32, 0, st>>>(p, src, status, kind, max_levels, max_steps, time_limit_ns);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_init(const StepParams &p, int grid, cudaStream_t st) {
-    k_init<<<grid, kBlock, 0, st>>>(p);
+cudaError_t launch_init(const StepParams &p, int32_t src, uint32_t *status, int kind, uint32_t max_levels,
+                        uint64_t max_steps, uint64_t time_limit_ns, int grid, cudaStream_t st) {
+    k_init<<<grid, kBlock, 0, st>>>(p, src, status, kind, max_levels, max_steps, time_limit_ns);
     return cudaGetLastError();
 }
 
