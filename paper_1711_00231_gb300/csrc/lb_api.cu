@@ -579,8 +579,7 @@ lb_status run_query(lb_graph *g, int kind, int s, int32_t src, void *out_dev, in
         a.time_limit_ns = time_limit_ns;
         a.number = g->query_number;
         a.seg_cap = fast_seg_cap(g->n);
-        a.far_shift = 5;
-        while (((g->n - 1) >> a.far_shift) >= 32 * (int64_t)kFarWords) ++a.far_shift;
+        a.far_shift = far_shift(g->n);
         a.team = kFastTeam < grid ? kFastTeam : grid;
         a.fast_seg = a.team == kFastTeam ? (int4 *)(((uintptr_t)g->fast_seg + 15u) & ~(uintptr_t)15u) : nullptr;
         LB_CU(launch_query_wd(sssp, p, a, grid, st));

@@ -127,6 +127,11 @@ struct QuerySync {
 // Blocks of the far set's bitmap (SSSP with a distance threshold): at most
 // 32 * kFarWords blocks of 2^s >= 32 vertices.
 constexpr int32_t kFarWords = 16384;
+__host__ __device__ inline int32_t far_shift(int64_t n) {
+    int32_t s = 5;
+    while (((n - 1) >> s) >= 32 * (int64_t)kFarWords) ++s;
+    return s;
+}
 
 struct Ctl {
     // query parameters (written by the set-up kernel)

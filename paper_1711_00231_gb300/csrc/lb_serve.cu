@@ -9,6 +9,8 @@
 // (generation << 32 | next tile); the CTA that finishes a job's last tile
 // finalises it and opens the slot's next job, so iterations of different
 // queries interleave freely on the GPU and no grid-wide barrier exists.
+// While a query's lists are short, that CTA runs its iterations alone
+// (solo_levels).
 //
 // Requests arrive through a ring in pinned, device-mapped host memory: the
 // host writes a request and then bumps `submitted`; a CTA that wins the
@@ -35,6 +37,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include "lb_far.cuh"
 #include "lb_steps.cuh"
 
 namespace lbk {
@@ -92,12 +95,13 @@ struct Req {
 
 // A query's workspace (one block of the server's device pool, reserved by
 // the host before the request enters the ring): the visited / queued
-// bitmap halves and two worklists sized for its own graph (n vertices, m
+// bitmap halves, the far set's bits and two worklists sized for its own graph (n vertices, m
 // edges), each piece 256-byte aligned.
 struct WsLayout {
     int64_t bmw;       // words per bitmap half (a multiple of 4)
     int64_t cap;       // worklist entries
     int64_t tcap;      // tile-start entries per list
+    uint64_t far;      // byte offset of the far set's bits (SSSP)
     uint64_t list0;    // byte offset of list 0 (list 1 follows at list0 + list_bytes)
     uint64_t v, beg, scan, tstart;  // byte offsets inside a list
     uint64_t list_bytes;
@@ -109,7 +113,8 @@ __host__ __device__ inline WsLayout ws_layout(int64_t n, int64_t m) {
     L.bmw = ((n + 31) / 32 + 3) / 4 * 4;
     L.cap = n;
     L.tcap = m / kTileGrain + 2;
-    L.list0 = al256(8u * (uint64_t)L.bmw);
+    L.far = al256(8u * (uint64_t)L.bmw);
+    L.list0 = L.far + al256(4u * (uint64_t)(((n - 1) >> far_shift(n) >> 5) + 1));
     L.v = 0;
     L.beg = al256(4u * (uint64_t)L.cap);
     L.scan = L.beg + al256(4u * (uint64_t)L.cap);
@@ -186,6 +191,10 @@ struct Slot {
     unsigned long long t_admit;
     uint32_t *status;
     unsigned char *ws;  // the query's workspace (ws_layout of its graph): set at admission
+    // SSSP threshold: in force (kInf: none), width of the next interval,
+    // whether it has been set, the interval's lists and largest list
+    uint32_t far_T, far_delta, far_engaged, int_lists;
+    unsigned long long int_edges;
 };
 
 struct Shared {  // device-global control of the persistent kernel
@@ -354,9 +363,66 @@ __device__ int32_t slot_status(const Slot *S) {
     return LB_OK;
 }
 
-// Finalises the slot's job after its last tile (single thread).  Returns
-// true when the slot has a next job open.
-__device__ bool finish_job(const Params &P, Slot *S, uint32_t kind) {
+// What follows a job: nothing (the query is complete), its next job is open,
+// or the CTA goes on with the query by itself (solo_levels).
+enum : int { kAfterNone = 0, kAfterJob = 1, kAfterSolo = 2 };
+
+// Worklist iterations a query may take (with a threshold an interval's add
+// up to at most its vertices and one more).
+__device__ __forceinline__ uint32_t level_cap(const GraphDev &g, int32_t kind) {
+    return kind == 1 && g.n < 0x7FFFFF00ll ? 2u * (uint32_t)g.n + 64u : (uint32_t)g.n;
+}
+
+// A list the finishing CTA may go on with alone: few edges, short entries on
+// average, and room for every edge's push in the worklists.
+#ifndef LB_SOLO_EDGES
+#define LB_SOLO_EDGES 8192
+#endif
+constexpr uint32_t kSoloEdges = LB_SOLO_EDGES, kSoloAvgDeg = 8, kSoloMaxDeg = 64;
+__device__ __forceinline__ bool solo_fits(const WsLayout &W, int64_t cnt, uint64_t edges) {
+    return edges <= kSoloEdges && edges <= kSoloAvgDeg * (uint64_t)cnt && (int64_t)edges <= W.cap;
+}
+
+// The query's worklist is empty (or it was stopped): overflow check or
+// completion (single thread).
+__device__ int end_query(const Params &P, Slot *S, const GraphDev &g, int32_t kind) {
+    if (kind == 1 && (atomicOr(&S->error, 0u) & kErrSaturated)) {
+        open_job(S, kJobCheck, (uint32_t)((g.n + kInitChunk - 1) / kInitChunk));
+        return kAfterJob;
+    }
+    complete_query(P, S, slot_status(S));
+    return kAfterNone;
+}
+
+// SSSP, after a list of E edges in iteration `level` (single thread): the
+// interval's books, and the distance threshold once lists get long, by the
+// rule of the whole-query kernel with the sizes of a single CTA's levels
+// (long lists go to many CTAs at 15-25 us per iteration).
+#ifndef LB_SERVE_FAR_EDGES
+#define LB_SERVE_FAR_EDGES 4096
+#endif
+constexpr uint64_t kServeFarEdges = LB_SERVE_FAR_EDGES, kServeFarEarly = 16384;
+__device__ void far_account(Slot *S, const GraphDev &g, uint32_t level, uint64_t E) {
+    volatile Slot *V = S;
+    V->int_lists = V->int_lists + 1u;
+    V->int_edges = V->int_edges + E;
+    if (V->far_engaged || E < kServeFarEdges) return;
+    if (!(level >= 32u || (level >= 6u && E >= kServeFarEarly && V->relaxed < (unsigned long long)g.m / 4u))) return;
+    // first width: 32 * mean weight (of 64 evenly spaced edges) / mean degree
+    unsigned long long w = 0;
+#pragma unroll 16
+    for (int k = 0; k < 64; ++k) w += __ldg(g.w + ((int64_t)k * g.m >> 6));
+    const float d = 32.f * ((float)w / 64.f) * (float)g.n / (float)g.m;
+    const uint32_t delta = d < 1.f ? 1u : d > (float)kFarMaxDelta ? kFarMaxDelta : (uint32_t)d;
+    V->far_engaged = 1u;
+    V->far_delta = delta;
+    V->far_T = far_add(0u, delta);
+    V->int_lists = 0u;
+    V->int_edges = 0ull;
+}
+
+// Finalises the slot's job after its last tile (single thread).
+__device__ int finish_job(const Params &P, Slot *S, uint32_t kind) {
     const SlotState st = slot_state(S);
     const GraphDev g = P.graphs[st.graph];
     if (kind == kJobInit) {
@@ -369,7 +435,7 @@ __device__ bool finish_job(const Params &P, Slot *S, uint32_t kind) {
         if (deg == 0) {
             S->level = 1;
             complete_query(P, S, LB_OK);
-            return false;
+            return kAfterNone;
         }
         const WsLayout W = ws_layout(g.n, g.m);
         NodeList L = ws_list(st.ws, W, 0);
@@ -381,9 +447,10 @@ __device__ bool finish_job(const Params &P, Slot *S, uint32_t kind) {
         for (int64_t k = 0; k < grains && k < W.tcap; ++k) L.tstart[k] = 0;
         S->in_cnt = 1;
         S->in_edges = (uint64_t)deg;
+        if (solo_fits(W, 1, (uint64_t)deg)) return kAfterSolo;
         const int64_t Tj = job_tile(P, deg);
         open_job(S, kJobRelax, (uint32_t)((deg + Tj - 1) / Tj), (uint32_t)(Tj / kTileGrain));
-        return true;
+        return kAfterJob;
     }
     if (kind == kJobRelax) {
         const unsigned long long pk = ld_volatile(&S->out_pack);
@@ -395,26 +462,25 @@ __device__ bool finish_job(const Params &P, Slot *S, uint32_t kind) {
         S->level = st.level + 1;
         const uint32_t out = st.par ^ 1u;
         const uint32_t err = atomicOr(&S->error, 0u);
-        if (cnt > 0 && st.level + 1 <= (uint32_t)g.n && !(err & (kErrCapacity | kErrBounds))) {
+        const bool broken = (err & (kErrCapacity | kErrBounds)) != 0u;
+        if (st.kind == 1) far_account(S, g, st.level, st.in_edges);
+        const bool pull = st.kind == 1 && cnt == 0 && ((const volatile Slot *)S)->far_T != kInf;
+        if ((cnt > 0 || pull) && st.level + 1 <= level_cap(g, st.kind) && !broken) {
             ws_list(st.ws, W, out).scan[cnt] = (int32_t)edges;
             S->par = out;
             S->in_cnt = (uint32_t)cnt;
             S->in_edges = (uint64_t)edges;
             S->out_pack = 0ull;
+            if (pull || solo_fits(W, cnt, (uint64_t)edges)) return kAfterSolo;
             const int64_t Tj = job_tile(P, edges);
             open_job(S, kJobRelax, (uint32_t)((edges + Tj - 1) / Tj), (uint32_t)(Tj / kTileGrain));
-            return true;
+            return kAfterJob;
         }
-        if (cnt > 0 && !(err & (kErrCapacity | kErrBounds))) atomicOr(&S->error, kErrIterCap);
-        if (st.kind == 1 && (err & kErrSaturated)) {
-            open_job(S, kJobCheck, (uint32_t)((g.n + kInitChunk - 1) / kInitChunk));
-            return true;
-        }
-        complete_query(P, S, slot_status(S));
-        return false;
+        if (cnt > 0 && !broken) atomicOr(&S->error, kErrIterCap);
+        return end_query(P, S, g, st.kind);
     }
     complete_query(P, S, slot_status(S));  // kJobCheck
-    return false;
+    return kAfterNone;
 }
 
 // ---- tile bodies (block-wide) ------------------------------------------------
@@ -436,6 +502,11 @@ __device__ void init_tile(const Params &P, Slot *S, int64_t k) {
     for (int64_t w = w0 + threadIdx.x; w < w1; w += blockDim.x) {
         bitmap[w] = (!sssp && w == (src >> 5)) ? (1u << (src & 31)) : 0u;
         if (sssp) bitmap[W.bmw + w] = 0u;
+    }
+    if (sssp) {  // the far set's words this chunk reaches into
+        uint32_t *far = (uint32_t *)(st.ws + W.far);
+        const int32_t sh = far_shift(g.n) + 5;
+        for (int64_t w = (v0 >> sh) + threadIdx.x; w <= (v1 - 1) >> sh; w += blockDim.x) far[w] = 0u;
     }
 }
 
@@ -489,6 +560,12 @@ __device__ void relax_tile(const Params &P, Slot *S, int64_t t, int64_t ntiles, 
     o.claim_bitmap = SSSP ? qcur : bitmap;
     o.claim_status = st.status;
     o.claim_level = st.level;
+    if (SSSP) {
+        __shared__ FarSet s_far;
+        if (threadIdx.x == 0) s_far = FarSet{((const volatile Slot *)S)->far_T, far_shift(g.n), (uint32_t *)(st.ws + W.far)};
+        __syncthreads();
+        o.far = &s_far;
+    }
     uint32_t cnt = 0;
     wd_walk_tile<SSSP, ITEMS, kLdCg>(g, ws_list(st.ws, W, st.par), (int32_t)st.in_cnt, (uint32_t)st.in_edges,
                                      (uint32_t)(q * kTileGrain), (uint32_t)t, bitmap, qcur, st.status, st.level, &S->error, wb, ws, cnt, o);
@@ -534,6 +611,11 @@ __device__ void admit(const Params &P) {
         S->relaxed = 0ull;
         S->pushes = 0ull;
         S->out_pack = 0ull;
+        S->far_T = kInf;
+        S->far_delta = 0;
+        S->far_engaged = 0;
+        S->int_lists = 0;
+        S->int_edges = 0ull;
         bool valid = r.graph >= 0 && r.graph < P.ngraphs && r.out != 0ull && (r.kind == 0 || r.kind == 1);
         if (valid) {
             const GraphDev g = P.graphs[r.graph];
@@ -574,6 +656,338 @@ __device__ void release_admit(const Params &P) {
     atomicExch(&P.sh->admit_lock, 0u);
 }
 
+// ---- solo levels -----------------------------------------------------------
+// A query on a high-diameter graph is a chain of hundreds of small
+// iterations.  As jobs each took 11 us (24 us among 128 queries): claim, done
+// count, finalisation and the next job's opening are some fifteen dependent
+// L2 trips beside the tile's own.  The CTA that finishes a job whose next list
+// has at most kSoloEdges edges therefore goes on with the query alone, one
+// level after another with only block barriers between them, until the list
+// grows, the query ends or the launch has to end (the next job is then opened
+// as usual).  Lists are kept in the query's own worklists as {vertex, first
+// edge, degree}; four lanes take an entry, and a lane group has kE entries in
+// flight.  SSSP lists may hold a vertex twice (its repeat relaxes nothing);
+// an interval's pull runs here too.
+//
+// Measured: 512 x 543 grid alone in the engine, BFS 10.9 -> 4.0 us per
+// iteration, SSSP 17.4 -> 10.0 ms; a burst of 128 queries over 12 graphs 24.6
+// -> 13.1 ms.  kSoloEdges 4096 / 8192 / 16384: 15.0 / 13.7 / 19.1 ms (longer
+// lists are many rounds for one CTA); kE 2 / 3 / 4 / 6: 14.0 / 13.7 / 13.3 /
+// 15.0 ms; kServeFarEdges 2048 / 4096 / 8192: 13.9 / 13.7 / 14.9 ms.
+struct SoloState {
+    uint32_t out_n, out_e, out_maxdeg, fmin, leave;
+    FarSet far;
+    // the slot's threshold fields, kept here meanwhile
+    uint32_t engaged, delta, int_lists;
+    unsigned long long int_edges;
+};
+
+__device__ __forceinline__ void solo_push(const NodeList &L, int64_t cap, SoloState &q, bool want, int32_t v,
+                                          int32_t beg, int32_t deg) {
+    const unsigned m = __ballot_sync(kFull, want);
+    if (!m) return;
+    const uint32_t lane = lane_id();
+    const uint32_t e = __reduce_add_sync(kFull, want ? (uint32_t)deg : 0u);
+    const uint32_t md = __reduce_max_sync(kFull, want ? (uint32_t)deg : 0u);
+    uint32_t base = 0;
+    if (lane == 0) {
+        base = atomicAdd(&q.out_n, (uint32_t)__popc(m));
+        atomicAdd(&q.out_e, e);
+        atomicMax(&q.out_maxdeg, md);
+    }
+    base = __shfl_sync(kFull, base, 0);
+    const uint32_t slot = base + __popc(m & lanemask_lt());
+    if (want && (int64_t)slot < cap) {
+        L.v[slot] = v;
+        L.beg[slot] = beg;
+        L.scan[slot] = deg;
+    }
+}
+
+// Every thread of the CTA calls it.  Returns (to every thread) what follows.
+template <bool SSSP>
+__device__ __noinline__ int solo_levels(const Params &P, Slot *S, SoloState &q, WarpBuf &wb, uint64_t t_launch,
+                                        uint64_t &last_admit) {
+    constexpr int kLanes = 4, kE = 4;
+    constexpr uint32_t kGroups = kBlock / kLanes;
+    const uint32_t tid = threadIdx.x;
+    const SlotState st = slot_state(S);
+    const GraphDev g = P.graphs[st.graph];
+    const WsLayout W = ws_layout(g.n, g.m);
+    uint32_t *const bitmap = (uint32_t *)st.ws;
+    uint32_t *const status = st.status;
+    uint32_t level = st.level, b = st.par, n = st.in_cnt, e = (uint32_t)st.in_edges;
+    unsigned long long relaxed = ((const volatile Slot *)S)->relaxed;
+    uint32_t T = kInf, from = kInf;  // the threshold; where the next interval is measured from
+    if (tid == 0) {
+        q.out_n = q.out_e = q.out_maxdeg = 0u;
+        q.leave = 0u;
+        q.fmin = kInf;
+        if (SSSP) {
+            const volatile Slot *V = S;
+            q.far = FarSet{V->far_T, far_shift(g.n), (uint32_t *)(st.ws + W.far)};
+            q.engaged = V->far_engaged;
+            q.delta = V->far_delta;
+            q.int_lists = V->int_lists;
+            q.int_edges = V->int_edges;
+        }
+    }
+    __syncthreads();
+    if (SSSP) T = from = q.far.T;
+    // the regular list, with degrees in place of prefixes, into the other
+    // buffer; SSSP: drop its queued bits (solo levels set none)
+    {
+        const NodeList in = ws_list(st.ws, W, b), out = ws_list(st.ws, W, b ^ 1u);
+        uint32_t *const qn = queued_half(bitmap, W.bmw, level + 1u);
+        for (uint32_t i0 = 0; i0 < n; i0 += kBlock) {
+            const uint32_t i = i0 + tid;
+            int32_t v = 0, beg = 0, deg = 0;
+            if (i < n) {
+                v = ldcg(in.v + i);
+                beg = ldcg(in.beg + i);
+                deg = (i + 1 < n ? ldcg(in.scan + i + 1) : (int32_t)e) - ldcg(in.scan + i);
+                if (beg < 0 || deg < 0 || (int64_t)beg + deg > g.m || v < 0 || (int64_t)v >= g.n) {
+                    atomicOr(&S->error, kErrBounds);
+                    v = beg = deg = 0;
+                }
+                if (SSSP) atomicAnd(qn + ((uint32_t)v >> 5), ~(1u << ((uint32_t)v & 31u)));
+            }
+            solo_push(out, W.cap, q, i < n && deg > 0, v, beg, deg);
+        }
+        b ^= 1u;
+    }
+    uint32_t steps = 0;
+    for (;;) {
+        __syncthreads();
+        n = q.out_n;
+        e = q.out_e;
+        const uint32_t maxdeg = q.out_maxdeg;
+        const bool pull = SSSP && n == 0u && T != kInf && from != kInf;
+        // the list stays with this CTA while it fits and the launch may go
+        // on; clocks, the host's flag and admission every 16 levels (every level:
+        // serving burst 13.1 -> 14.2 ms)
+        const bool look = (steps++ & 15u) == 0u;
+        if (look && tid == 0) {
+            const uint64_t now = global_ns();
+            q.leave = now - t_launch > P.hard_ns || ld_acquire_sys32(&P.host->stop) != 0u ? 1u : 0u;
+            if (now - last_admit > kAdmitPeriodNs && __ldcg(&P.sh->active) < (uint32_t)P.nslots) {
+                last_admit = now;
+                bool admitted = false;
+                if (try_admit(P, &admitted)) release_admit(P);
+            }
+        }
+        __syncthreads();
+        if (tid == 0) q.out_n = q.out_e = q.out_maxdeg = 0u;
+        const bool leave = q.leave != 0u;
+        __syncthreads();
+        if (n == 0u && !pull) break;
+        if (level > level_cap(g, SSSP ? 1 : 0)) break;
+        if (n > 0u && (leave || e > kSoloEdges || maxdeg > kSoloMaxDeg || (int64_t)e > W.cap)) break;
+        if (n == 0u && leave) break;
+        const NodeList in = ws_list(st.ws, W, b), out = ws_list(st.ws, W, b ^ 1u);
+        if (SSSP && pull) {
+            // the next interval [T, from + delta), its width by the lists of the last one
+            const uint32_t T0 = T, T1 = far_add(from, q.delta);
+            uint32_t mn = kInf;
+            far_blocks(
+                status, g.n, q.far, 0u, 1u, true,
+                [&](int32_t v, uint32_t d) { solo_push(out, W.cap, q, d >= T0 && d < T1, v, 0, 0); },
+                [&](uint32_t d) {
+                    const bool k = d != kInf && d >= T1;
+                    if (k) mn = min(mn, d);
+                    return k;
+                });
+            mn = __reduce_min_sync(kFull, mn);
+            if (lane_id() == 0 && mn != kInf) atomicMin(&q.fmin, mn);
+            __syncthreads();
+            // the pulled vertices' edges, all at once (none: an entry without effect)
+            const uint32_t pulled = q.out_n;
+            uint32_t se = 0, md = 0;
+            for (uint32_t i = tid; i < pulled; i += kBlock) {
+                const int32_t v = ldcg(out.v + i);
+                const int32_t b0 = (int32_t)__ldg(g.off + v), d = (int32_t)__ldg(g.off + v + 1) - b0;
+                out.beg[i] = b0;
+                out.scan[i] = d;
+                se += (uint32_t)d;
+                md = max(md, (uint32_t)d);
+            }
+            se = __reduce_add_sync(kFull, se);
+            md = __reduce_max_sync(kFull, md);
+            if (lane_id() == 0) {
+                atomicAdd(&q.out_e, se);
+                atomicMax(&q.out_maxdeg, md);
+            }
+            // an empty interval: on to the nearest vertex left, if any
+            from = pulled > 0u ? T1 : q.fmin;
+            T = T1;
+            __syncthreads();
+            if (tid == 0) {
+                q.fmin = kInf;
+                if (q.int_lists > 0u) {
+                    const unsigned long long avg = q.int_edges / q.int_lists;
+                    if (avg < kSoloEdges / 8u && q.delta < kFarMaxDelta) q.delta *= 2u;
+                    if (avg > kSoloEdges / 2u) q.delta = max(q.delta / 2u, 1u);
+                }
+                q.int_lists = 0u;
+                q.int_edges = 0ull;
+            }
+            b ^= 1u;
+            continue;
+        }
+        for (uint32_t i0 = 0; i0 < n; i0 += kE * kGroups) {
+            int32_t xb[kE], xd[kE], longest = 0;
+            uint32_t du[kE];
+#pragma unroll
+            for (int k = 0; k < kE; ++k) {
+                const uint32_t i = i0 + k * kGroups + tid / kLanes;
+                xb[k] = i < n ? ldcg(in.beg + i) : 0;
+                xd[k] = i < n ? ldcg(in.scan + i) : 0;
+                du[k] = SSSP && i < n ? (uint32_t)ldcg(in.v + i) : 0u;
+            }
+#pragma unroll
+            for (int k = 0; k < kE; ++k) {
+                longest = max(longest, xd[k]);
+                if (SSSP && xd[k] > 0) du[k] = ldcg(status + du[k]);
+            }
+            for (int32_t r = (int32_t)(tid % kLanes); __any_sync(kFull, r < longest); r += kLanes) {
+                int32_t c[kE], b0[kE], b1[kE];
+                uint32_t w[kE], old[kE];
+#pragma unroll
+                for (int k = 0; k < kE; ++k) {
+                    c[k] = r < xd[k] ? __ldg(g.col + xb[k] + r) : -1;
+                    w[k] = SSSP && r < xd[k] ? __ldg(g.w + xb[k] + r) : 0u;
+                }
+#pragma unroll
+                for (int k = 0; k < kE; ++k) {
+                    old[k] = SSSP ? 0u : kInf;
+                    b0[k] = b1[k] = 0;
+                    if (SSSP) {
+                        const uint32_t s32 = du[k] + w[k];
+                        w[k] = (s32 < w[k] || s32 >= kSat) ? kSat : s32;
+                    }
+                    if (c[k] >= 0) {
+                        if (SSSP) old[k] = atomicMin(status + c[k], w[k]);
+                        else old[k] = atomicOr(bitmap + ((uint32_t)c[k] >> 5), 1u << ((uint32_t)c[k] & 31u));
+                        b0[k] = (int32_t)__ldg(g.off + c[k]);
+                        b1[k] = (int32_t)__ldg(g.off + c[k] + 1);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < kE; ++k) {
+                    bool want;
+                    if (SSSP) {
+                        want = w[k] < old[k];
+                        if (want && w[k] == kSat) atomicOr(&S->error, kErrSaturated);
+                        if (want && w[k] >= T) {
+                            const uint32_t blk = (uint32_t)c[k] >> q.far.shift;
+                            atomicOr(q.far.bits + (blk >> 5), 1u << (blk & 31u));
+                            want = false;
+                        }
+                    } else {
+                        want = !((old[k] >> ((uint32_t)c[k] & 31u)) & 1u);
+                        if (want) status[c[k]] = level + 1u;
+                    }
+                    solo_push(out, W.cap, q, want && b1[k] > b0[k], c[k], b0[k], b1[k] - b0[k]);
+                }
+            }
+        }
+        relaxed += e;
+        if (SSSP && !q.engaged && e >= kServeFarEdges) {  // uniform
+            __syncthreads();
+            if (tid == 0) {
+                volatile Slot *V = S;
+                V->relaxed = relaxed;
+                far_account(S, g, level, e);
+                if (V->far_engaged) {
+                    q.engaged = 1u;
+                    q.far.T = V->far_T;
+                    q.delta = V->far_delta;
+                    q.int_lists = 0u;
+                    q.int_edges = 0ull;
+                }
+            }
+            __syncthreads();
+            T = q.far.T;
+        } else if (SSSP && tid == 0) {
+            ++q.int_lists;
+            q.int_edges += e;
+        }
+        from = T;
+        level += 1u;
+        b ^= 1u;
+    }
+    // leave: the query ends, or a regular list goes to the next job
+    int after = kAfterNone;
+    const bool ends = (n == 0u && !(SSSP && T != kInf && from != kInf)) || level > level_cap(g, SSSP ? 1 : 0);
+    if (!ends && n > 0u) {
+        const NodeList in = ws_list(st.ws, W, b), out = ws_list(st.ws, W, b ^ 1u);
+        FlushOut o;
+        o.list = out;
+        o.elist = nullptr;
+        o.pack = &S->out_pack;
+        o.err = &S->error;
+        o.pushes = nullptr;
+        o.child_first = nullptr;
+        o.cap = W.cap;
+        o.tile_cap = W.tcap;
+        o.tile = (int32_t)kTileGrain;
+        o.mdt = 1;
+        NoScratch ns;
+        uint32_t cnt = 0;
+        uint32_t *const qb = queued_half(bitmap, W.bmw, level + 1u);
+        for (uint32_t i0 = 0; i0 < n; i0 += kBlock) {
+            const uint32_t i = i0 + tid;
+            const int32_t v = i < n ? ldcg(in.v + i) : 0;
+            // (a pulled vertex may have no edges: a regular list has no such entries)
+            bool want = i < n && ldcg(in.scan + i) > 0;
+            if (SSSP && want) {
+                // each vertex once, with the queued bit of the level before
+                const uint32_t bit = 1u << ((uint32_t)v & 31u);
+                want = !(atomicOr(qb + ((uint32_t)v >> 5), bit) & bit);
+            }
+            wpush(wb, cnt, want, v, i < n ? ldcg(in.beg + i) : 0, i < n ? (uint32_t)ldcg(in.scan + i) : 0u);
+            if (cnt > kWB - 32) wflush<kOutNode, true>(wb, ns, cnt, o);
+        }
+        wflush_block<kOutNode, true>(wb, ns, cnt, o);
+    }
+    __syncthreads();
+    __shared__ int s_after;
+    if (tid == 0) {
+        __threadfence();
+        S->level = level;
+        S->relaxed = relaxed;
+        if (SSSP) {
+            S->far_T = T;
+            S->far_delta = q.delta;
+            S->int_lists = q.int_lists;
+            S->int_edges = q.int_edges;
+        }
+        if (ends) {
+            if (n > 0u) atomicOr(&S->error, kErrIterCap);
+            s_after = end_query(P, S, g, SSSP ? 1 : 0);
+        } else {
+            // (an empty list with a threshold in force and the launch ending:
+            // one empty tile, after which the pull comes up again)
+            const unsigned long long pk = ld_volatile(&S->out_pack);
+            const uint32_t cnt = (uint32_t)(pk >> 32);
+            const int64_t edges = (int64_t)(pk & 0xFFFFFFFFull);
+            ws_list(st.ws, W, b ^ 1u).scan[cnt] = (int32_t)edges;
+            S->par = b ^ 1u;
+            S->in_cnt = cnt;
+            S->in_edges = (uint64_t)edges;
+            S->out_pack = 0ull;
+            const int64_t Tj = job_tile(P, edges);
+            const int64_t tiles = (edges + Tj - 1) / Tj;
+            open_job(S, kJobRelax, (uint32_t)(tiles > 0 ? tiles : 1), (uint32_t)(Tj / kTileGrain));
+            s_after = kAfterJob;
+        }
+    }
+    __syncthreads();
+    after = s_after;
+    __syncthreads();
+    return after;
+}
+
 // ---- the persistent kernel -------------------------------------------------
 
 template <int ITEMS>
@@ -585,6 +999,8 @@ __global__ void __launch_bounds__(kBlock, LB_SERVE_MIN_BLOCKS) k_serve(Params P)
     __shared__ long long s_tile;
     __shared__ int s_exit;
     __shared__ uint32_t s_scan_from;
+    __shared__ int s_next;
+    __shared__ SoloState s_solo;
     const uint32_t warp = threadIdx.x >> 5;
     uint64_t idle_since = 0;
     uint64_t last_admit = 0;
@@ -803,12 +1219,22 @@ __global__ void __launch_bounds__(kBlock, LB_SERVE_MIN_BLOCKS) k_serve(Params P)
 #endif
             __threadfence();
             const uint32_t d = atomicAdd(&S->job_done, 1u);
-            bool reopened = false;
+            s_next = kAfterNone;
             if (d == s_tiles - 1) {
                 __threadfence();
-                reopened = finish_job(P, S, kind);
+                s_next = finish_job(P, S, kind);
                 PF_ADD(6, 1);
             }
+        }
+        __syncthreads();
+        if (s_next == kAfterSolo) {
+            const int after = ((const volatile Slot *)S)->kind == 1
+                                  ? solo_levels<true>(P, S, s_solo, s_wb[warp], t_launch, last_admit)
+                                  : solo_levels<false>(P, S, s_solo, s_wb[warp], t_launch, last_admit);
+            if (threadIdx.x == 0) s_next = after;
+        }
+        if (threadIdx.x == 0) {
+            const bool reopened = s_next == kAfterJob;
 #if LB_SERVE_PROFILE
             long long c_d = clock64();
             PF_ADD(3, c_d - c_b);

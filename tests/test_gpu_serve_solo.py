@@ -1,0 +1,67 @@
+"""Queries that one CTA of the serving kernel runs alone (short lists), with
+the distance threshold of SSSP: results must equal the oracle's when lists
+move between the single CTA and many, at the rule's sizes, across launches
+that end part way, and with saturated distances."""
+import numpy as np
+import pytest
+
+import graphgen as gg
+import oracle
+from paper_1711_00231_gb300 import lb
+from paper_1711_00231_gb300 import serve as sv
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_1711_00231_gb300 import _build
+    _build.build()
+
+
+def fan(k, deg):
+    """A source, k middle vertices of out-degree deg, a shared layer, a tail."""
+    mid = 1 + np.arange(k)
+    low = 1 + k + np.arange(max(deg, 1))
+    src = np.concatenate([np.zeros(k, int), np.repeat(mid, deg), low])
+    dst = np.concatenate([mid, np.tile(low, k)[:k * deg], np.full(low.size, 1 + k + low.size)])
+    n = 2 + k + low.size
+    return gg.from_edges(n, src, dst, 1 + (np.arange(src.size) * 37) % 200)
+
+
+def graphs():
+    over = gg.grid(40, 40, seed=1)
+    over.weights[:] = np.random.default_rng(0).integers(1 << 27, 1 << 30, over.m)
+    heavy = gg.grid(160, 170, seed=4)
+    heavy.weights[:] = np.where(np.random.default_rng(1).random(heavy.m) < 0.5, 0, 100000)
+    return [gg.grid(300, 333, seed=2), gg.grid(700, 650, seed=3), gg.rmat(13, 8, seed=5), gg.erdos_renyi(40000, 160000, seed=6),
+            fan(8, 64), fan(8, 65), fan(1000, 8), fan(1100, 8), gg.from_edges(3, [0, 1], [1, 2], [4, 5]),
+            gg.from_edges(1, [], [], []), over, heavy]
+
+
+@pytest.mark.parametrize("launch_ms", [0, 1])
+def test_solo_levels_match_oracle(launch_ms):
+    import torch
+    cg = graphs()
+    G = [lb.Graph.from_csr(g) for g in cg]
+    S = sv.Server(G, slots=24, mem_fraction=0.05, launch_ms=launch_ms)
+    try:
+        reqs = []
+        for gi, g in enumerate(cg):
+            for src in sorted({0, g.n // 2, g.n - 1}):
+                reqs += [sv.Request(0.0, gi, int(src), "bfs"), sv.Request(0.0, gi, int(src), "sssp")]
+        outs = [torch.empty(cg[r.graph].n, dtype=torch.int32, device="cuda") for r in reqs]
+        status = S.run_batch(reqs, outs, timeout_s=120.0)
+        torch.cuda.synchronize()
+        for r, o, st in zip(reqs, outs, status):
+            g, got = cg[r.graph], o.cpu().numpy()
+            if r.kind == "bfs":
+                assert st == lb.LB_OK and np.array_equal(got, oracle.bfs(g, r.src)[0]), (r.graph, r.src)
+            else:
+                ref, ov = oracle.dijkstra(g, r.src)
+                assert st == (lb.LB_ERR_OVERFLOW if ov else lb.LB_OK), (r.graph, r.src, st)
+                assert np.array_equal(got.view(np.uint32), ref), (r.graph, r.src)
+    finally:
+        S.close()
+        for g in G:
+            g.close()
