@@ -91,7 +91,10 @@ typedef struct lb_options {
     int32_t wd_tile;       /* largest WD tile in worklist edges: 256..32768,
                               a multiple of 256 (8192); each iteration uses
                               the smallest multiple of 256 up to this that
-                              gives every CTA about two tiles */
+                              gives every CTA about two tiles.  WD's device
+                              loop walks long lists (16 * 256 edges per warp
+                              and more) in slices that warps claim, of at
+                              most this many edges (BFS) or half (SSSP) */
     int32_t ctas_per_sm;   /* CTAs per SM the fixed relax grid is sized for;
                               0 = the occupancy limit */
     int32_t hp_mode;       /* HP form: 0 = the paper's sub-iterations (Sec.

@@ -119,6 +119,9 @@ struct QuerySync {
         uint32_t far_min;      // pull step: smallest distance left in the far set
         uint32_t maxdeg;       // largest degree listed
     } pack[3];  // step L counts its output in pack[L % 3]
+    struct alignas(128) Claim {
+        uint32_t next;  // slices of a long list claimed so far
+    } claim[3];         // step L claims from claim[L % 3]
     alignas(128) unsigned long long fast_pack[2];  // fast levels: list counter of the way back
     alignas(128) uint32_t team_here;  // team ranks taken
     uint32_t sm_ctas[kMaxSms];        // CTAs per SM

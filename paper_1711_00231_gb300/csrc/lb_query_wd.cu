@@ -478,6 +478,7 @@ __device__ __forceinline__ bool fast_levels(const StepParams &p, const QueryArgs
                 sync->pack[k].v = 0ull;
                 sync->pack[k].far_min = kInf;
                 sync->pack[k].maxdeg = 0u;
+                sync->claim[k].next = 0u;
             }
         if (tid == 0) ++q.fast_conv;
     }
@@ -667,6 +668,69 @@ __device__ __noinline__ void pull_level(const StepParams &p, const QueryArgs &a,
 
 // One regular level up to its barrier: the walk over the list's tiles and
 // the flushes.
+// Long lists are walked in slices that the warps claim one by one, in list
+// order, instead of two tiles per CTA laid down ahead.  A warp's time per
+// edge depends on what it finds (candidates, flushes, hubs, the die its
+// lines live on): with the fixed split the grid waited 50-155 us per level
+// of 0.8-1.75 ms at scale 24 for its last CTA (measured with per-CTA
+// clocks), and a 4096-edge slice starts 4x less often than a 1024-edge one
+// (a start is a chain of ~5 dependent loads, ~1.8 us).  R-MAT edge factor
+// 32, highest-degree source, fixed -> claimed: BFS scale 21 294 -> 284, 22
+// 500 -> 476, 23 891 -> 836, 24 1706 -> 1601 us; SSSP 1228 -> 1217, 1994
+// -> 1950, 3367 -> 3135, 5466 -> 5060 us.
+//
+// A slice is wd_tile edges (BFS) or half of that (SSSP: list order keeps
+// the distances fresher; 4096 against 8192 / 16384 edges: 5.06 / 5.35 / 5.67
+// ms), at most half a warp's share; when less than two such rounds are left,
+// slices halve from half of what is left down to LB_SLICE_LOW grains (1 / 2
+// / 4 grains: BFS 1613 / 1607 / 1617, SSSP 5111 / 5094 / 5122 us).  A claim is one
+// atomic on one word, made while the warp walks the slice before: 2048-edge
+// slices (BFS 1645 us) and 1024-edge slices (1803 us) pay for the starts and
+// the claims.
+//
+// Lists of fewer than LB_CLAIM_SHARE grains per warp keep the fixed split:
+// there the claimed slices become so short that their starts cost what the
+// balance gains (scale 20, edge factor 16, 6-12 grains per warp: BFS 134 ->
+// 138, SSSP 471 -> 476 us; a line at 8 / 16 / 32 at scale 21: BFS 284 / 284 /
+// 289 us).
+#ifndef LB_CLAIM_SHARE
+#define LB_CLAIM_SHARE 16
+#endif
+#ifndef LB_SLICE_LOW
+#define LB_SLICE_LOW 2
+#endif
+
+// Grains of a full slice; share: grains per warp, at least 2.
+template <bool SSSP>
+__device__ __forceinline__ uint32_t full_slice(uint32_t share, uint32_t tile) {
+    return min(max(tile / (uint32_t)(SSSP ? 2 * kTileGrain : kTileGrain), 1u), share / 2u);
+}
+
+// Slice k of a list claimed in slices: its first edge and its edges.  Slices
+// follow one another without gaps for every k; the first past the list's end
+// tells a warp that it is done (k stays below the list's grains + warps).
+template <bool SSSP>
+__device__ __forceinline__ void claimed_slice(uint32_t k, uint32_t share, uint32_t tile, uint32_t warps, uint32_t &w0,
+                                              uint32_t &len) {
+    uint32_t s = full_slice<SSSP>(share, tile);
+    const uint32_t full = (share - s) / s;  // rounds of the grid in slices of s grains
+    uint32_t pos = 0;
+    if (k >= full * warps) {
+        k -= full * warps;
+        pos = full * warps * s;
+        uint32_t r = share - full * s;  // grains left per warp
+        s = max(r / 2u, (uint32_t)LB_SLICE_LOW);
+        while (s > (uint32_t)LB_SLICE_LOW && k >= warps) {
+            pos += warps * s;
+            k -= warps;
+            r -= s;
+            s = max(r / 2u, (uint32_t)LB_SLICE_LOW);
+        }
+    }
+    w0 = (pos + k * s) * (uint32_t)kTileGrain;
+    len = s * (uint32_t)kTileGrain;
+}
+
 template <bool SSSP, int ITEMS>
 __device__ __forceinline__ void regular_level(const StepParams &p, const QueryArgs &a, QuerySync *sync, QueryState &q,
                                            WarpBufT<SSSP ? LB_KWB_WD_SSSP : LB_KWB_WD_BFS> &wb, uint32_t me,
@@ -710,11 +774,20 @@ __device__ __forceinline__ void regular_level(const StepParams &p, const QueryAr
     o.claim_status = status;
     o.claim_level = level;
     uint32_t cnt = 0;
+    const uint32_t warp = threadIdx.x >> 5, warps = ctas * kWarps;
+    const uint32_t share = E / ((uint32_t)kTileGrain * warps);  // grains per warp
+    const bool claims = share >= (uint32_t)LB_CLAIM_SHARE;  // a team's lists are far shorter
     const uint32_t T = (uint32_t)iteration_tile(E, ctas, p.tile);
-    const uint32_t ntiles = (E + T - 1u) / T;
-    for (uint32_t t = me; t < ntiles; t += ctas)
-        wd_walk_tile<SSSP, ITEMS, kLdPlain>(p.g, in, (int32_t)in_cnt, E, T, t, p.bitmap, qcur, status, level,
-                                            &ctl->error, wb, ns, cnt, o);
+    uint32_t len = claims ? full_slice<SSSP>(share, (uint32_t)p.tile) * (uint32_t)kTileGrain : T / kWarps;
+    uint32_t w0 = (me * kWarps + warp) * len;
+    while (w0 < E) {  // warp-uniform
+        uint32_t k = 0;  // the next slice, claimed ahead
+        if (claims && lane_id() == 0) k = atomicAdd(&sync->claim[level % 3u].next, 1u);
+        wd_walk_slice<SSSP, ITEMS, kLdPlain>(p.g, in, (int32_t)in_cnt, E, w0, min(w0 + len, E), p.bitmap, qcur, status,
+                                             level, &ctl->error, wb, ns, cnt, o);
+        if (claims) claimed_slice<SSSP>(warps + __shfl_sync(kFull, k, 0), share, (uint32_t)p.tile, warps, w0, len);
+        else w0 += warps * len;
+    }
     wflush_block<kOutNode, true>(wb, ns, cnt, o);
 }
 
@@ -881,6 +954,7 @@ __global__ void __launch_bounds__(kBlock, SSSP ? LB_QUERY_MIN_BLOCKS_SSSP : LB_Q
         if (q.rank == 0u && threadIdx.x == 0) {
             sync->pack[(level + 1u) % 3u].v = 0ull;
             sync->pack[(level + 1u) % 3u].maxdeg = 0u;
+            sync->claim[(level + 1u) % 3u].next = 0u;
             if (SSSP) sync->pack[(level + 1u) % 3u].far_min = kInf;
         }
         if (SSSP && pull) pull_level(p, a, sync, q, s_wb[threadIdx.x >> 5], me, ctas);

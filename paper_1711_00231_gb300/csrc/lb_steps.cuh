@@ -95,18 +95,6 @@ __host__ __device__ constexpr bool wd_run_loop() {
 #define LB_SSSP_SKIP_STALE 1
 #endif
 
-// A warp's slice that starts on a tile-start grain takes its first list
-// entry from the recorded tile starts instead of a warp-wide search (SSSP,
-// and BFS in the persistent kernels).  Measured: R-MAT scale 24 SSSP 1.2%
-// faster, 4096^2 grid BFS 2.6% and SSSP 4.4% faster; the single-level BFS
-// step keeps the search (2% slower with the lookup: more spills).
-#ifndef LB_WD_GRAIN_START
-#define LB_WD_GRAIN_START 1
-#endif
-template <bool SSSP, int LD>
-__host__ __device__ constexpr bool wd_grain_start() {
-    return LB_WD_GRAIN_START && (SSSP || LD != 0);
-}
 // The final flush of a WD iteration (and of a serving RELAX tile) as one
 // list reservation per CTA (wflush_block) instead of one per warp.
 #ifndef LB_BLOCK_FLUSH
@@ -333,7 +321,10 @@ __device__ __forceinline__ KT warp_search(const int32_t *scan, KT lo, KT hi, IT 
     return lo;
 }
 
-// The walk of one tile with a 64-entry window of the list in registers.
+// The walk of one warp's slice, list edges [w0u, w1u) (w0u < w1u <= E), with
+// a 64-entry window of the list in registers.  A slice that starts on a
+// tile-start grain takes its first entry from the recorded tile starts,
+// another one searches between the two grains around it.
 // Lane l holds entries kb + l and kb + 32 + l: the entry's first list edge
 // s, the delta d = first CSR edge - s (an edge's CSR index is d + list
 // edge) and, for SSSP, the distance du its edges relax with (kInf when the
@@ -347,46 +338,28 @@ __device__ __forceinline__ KT warp_search(const int32_t *scan, KT lo, KT hi, IT 
 // 32 positions) and takes its fields from the window by shuffle.  32-bit
 // list edges and edge ids (< 2^31, checked when the graph is created).
 template <bool SSSP, int R, int LD, class WB, class WS, class FO>
-__device__ __forceinline__ void wd_walk_win(const GraphDev &g, const NodeList &in, int32_t in_cnt, uint32_t E,
-                                            uint32_t T, uint32_t t, uint32_t *bitmap, uint32_t *qcur,
-                                            uint32_t *status, uint32_t level, uint32_t *err, WB &wb,
-                                            WS &ws, uint32_t &cnt, const FO &o) {
-    // 32-bit tile arithmetic: a list has < 2^31 edges and a tile <= 32768
-    const uint32_t q = T / (uint32_t)kTileGrain;
-    const uint32_t W = T / kWarps;  // edges per warp and tile (a multiple of 32)
+__device__ __forceinline__ void wd_walk_slice(const GraphDev &g, const NodeList &in, int32_t in_cnt, uint32_t E,
+                                              uint32_t w0u, uint32_t w1u, uint32_t *bitmap, uint32_t *qcur,
+                                              uint32_t *status, uint32_t level, uint32_t *err, WB &wb,
+                                              WS &ws, uint32_t &cnt, const FO &o) {
     const uint32_t lane = lane_id();
-    const uint32_t warp = threadIdx.x >> 5;
-    const uint32_t e0 = t * T;
-    const uint32_t e1 = min(e0 + T, E);
-    const uint32_t w0u = e0 + warp * W;
-    if (w0u >= e1) return;  // warp-uniform
-    const int32_t w0 = (int32_t)w0u;
-    // A slice that starts on a tile-start grain (every slice of a tile of
-    // a multiple of 8 x 256 edges) takes its first entry from the tile
-    // starts the push recorded; the load is issued with the tile's bounds.
-    const bool on_grain = wd_grain_start<SSSP, LD>() && (w0 & (int32_t)(kTileGrain - 1)) == 0;
-    const int32_t kg = on_grain ? ld_list<LD>(in.tstart + (w0 >> 8)) : 0;
-    const int32_t i0 = ld_list<LD>(in.tstart + t * q);
-    const int32_t ihiK = e0 + T < E ? min(ld_list<LD>(in.tstart + (t + 1u) * q) + 1, in_cnt) : in_cnt;
+    // the slice's first and last entries lie between the entries at the
+    // tile-start grains around it (loads issued together)
+    const uint32_t gend = (w1u + (uint32_t)kTileGrain - 1u) / (uint32_t)kTileGrain;
+    const int32_t i0 = ld_list<LD>(in.tstart + w0u / (uint32_t)kTileGrain);
+    const int32_t ihiK = gend * (uint32_t)kTileGrain < E ? min(ld_list<LD>(in.tstart + gend) + 1, in_cnt) : in_cnt;
     if (i0 < 0 || i0 >= ihiK) {
         if (lane == 0) atomicOr(err, kErrBounds);
         return;
     }
-    const int32_t w1 = (int32_t)min(w0u + W, e1);
+    const int32_t w0 = (int32_t)w0u, w1 = (int32_t)w1u;
     const int32_t m = (int32_t)g.m;
     const bool vec_ok = wd_vec<SSSP, R>() &&
                         ((reinterpret_cast<uintptr_t>(g.col) | (SSSP ? reinterpret_cast<uintptr_t>(g.w) : 0u)) &
                          15u) == 0;
-    int32_t kcur;
-    if (on_grain) {
-        if (kg < i0 || kg >= ihiK) {
-            if (lane == 0) atomicOr(err, kErrBounds);
-            return;
-        }
-        kcur = kg;
-    } else {
-        kcur = warp_search<LD, uint32_t, int32_t>(in.scan, i0, ihiK, (uint32_t)w0, lane);
-    }
+    int32_t kcur = i0;
+    if ((w0u & (uint32_t)(kTileGrain - 1)) != 0u)
+        kcur = warp_search<LD, uint32_t, int32_t>(in.scan, i0, ihiK, w0u, lane);
     int32_t kb = kcur;
     int32_t s0 = INT32_MAX, d0 = 0, s1 = INT32_MAX, d1 = 0;
     uint32_t u0 = kInf, u1 = kInf;  // SSSP: distance the entry relaxes with
@@ -580,14 +553,19 @@ __device__ __forceinline__ void wd_walk_win(const GraphDev &g, const NodeList &i
     }
 }
 
-// One tile of the walk.  LD selects how everything other CTAs write is read
-// (kLdRo, kLdCg or kLdPlain).
+// One tile of the walk: each warp takes a T / kWarps-edge slice.  LD selects
+// how everything other CTAs write is read (kLdRo, kLdCg or kLdPlain).
 template <bool SSSP, int STEPS, int LD, class WB, class WS, class FO>
 __device__ __forceinline__ void wd_walk_tile(const GraphDev &g, const NodeList &in, int32_t in_cnt, uint32_t E,
                                              uint32_t T, uint32_t t, uint32_t *bitmap, uint32_t *qcur,
                                              uint32_t *status, uint32_t level, uint32_t *err, WB &wb,
                                              WS &ws, uint32_t &cnt, const FO &o) {
-    wd_walk_win<SSSP, STEPS, LD>(g, in, in_cnt, E, T, t, bitmap, qcur, status, level, err, wb, ws, cnt, o);
+    // 32-bit tile arithmetic: a list has < 2^31 edges and a tile <= 32768
+    const uint32_t W = T / kWarps;  // a multiple of 32
+    const uint32_t w0 = t * T + (threadIdx.x >> 5) * W;
+    const uint32_t w1 = min(min(t * T + T, E), w0 + W);
+    if (w0 >= w1) return;  // warp-uniform
+    wd_walk_slice<SSSP, STEPS, LD>(g, in, in_cnt, E, w0, w1, bitmap, qcur, status, level, err, wb, ws, cnt, o);
 }
 
 template <bool SSSP, int STEPS, class WB, class WS, class FO>

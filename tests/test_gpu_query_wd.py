@@ -162,3 +162,37 @@ def test_sssp_distance_threshold_on_a_grid():
             assert rc == lb.LB_OK and np.array_equal(d, oracle.dijkstra(g, 450 * 1100 + 7)[0])
     finally:
         G.close()
+
+
+@pytest.mark.parametrize("off", ["line-1", "line", "line+255", "rounds"])
+def test_lists_walked_in_claimed_slices(off):
+    # one CTA per SM: lists of 16 grains of 256 edges per warp and more are
+    # claimed in slices; level 1 has exactly E list edges, over ragged entries
+    import torch
+    warps = 8 * torch.cuda.get_device_properties(0).multi_processor_count
+    line = 16 * 256 * warps
+    E = {"line-1": line - 1, "line": line, "line+255": line + 255, "rounds": 2 * line + line // 3 + 77}[off]
+    r = np.random.default_rng(len(off))
+    leaves = 200000
+    deg = []
+    while sum(deg) < E:
+        deg.append(int(min(r.choice([1, 2, 31, 33, 255, 257, 5000, 150000]), E - sum(deg))))
+    deg = np.array(deg)
+    H = deg.size
+    first = np.repeat(np.cumsum(deg) - deg, deg)
+    dst = 1 + H + (np.repeat(r.integers(0, leaves, H), deg) + np.arange(E) - first) % leaves
+    src = np.repeat(1 + np.arange(H), deg)
+    g = gg.from_edges(1 + H + leaves, np.concatenate([np.zeros(H, int), src]), np.concatenate([1 + np.arange(H), dst]),
+                      1 + r.integers(0, 200, H + E))
+    G = lb.Graph.from_csr(g)
+    ref, ov = oracle.dijkstra(g, 0)
+    lev = oracle.bfs(g, 0)[0]
+    try:
+        for tile in (256, 512, 8192, 32768):
+            G.set_options(ctas_per_sm=1, wd_tile=tile)
+            assert np.array_equal(G.bfs(0, "WD"), lev), tile
+            assert list(G.trace()["edges"][:2]) == [H, E]
+            d, rc = G.sssp(0, "WD")
+            assert not ov and rc == lb.LB_OK and np.array_equal(d, ref), tile
+    finally:
+        G.close()
