@@ -96,7 +96,8 @@ typedef struct lb_options {
                               and more) in slices that warps claim, of at
                               most this many edges (BFS) or half (SSSP) */
     int32_t ctas_per_sm;   /* CTAs per SM the fixed relax grid is sized for;
-                              0 = the occupancy limit */
+                              0 = the occupancy limit (WD BFS device loop: 4
+                              up to 2^23 edges, 3 up to 2^21) */
     int32_t hp_mode;       /* HP form: 0 = the paper's sub-iterations (Sec.
                               III-C: every node relaxes at most MDT edges per
                               sub-iteration, unfinished nodes form the next

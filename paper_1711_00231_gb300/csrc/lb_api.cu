@@ -477,11 +477,19 @@ int step_grid(lb_graph *g, int s, bool sssp) {
 }
 
 // Grid of the whole-query WD launch: every CTA resident (a cooperative
-// launch), at most ctas_per_sm per SM.
+// launch), at most ctas_per_sm per SM.  BFS on a small graph is launches,
+// barriers and list ends more than edges, and these get cheaper with fewer
+// CTAs: 5 / 4 / 3 per SM took, at 64K edges (R-MAT scale 12) 48.2 / 46.7 /
+// 46.7 us, 400K (Erdos-Renyi) 94.8 / 89.5 / 87.7, 2M (R-MAT 17) 73.2 / 72.0 /
+// 69.3, 2M (Erdos-Renyi) 132 / 127 / 130, 4M (R-MAT 18) 90.6 / 85.3 / 82.7, 4M
+// (Erdos-Renyi) 164 / 164 / 171, 8M 125 / 125 / 128, 16M (R-MAT 20) 134 / 137 /
+// 156 us.  SSSP (4 per SM) gained nothing from 3.
 int query_grid(lb_graph *g, bool sssp) {
     int &gr = g->query_grid[sssp ? 1 : 0];
     if (gr == 0) {
         int occ = query_wd_blocks_per_sm(sssp);
+        const int want = sssp || g->m > (1 << 23) ? occ : g->m > (1 << 21) ? 4 : 3;
+        if (g->opt.ctas_per_sm == 0 && want < occ) occ = want;
         if (g->opt.ctas_per_sm > 0 && g->opt.ctas_per_sm < occ) occ = g->opt.ctas_per_sm;
         gr = occ * g->sms;
     }
