@@ -555,8 +555,11 @@ lb_status status_from_error(uint32_t e) {
     return LB_OK;
 }
 
+// One launch runs the whole query (WD, device loop).
+bool whole_query(const lb_graph *g, int s) { return g->opt.loop_mode == 0 && (s == LB_WD || s == LB_AUTO); }
+
 lb_status run_query(lb_graph *g, int kind, int s, int32_t src, void *out_dev, int32_t *parents_dev,
-                    cudaStream_t st) {
+                    cudaStream_t st, uint32_t *prev_error = nullptr) {
     if (!g) return fail(LB_ERR_ARG, "graph is NULL");
     if (src < 0 || (int64_t)src >= g->n) return fail(LB_ERR_ARG, "source %d out of range [0, %lld)", src, (long long)g->n);
     if (s == LB_AUTO) s = LB_WD;
@@ -568,16 +571,18 @@ lb_status run_query(lb_graph *g, int kind, int s, int32_t src, void *out_dev, in
     const bool sssp = kind == LB_KIND_SSSP;
     LB_TRY(ensure_workspace(g, s));
     if (g->has_last && g->last_stream != st) LB_CU(cudaStreamWaitEvent(st, g->ev_done, 0));
-    // workspace set-up ran on g->stream
-    LB_CU(cudaEventRecord(g->ev_done, g->stream));
-    LB_CU(cudaStreamWaitEvent(st, g->ev_done, 0));
+    if (st != g->stream) {  // workspace set-up ran on g->stream
+        LB_CU(cudaEventRecord(g->ev_done, g->stream));
+        LB_CU(cudaStreamWaitEvent(st, g->ev_done, 0));
+    }
     StepParams p = make_params(g, s);
     const uint32_t max_levels = (uint32_t)(g->n + 1 < 0xFFFFFFF0ll ? g->n + 1 : 0xFFFFFFF0ll);
     const uint64_t max_steps = (uint64_t)1 << 40;
     const uint64_t time_limit_ns = (uint64_t)120 * 1000000000ull;  // safety net; no query comes close
-    const int grid = g->opt.loop_mode == 0 && s == LB_WD ? query_grid(g, sssp) : step_grid(g, s, sssp);
+    const bool whole = whole_query(g, s);
+    const int grid = whole ? query_grid(g, sssp) : step_grid(g, s, sssp);
     LB_CU(cudaEventRecord(g->ev_start, st));
-    if (g->opt.loop_mode == 0 && s == LB_WD) {
+    if (whole) {
         QueryArgs a;
         a.status = (uint32_t *)out_dev;
         a.src = src;
@@ -588,6 +593,7 @@ lb_status run_query(lb_graph *g, int kind, int s, int32_t src, void *out_dev, in
         a.number = g->query_number;
         a.seg_cap = fast_seg_cap(g->n);
         a.far_shift = far_shift(g->n);
+        a.prev_error = prev_error;
         a.team = kFastTeam < grid ? kFastTeam : grid;
         a.fast_seg = a.team == kFastTeam ? (int4 *)(((uintptr_t)g->fast_seg + 15u) & ~(uintptr_t)15u) : nullptr;
         LB_CU(launch_query_wd(sssp, p, a, grid, st));
@@ -649,8 +655,9 @@ lb_status host_query(lb_graph *g, int kind, lb_strategy s, int32_t src, void *ho
 // k host-output queries with the copy of query i's result overlapping query
 // i + 1: results alternate between two device buffers; query i's copy runs
 // on copy_stream after query i (ev_comp), and query i + 2, which reuses the
-// buffer, waits for that copy (ev_copy).  Each query's error word is copied
-// beside it on the device and read once at the end.  Every copy has
+// buffer, waits for that copy (ev_copy).  Each query's error word is kept
+// on the device (by the next query's set-up where one launch runs a query,
+// else and for the last query by a copy) and read once at the end.  Every copy has
 // finished before the call returns, on success or error.
 lb_status host_query_batch(lb_graph *g, int kind, lb_strategy s, const int32_t *srcs, int64_t k, void *host_out) {
     if (!g) return fail(LB_ERR_ARG, "graph is NULL");
@@ -685,9 +692,10 @@ lb_status host_query_batch(lb_graph *g, int kind, lb_strategy s, const int32_t *
         const int b = (int)(i & 1);
         if (i >= 2) e = cudaStreamWaitEvent(g->stream, g->ev_copy[b], 0);
         if (e != cudaSuccess) break;
-        st = run_query(g, kind, s, srcs[i], buf[b], nullptr, g->stream);
+        st = run_query(g, kind, s, srcs[i], buf[b], nullptr, g->stream, i > 0 ? g->batch_err + i - 1 : nullptr);
         if (st != LB_OK) break;
-        e = cudaMemcpyAsync(g->batch_err + i, &g->ctl->error, sizeof(uint32_t), cudaMemcpyDeviceToDevice, g->stream);
+        if (!whole_query(g, s) || i == k - 1)
+            e = cudaMemcpyAsync(g->batch_err + i, &g->ctl->error, sizeof(uint32_t), cudaMemcpyDeviceToDevice, g->stream);
         if (e == cudaSuccess) e = cudaEventRecord(g->ev_comp[b], g->stream);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(g->copy_stream, g->ev_comp[b], 0);
         if (e == cudaSuccess)

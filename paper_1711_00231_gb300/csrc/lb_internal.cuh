@@ -264,6 +264,7 @@ struct QueryArgs {
     int4 *fast_seg;     // 2 * kFastTeam * seg_cap entries (NULL: no fast levels)
     int32_t seg_cap;    // entries per CTA segment, at most kFastSeg
     int32_t far_shift;  // SSSP: blocks of 2^far_shift vertices in Ctl::far_bits
+    uint32_t *prev_error;  // receives the previous query's error word (NULL: no one asks)
 };
 cudaError_t launch_query_wd(bool sssp, const StepParams &p, const QueryArgs &a, int grid, cudaStream_t st);
 int query_wd_blocks_per_sm(bool sssp);

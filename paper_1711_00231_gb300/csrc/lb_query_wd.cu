@@ -870,6 +870,7 @@ __global__ void __launch_bounds__(kBlock, SSSP ? LB_QUERY_MIN_BLOCKS_SSSP : LB_Q
                 ctl->status = status;
                 ctl->src = src;
                 ctl->kind = SSSP ? 1 : 0;
+                if (a.prev_error) *a.prev_error = ctl->error;
                 ctl->error = 0;
                 ctl->t_start = q.t0;
             }
