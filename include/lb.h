@@ -102,13 +102,13 @@ typedef struct lb_options {
                               III-C: every node relaxes at most MDT edges per
                               sub-iteration, unfinished nodes form the next
                               sub-list); 1 = one step per super-iteration
-                              with the list's nodes binned by degree into
-                              sub-worklists served by a thread (<= min(MDT,
-                              thread_max) edges), a warp (<= hp_warp_max) or
-                              the whole CTA (more) (0) */
-    int32_t hp_warp_max;   /* binned forms (hp_mode 1, ns_mode 1): largest
-                              entry a warp serves; larger entries go to the
-                              CTA bin (4096) */
+                              that relaxes every edge of the list's nodes.
+                              In both a node's edges of the step are served by
+                              a thread (<= min(MDT, thread_max) edges), a warp
+                              (<= hp_warp_max) or the whole CTA (more) (0) */
+    int32_t hp_warp_max;   /* binned forms (HP, ns_mode 1): largest entry a
+                              warp serves; larger entries go to the CTA bin
+                              (4096) */
     int32_t ns_mode;       /* NS form: 0 = the paper's thread per granule
                               (Sec. III-B: a split node's ceil(d/MDT) runs of
                               at most MDT edges, one thread each); 1 = the
@@ -133,8 +133,9 @@ typedef struct lb_options {
                               of such levels.  0..16777216; 0 = off (a graph
                               starts with 16384) */
     int32_t test_barrier_skip; /* test hook, 0 in normal use: 1 makes CTA 1 of
-                              a WD query leave before its first grid barrier, so the other CTAs' bounded waits
-                              run out (2 s) and the query returns
+                              a WD query leave before its first grid
+                              barrier, so the other CTAs' bounded waits run
+                              out (2 s) and the query returns
                               LB_ERR_TIMEOUT with the device still usable */
     int32_t bitmap_place;  /* 0..7 (0): where the visited / queued bitmap
                               starts inside its allocation, in steps of
@@ -168,7 +169,8 @@ typedef struct lb_mem_stats {
     int64_t edge_lists;    /* EP: edge worklists (two buffers of m ids) */
     int64_t sub_lists;     /* HP: sub-worklists (two buffers) */
     int64_t control;       /* counters, step trace; WD: list segments of the
-                              small-list team (2 MiB) */
+                              small-list team (4 MiB; 512 KiB up to 32768
+                              vertices) */
     int64_t extra_total;   /* sum of the fields from status to control */
     int64_t base_total;    /* csr_offsets + csr_cols + csr_weights */
     int64_t resident;      /* bytes this graph holds on the device now */
@@ -464,7 +466,7 @@ lb_status lb_server_stop(lb_server *s);
  * device before the traversal (offsets[0] = 0, non-decreasing, offsets[n] =
  * m, every column in [0, n)); a malformed one returns LB_ERR_ARG and
  * nothing else runs.  All other memory comes from one fixed array of device
- * memory inside the library (about 3.6 MiB; every GPU that loads the
+ * memory inside the library (about 3.7 MiB; every GPU that loads the
  * library holds it until the process exits), so the call allocates
  * nothing.  Limits: n <= 131072
  * and m <= 16777216; larger sizes return LB_ERR_ARG.  The first call on a

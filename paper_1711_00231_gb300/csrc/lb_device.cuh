@@ -969,13 +969,4 @@ __device__ __forceinline__ int64_t iteration_tile(int64_t E, int64_t grid, int64
     return q * kTileGrain;
 }
 
-// Largest k in [lo, hi) with scan[k] <= e (read-only list, L1-cached).
-__device__ __forceinline__ int64_t list_search(const int32_t *__restrict__ scan, int64_t lo, int64_t hi, int64_t e) {
-    while (hi - lo > 1) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (__ldg(scan + mid) <= e) lo = mid; else hi = mid;
-    }
-    return lo;
-}
-
 }  // namespace lbk

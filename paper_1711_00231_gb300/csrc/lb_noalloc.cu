@@ -10,7 +10,7 @@
 // state) in one fixed-size array of device memory declared in this file.
 // Each GPU that loads the library holds that array until the process exits.
 //
-// Limits: n <= 131072 vertices and m <= 16777216 edges (about 3.6 MiB of
+// Limits: n <= 131072 vertices and m <= 16777216 edges (about 3.7 MiB of
 // scratch).  Every call on a device shares the array and finds the previous
 // call's contents in it; the kernels reset what must start at zero (loop
 // counters, the visited bitmap, the validation word and the output levels).

@@ -259,36 +259,6 @@ __device__ __forceinline__ void st_release_sys(unsigned long long *p, unsigned l
     asm volatile("st.release.sys.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-__device__ __forceinline__ int64_t list_search_cg(const int32_t *scan, int64_t lo, int64_t hi, int64_t e) {
-    while (hi - lo > 1) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (__ldcg(scan + mid) <= e) lo = mid; else hi = mid;
-    }
-    return lo;
-}
-
-__device__ __forceinline__ bool bfs_claim_cg(uint32_t *bitmap, uint32_t *status, int32_t v, uint32_t newlev) {
-    const uint32_t word = (uint32_t)v >> 5, bit = 1u << ((uint32_t)v & 31u);
-    if (__ldcg(bitmap + word) & bit) return false;
-    if (atomicOr(&bitmap[word], bit) & bit) return false;
-    status[v] = newlev;
-    return true;
-}
-
-__device__ __forceinline__ bool sssp_relax_cg(uint32_t *status, uint32_t *q, int32_t v, uint32_t du, uint32_t w,
-                                              uint32_t *err) {
-    if (du == kInf) return false;
-    const uint64_t a64 = (uint64_t)du + (uint64_t)w;
-    const uint32_t alt = a64 >= kSat ? kSat : (uint32_t)a64;
-    if (alt >= __ldcg(status + v)) return false;
-    const uint32_t old = atomicMin(&status[v], alt);
-    if (alt >= old) return false;
-    if (alt == kSat) atomicOr(err, kErrSaturated);
-    if (is_queued<kLdCg>(q, v)) return false;
-    const uint32_t bit = 1u << ((uint32_t)v & 31u);
-    return !(atomicOr(&q[(uint32_t)v >> 5], bit) & bit);
-}
-
 // Dynamic slot fields change between jobs and are written by other SMs, so
 // they are read through a volatile view (no L1); the pointer fields are
 // fixed at server creation.
@@ -401,13 +371,34 @@ __device__ int end_query(const Params &P, Slot *S, const GraphDev &g, int32_t ki
 #ifndef LB_SERVE_FAR_EDGES
 #define LB_SERVE_FAR_EDGES 4096
 #endif
-constexpr uint64_t kServeFarEdges = LB_SERVE_FAR_EDGES, kServeFarEarly = 16384;
+#ifndef LB_SERVE_FAR_MAX
+#define LB_SERVE_FAR_MAX 32768
+#endif
+constexpr uint64_t kServeFarEdges = LB_SERVE_FAR_EDGES, kServeFarMax = LB_SERVE_FAR_MAX;
+// List edges an interval should have per read of 32 distances in the pull
+// that starts it: a long front has a far set of many blocks, which this CTA
+// reads alone, so intervals widen until their lists outweigh the pull, past
+// this CTA's list limit too.  Lone SSSP on a 512 / 1024 / 2048 / 4096 squared grid:
+// without this rule 11.1 / 33.7 / 182 / 1731 ms; 8: 11.3 / 32 / 148 / 598; 32:
+// 11.2 / 31.5 / 93 / 276; 64: 11.2 / 31.5 / 93 / 274; 128: 12.1 / 32 / 83 / 223 ms
+// (without a threshold 19 / 88 / 328 / 1041 ms).
+#ifndef LB_PULL_EDGES
+#define LB_PULL_EDGES 64
+#endif
+// Only for graphs of more than this many words of block bits: among many
+// queries on smaller ones a single CTA's iterations cost less than jobs (128
+// mixed queries over 12 graphs of up to 2^18 vertices: 13.4 ms, with the rule
+// 15.1 ms).
+#ifndef LB_PULL_WORDS
+#define LB_PULL_WORDS 1024
+#endif
+constexpr unsigned long long kPullEdges = LB_PULL_EDGES;
+constexpr int64_t kPullWords = LB_PULL_WORDS;
 __device__ void far_account(Slot *S, const GraphDev &g, uint32_t level, uint64_t E) {
     volatile Slot *V = S;
     V->int_lists = V->int_lists + 1u;
     V->int_edges = V->int_edges + E;
-    if (V->far_engaged || E < kServeFarEdges) return;
-    if (!(level >= 32u || (level >= 6u && E >= kServeFarEarly && V->relaxed < (unsigned long long)g.m / 4u))) return;
+    if (V->far_engaged || level < 32u || E < kServeFarEdges || E > kServeFarMax) return;
     // first width: 32 * mean weight (of 64 evenly spaced edges) / mean degree
     unsigned long long w = 0;
 #pragma unroll 16
@@ -678,7 +669,7 @@ struct SoloState {
     uint32_t out_n, out_e, out_maxdeg, fmin, leave;
     FarSet far;
     // the slot's threshold fields, kept here meanwhile
-    uint32_t engaged, delta, int_lists;
+    uint32_t engaged, delta, int_lists, reads;
     unsigned long long int_edges;
 };
 
@@ -723,6 +714,7 @@ __device__ __noinline__ int solo_levels(const Params &P, Slot *S, SoloState &q, 
         q.out_n = q.out_e = q.out_maxdeg = 0u;
         q.leave = 0u;
         q.fmin = kInf;
+        q.reads = 0u;
         if (SSSP) {
             const volatile Slot *V = S;
             q.far = FarSet{V->far_T, far_shift(g.n), (uint32_t *)(st.ws + W.far)};
@@ -788,17 +780,21 @@ __device__ __noinline__ int solo_levels(const Params &P, Slot *S, SoloState &q, 
         if (SSSP && pull) {
             // the next interval [T, from + delta), its width by the lists of the last one
             const uint32_t T0 = T, T1 = far_add(from, q.delta);
-            uint32_t mn = kInf;
+            uint32_t mn = kInf, reads = 0;  // reads: this warp's reads of 32 distances
             far_blocks(
                 status, g.n, q.far, 0u, 1u, true,
                 [&](int32_t v, uint32_t d) { solo_push(out, W.cap, q, d >= T0 && d < T1, v, 0, 0); },
                 [&](uint32_t d) {
                     const bool k = d != kInf && d >= T1;
                     if (k) mn = min(mn, d);
+                    ++reads;
                     return k;
                 });
             mn = __reduce_min_sync(kFull, mn);
-            if (lane_id() == 0 && mn != kInf) atomicMin(&q.fmin, mn);
+            if (lane_id() == 0) {
+                if (mn != kInf) atomicMin(&q.fmin, mn);
+                atomicAdd(&q.reads, reads);
+            }
             __syncthreads();
             // the pulled vertices' edges, all at once (none: an entry without effect)
             const uint32_t pulled = q.out_n;
@@ -825,9 +821,15 @@ __device__ __noinline__ int solo_levels(const Params &P, Slot *S, SoloState &q, 
                 q.fmin = kInf;
                 if (q.int_lists > 0u) {
                     const unsigned long long avg = q.int_edges / q.int_lists;
-                    if (avg < kSoloEdges / 8u && q.delta < kFarMaxDelta) q.delta *= 2u;
-                    if (avg > kSoloEdges / 2u) q.delta = max(q.delta / 2u, 1u);
+                    const bool wide = (((g.n - 1) >> q.far.shift) >> 5) >= kPullWords;
+                    const unsigned long long least = wide ? kPullEdges * q.reads : 0ull;
+                    if (q.int_edges < least || avg < kSoloEdges / 8u) {
+                        if (q.delta < kFarMaxDelta) q.delta *= 2u;
+                    } else if (avg > kSoloEdges / 2u && q.int_edges > 4u * least) {
+                        q.delta = max(q.delta / 2u, 1u);
+                    }
                 }
+                q.reads = 0u;
                 q.int_lists = 0u;
                 q.int_edges = 0ull;
             }

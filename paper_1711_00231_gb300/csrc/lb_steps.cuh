@@ -3,7 +3,8 @@
 // Every kernel runs on a fixed, persistent-style grid (a multiple of the SM
 // count) and reads the sizes of its input list from the device control
 // block, so the same launch can be captured once into a CUDA graph and
-// replayed by a conditional WHILE node until the worklist is empty.
+// replayed by a conditional WHILE node until the worklist is empty (WD's
+// device loop is one launch of its own: lb_query_wd.cu).
 #pragma once
 
 #include <type_traits>

@@ -65,3 +65,23 @@ def test_solo_levels_match_oracle(launch_ms):
         S.close()
         for g in G:
             g.close()
+
+
+@pytest.mark.parametrize("launch_ms", [0, 3])
+def test_wide_fronts_match_oracle(launch_ms):
+    # fronts of over a thousand vertices: the pulls cost more than the lists,
+    # so intervals widen until their lists pass what one CTA takes
+    import torch
+    g = gg.grid(1500, 1400, seed=8)
+    G = lb.Graph.from_csr(g)
+    S = sv.Server([G], slots=4, mem_fraction=0.05, launch_ms=launch_ms)
+    try:
+        src = [0, g.n // 2 + 700]
+        outs = [torch.empty(g.n, dtype=torch.int32, device="cuda") for _ in src]
+        status = S.run_batch([sv.Request(0.0, 0, s, "sssp") for s in src], outs, timeout_s=120.0)
+        torch.cuda.synchronize()
+        for s, o, st in zip(src, outs, status):
+            assert st == lb.LB_OK and np.array_equal(o.cpu().numpy().view(np.uint32), oracle.dijkstra(g, s)[0]), s
+    finally:
+        S.close()
+        G.close()
