@@ -56,7 +56,7 @@ def parse():
     ap.add_argument("--no-cpu", action="store_true")
     ap.add_argument("--cpu-seconds", type=float, default=20.0)
     ap.add_argument("--loop-mode", type=int, default=0,
-                    help="0: device-resident loop (CUDA graph WHILE); 1: host loop (for per-kernel profiling)")
+                    help="0: device-resident loop; 1: host loop (for per-kernel profiling)")
     ap.add_argument("--kinds", default="bfs,sssp")
     ap.add_argument("--wd-tile", type=int, default=0, help="largest WD tile in list edges (0 = library default)")
     ap.add_argument("--hp-mode", type=int, default=0, help="HP form: 0 sub-iterations, 1 degree-binned")
@@ -641,7 +641,7 @@ def main():
                 "traffic_note": "captured at R-MAT scale 22 only (profiles/k_step_wd_traffic_rmat22_ef32.md: BFS "
                                 "0.65x, SSSP 1.72x the algorithmic bytes per query); not scaled, since at scale 24 "
                                 "the distance array no longer fits in L2 and traffic does not grow in proportion",
-                "kernel": f"k_step_wd ({kind})", "peak_source": f"{peak_kind} hbm_gbs",
+                "kernel": f"{'k_step_wd' if args.loop_mode else 'k_query_wd'} ({kind})", "peak_source": f"{peak_kind} hbm_gbs",
                 "unit_of_work": "one query (all its relax launches + set-up); algorithmic bytes per query "
                                 f"= {BYTES[kind][0]} B x m_reached + {BYTES[kind][1]} B x n_reached"}
     roofline = roof(dom)
@@ -764,7 +764,7 @@ def main():
                 "scaling": "weak", "vs_baseline": None, "dtype": "uint32", "data": "synthetic",
                 "config": dict(WORKLOAD, strategy=strat, parallelism=f"replicas{world}", n=g.n, m=g.m,
                                scale=args.scale, edge_factor=args.edge_factor, sources=len(srcs), kinds=list(kinds),
-                               loop="device (CUDA graph WHILE)" if args.loop_mode == 0 else "host",
+                               loop="device (WD: one cooperative launch per query)" if args.loop_mode == 0 else "host",
                                options=run_opts, autotune=tune),
                 "roofline": roofline, "roofline_by_kind": roofline_by_kind, "cpu_baseline": cpu, "e2e": e2e,
                 "clocks": clocks,

@@ -365,9 +365,11 @@ __device__ int end_query(const Params &P, Slot *S, const GraphDev &g, int32_t ki
 }
 
 // SSSP, after a list of E edges in iteration `level` (single thread): the
-// interval's books, and the distance threshold once lists get long, by the
-// rule of the whole-query kernel with the sizes of a single CTA's levels
-// (long lists go to many CTAs at 15-25 us per iteration).
+// interval's books, and the distance threshold once lists get long after
+// many iterations (a grid's).  A list past kServeFarMax by then belongs to a
+// graph whose far set one CTA should not pull: random graphs that took the
+// whole-query kernel's rule got slower (Erdos-Renyi, 1M vertices, 8M edges:
+// 2.4 -> 4.2 ms).
 #ifndef LB_SERVE_FAR_EDGES
 #define LB_SERVE_FAR_EDGES 4096
 #endif
