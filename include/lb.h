@@ -136,7 +136,10 @@ typedef struct lb_options {
                               a WD query leave before its first grid
                               barrier, so the other CTAs' bounded waits run
                               out (2 s) and the query returns
-                              LB_ERR_TIMEOUT with the device still usable */
+                              LB_ERR_TIMEOUT with the device still usable.
+                              Device loop: 2 makes the CTAs outside the
+                              small-list team 200 us late in reading what a
+                              grid barrier published */
     int32_t bitmap_place;  /* 0..7 (0): where the visited / queued bitmap
                               starts inside its allocation, in steps of
                               min(1 MiB, one bitmap half rounded up to 4

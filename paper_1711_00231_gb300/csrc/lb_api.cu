@@ -240,7 +240,7 @@ lb_status normalise_options(const lb_options *in, lb_options *out) {
     if (o.thread_max < 1 || o.thread_max > 1024) return fail(LB_ERR_ARG, "thread_max must be in [1, 1024]");
     if (o.hp_depth < 1 || o.hp_depth > 8) return fail(LB_ERR_ARG, "hp_depth must be in [1, 8]");
     if (o.small_edges < 0 || o.small_edges > (1 << 24)) return fail(LB_ERR_ARG, "small_edges must be in [0, 2^24]");
-    if (o.test_barrier_skip != 0 && o.test_barrier_skip != 1) return fail(LB_ERR_ARG, "test_barrier_skip must be 0 or 1");
+    if (o.test_barrier_skip < 0 || o.test_barrier_skip > kTestMax) return fail(LB_ERR_ARG, "test_barrier_skip must be 0..%d", kTestMax);
     if (o.bitmap_place < 0 || o.bitmap_place >= kBitmapPlaces) return fail(LB_ERR_ARG, "bitmap_place must be in [0, 7]");
     for (int i = 0; i < 2; ++i)
         if (o.reserved[i] != 0) return fail(LB_ERR_ARG, "reserved option fields must be 0");

@@ -22,6 +22,7 @@ struct QueryState {
     FarSet far;  // far.T == u.T
     uint32_t ok, rank;            // rank: this CTA in the team (kNoRank: outside); 0 leads
     uint32_t full, team, resume;  // barriers and publications so far
+    uint32_t grid_steps, team_steps;  // regular steps of the whole grid / of the team so far
     uint32_t fmin;                // a pull's smallest distance left
     uint32_t maxdeg;              // largest degree this CTA listed in the level
     uint32_t trace;               // leader: records written

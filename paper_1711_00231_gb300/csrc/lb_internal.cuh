@@ -87,6 +87,13 @@ struct TraceRec {
 constexpr int kFastTeam = LB_FAST_TEAM;  // CTAs of the small-list team (a multiple of 32)
 constexpr int kFastSeg = LB_FAST_SEG;    // entries per CTA segment of a fast level's list (two buffers)
 
+// lb_options.test_barrier_skip
+enum : int32_t {
+    kTestSkip = 1,       // CTA 1 leaves before its first grid barrier
+    kTestLateReads = 2,  // CTAs outside the team are slow to read a step's counters after its barrier
+    kTestMax = 2,
+};
+
 constexpr uint32_t kMaxSms = 512;
 constexpr uint32_t kNoRank = 0xFFFFFFFFu;
 
@@ -114,14 +121,19 @@ struct QuerySync {
     alignas(128) uint32_t resume;       // publications of `loop` (kResumeAbort: a wait ran out)
     alignas(128) QueryLoop loop;
     uint32_t delta0;                    // SSSP: first interval width
-    struct alignas(128) Pack {
-        unsigned long long v;  // (entries << 32) | edges; bit 63: the time limit has passed
-        uint32_t far_min;      // pull step: smallest distance left in the far set
-        uint32_t maxdeg;       // largest degree listed
-    } pack[3];  // step L counts its output in pack[L % 3]
-    struct alignas(128) Claim {
-        uint32_t next;  // slices of a long list claimed so far
-    } claim[3];         // step L claims from claim[L % 3]
+    // Counters of a step.  The steps of the whole grid and those of the team
+    // have three sets each, used in turn, all zero at first: the n-th step
+    // of its kind counts in set n % 3 and clears set (n + 1) % 3, which was
+    // last read after the barrier that ended step n - 2.  Every reader has
+    // since arrived at the barrier of step n - 1.  (A set shared by both kinds
+    // would be cleared by the team while CTAs outside it, which only wait
+    // at barriers of the whole grid, may still have to read it.)
+    struct Step {
+        alignas(128) unsigned long long v;  // (entries << 32) | edges; bit 63: the time limit has passed
+        uint32_t far_left;                  // pull step: largest ~d of the distances d left in the far set
+        uint32_t maxdeg;                    // largest degree listed
+        alignas(128) uint32_t next;         // slices of a long list claimed so far
+    } grid_step[3], team_step[3];
     alignas(128) unsigned long long fast_pack[2];  // fast levels: list counter of the way back
     alignas(128) uint32_t team_here;  // team ranks taken
     uint32_t sm_ctas[kMaxSms];        // CTAs per SM
@@ -237,7 +249,7 @@ struct StepParams {
     int32_t ns_mode;       // 0: thread per granule, 1: binned granules
     int32_t hp_depth;      // HP: lists of a super-iteration's chain with their own MDT
     int32_t hist_bins;     // HistogramBinCount of the MDT heuristic
-    int32_t test_barrier_skip;  // test hook: CTA 1 of the small-list launch skips its first barrier
+    int32_t test_barrier_skip;  // test hook (kTest...)
     int32_t strategy;
     int32_t use_cond;
     int32_t small_edges;   // WD: lists of at most this many edges run on a small-list team of CTAs (0: off)

@@ -263,6 +263,11 @@ cudaError_t launch_team_pick(Ctl *ctl, int sms, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+// The counters of this step (ahead 0) or of the next one of its kind (1).
+__device__ __forceinline__ QuerySync::Step *step_counters(QuerySync *sync, const QueryState &q, bool team, uint32_t ahead) {
+    return team ? sync->team_step + (q.team_steps + ahead) % 3u : sync->grid_step + (q.grid_steps + ahead) % 3u;
+}
+
 // The leader's thread 0: the state the CTAs outside the team go on from.
 __device__ __forceinline__ void publish(QuerySync *sync, QueryState &q) {
     sync->loop = q.u;
@@ -472,14 +477,6 @@ __device__ __forceinline__ bool fast_levels(const StepParams &p, const QueryArgs
             fast_push(mine, a.seg_cap, q, i < n && deg > 0, v, beg, deg);
         }
         if (!fast_exchange(ctl, q)) return false;
-        // every CTA has read the output counters of the levels before
-        if (rank == 0 && tid == 0)
-            for (int k = 0; k < 3; ++k) {
-                sync->pack[k].v = 0ull;
-                sync->pack[k].far_min = kInf;
-                sync->pack[k].maxdeg = 0u;
-                sync->claim[k].next = 0u;
-            }
         if (tid == 0) ++q.fast_conv;
     }
     uint32_t buf = 0, err = 0;
@@ -646,13 +643,13 @@ __device__ __forceinline__ bool fast_levels(const StepParams &p, const QueryArgs
 // A pull step up to its barrier, out of line: its registers are not the
 // walk's.
 template <class WB>
-__device__ __noinline__ void pull_level(const StepParams &p, const QueryArgs &a, QuerySync *sync, QueryState &q,
+__device__ __noinline__ void pull_level(const StepParams &p, const QueryArgs &a, QuerySync::Step *step, QueryState &q,
                                         WB &wb, uint32_t me, uint32_t ctas) {
     NoScratch ns;
     FlushOutT<1> o;
     o.list = p.lists[q.u.par ^ 1u];
     o.elist = nullptr;
-    o.pack = &sync->pack[q.u.level % 3u].v;
+    o.pack = &step->v;
     o.cap = p.list_cap;
     o.tile_cap = p.tile_cap;
     o.tile = (int32_t)kTileGrain;
@@ -732,7 +729,7 @@ __device__ __forceinline__ void claimed_slice(uint32_t k, uint32_t share, uint32
 }
 
 template <bool SSSP, int ITEMS>
-__device__ __forceinline__ void regular_level(const StepParams &p, const QueryArgs &a, QuerySync *sync, QueryState &q,
+__device__ __forceinline__ void regular_level(const StepParams &p, const QueryArgs &a, QuerySync::Step *step, QueryState &q,
                                            WarpBufT<SSSP ? LB_KWB_WD_SSSP : LB_KWB_WD_BFS> &wb, uint32_t me,
                                            uint32_t ctas, bool team_mode) {
     Ctl *const ctl = p.ctl;
@@ -759,7 +756,7 @@ __device__ __forceinline__ void regular_level(const StepParams &p, const QueryAr
     FlushOutT<SSSP ? 3 : 2> o;
     o.list = p.lists[par ^ 1u];
     o.elist = nullptr;
-    o.pack = &sync->pack[level % 3u].v;
+    o.pack = &step->v;
     o.cap = p.list_cap;
     o.tile_cap = p.tile_cap;
     o.tile = (int32_t)kTileGrain;
@@ -782,7 +779,7 @@ __device__ __forceinline__ void regular_level(const StepParams &p, const QueryAr
     uint32_t w0 = (me * kWarps + warp) * len;
     while (w0 < E) {  // warp-uniform
         uint32_t k = 0;  // the next slice, claimed ahead
-        if (claims && lane_id() == 0) k = atomicAdd(&sync->claim[level % 3u].next, 1u);
+        if (claims && lane_id() == 0) k = atomicAdd(&step->next, 1u);
         wd_walk_slice<SSSP, ITEMS, kLdPlain>(p.g, in, (int32_t)in_cnt, E, w0, min(w0 + len, E), p.bitmap, qcur, status,
                                              level, &ctl->error, wb, ns, cnt, o);
         if (claims) claimed_slice<SSSP>(warps + __shfl_sync(kFull, k, 0), share, (uint32_t)p.tile, warps, w0, len);
@@ -896,7 +893,7 @@ __global__ void __launch_bounds__(kBlock, SSSP ? LB_QUERY_MIN_BLOCKS_SSSP : LB_Q
             }
         }
         // test hook: a CTA that never arrives makes the others' waits run out
-        if (p.test_barrier_skip && blockIdx.x == 1) return;
+        if (p.test_barrier_skip == kTestSkip && blockIdx.x == 1) return;
         __syncthreads();
         if (threadIdx.x == 0) {
             q.full = 1;
@@ -950,32 +947,36 @@ __global__ void __launch_bounds__(kBlock, SSSP ? LB_QUERY_MIN_BLOCKS_SSSP : LB_Q
         const uint32_t level = q.u.level, par = q.u.par;
         const uint32_t in_cnt = q.u.cnt;
         const bool pull = SSSP && q.u.pull != 0u;
-        // the next level's output counter (its last reads were before the
-        // barrier that ended the previous level)
+        // the next step of this kind finds its counters cleared
         if (q.rank == 0u && threadIdx.x == 0) {
-            sync->pack[(level + 1u) % 3u].v = 0ull;
-            sync->pack[(level + 1u) % 3u].maxdeg = 0u;
-            sync->claim[(level + 1u) % 3u].next = 0u;
-            if (SSSP) sync->pack[(level + 1u) % 3u].far_min = kInf;
+            QuerySync::Step *const nx = step_counters(sync, q, team_mode, 1u);
+            nx->v = 0ull;
+            nx->far_left = 0u;
+            nx->maxdeg = 0u;
+            nx->next = 0u;
         }
-        if (SSSP && pull) pull_level(p, a, sync, q, s_wb[threadIdx.x >> 5], me, ctas);
-        else regular_level<SSSP, ITEMS>(p, a, sync, q, s_wb[threadIdx.x >> 5], me, ctas, team_mode);
+        if (SSSP && pull) pull_level(p, a, step_counters(sync, q, team_mode, 0u), q, s_wb[threadIdx.x >> 5], me, ctas);
+        else regular_level<SSSP, ITEMS>(p, a, step_counters(sync, q, team_mode, 0u), q, s_wb[threadIdx.x >> 5], me, ctas, team_mode);
         __syncthreads();
         if (threadIdx.x == 0) {
-            unsigned long long *const pk = &sync->pack[level % 3u].v;
+            QuerySync::Step *const step = step_counters(sync, q, team_mode, 0u);
             if (SSSP && pull && q.fmin != kInf) {
-                atomicMin(&sync->pack[level % 3u].far_min, q.fmin);
+                atomicMax(&step->far_left, ~q.fmin);
                 q.fmin = kInf;
             }
             if (q.maxdeg > 0u) {
-                atomicMax(&sync->pack[level % 3u].maxdeg, q.maxdeg);
+                atomicMax(&step->maxdeg, q.maxdeg);
                 q.maxdeg = 0u;
             }
-            if (q.rank == 0u && global_ns() > q.deadline) atomicOr(pk, 1ull << 63);
+            if (q.rank == 0u && global_ns() > q.deadline) atomicOr(&step->v, 1ull << 63);
             q.ok = (team_mode ? arrive_team(sync, ctas, ++q.team) : arrive_full(sync, ctas, ++q.full)) ? 1u : 0u;
-            const unsigned long long x = __ldcg(pk);
-            q.u.maxdeg = __ldcg(&sync->pack[level % 3u].maxdeg);
-            const uint32_t fmin = SSSP && pull ? __ldcg(&sync->pack[level % 3u].far_min) : 0u;
+            // test hook: the team is far ahead when these CTAs read
+            if (p.test_barrier_skip == kTestLateReads && q.rank == kNoRank)
+                for (const uint64_t t = global_ns(); global_ns() - t < 200000u;) __nanosleep(1000);
+            const unsigned long long x = __ldcg(&step->v);
+            q.u.maxdeg = __ldcg(&step->maxdeg);
+            const uint32_t fmin = SSSP && pull ? ~__ldcg(&step->far_left) : 0u;
+            ++(team_mode ? q.team_steps : q.grid_steps);
             uint32_t ncnt = (uint32_t)(x >> 32) & 0x7FFFFFFFu;
             uint32_t err = 0;
             if ((int64_t)ncnt > p.list_cap) {

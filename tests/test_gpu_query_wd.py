@@ -196,3 +196,57 @@ def test_lists_walked_in_claimed_slices(off):
             assert not ov and rc == lb.LB_OK and np.array_equal(d, ref), tile
     finally:
         G.close()
+
+
+def swinging(rounds, width, chain, arms):
+    """Lists that swing between the whole grid and the team: a hub's `width`
+    edges, as many one-edge entries, one entry, then `chain` vertices of `arms`
+    edges (too many for a fast level: regular levels of the team), the next hub."""
+    src, dst, at = [], [], 0
+    for _ in range(rounds):
+        leaves = at + 1 + np.arange(width)
+        end = at + 1 + width
+        src += [np.full(width, at), leaves]
+        dst += [leaves, np.full(width, end)]
+        at = end
+        for _ in range(chain):
+            src.append(np.full(arms, at))
+            dst.append(at + 1 + np.arange(arms))
+            at += arms
+        src.append(np.array([at]))
+        dst.append(np.array([at + 1]))
+        at += 1
+    src, dst = np.concatenate(src), np.concatenate(dst)
+    return gg.from_edges(at + 1, src, dst, 1 + (np.arange(src.size) * 31) % 500)
+
+
+@pytest.mark.parametrize("width", [40000, 70000])
+@pytest.mark.parametrize("chain", [0, 1, 2, 3, 4, 5])
+def test_late_reads_of_a_steps_counters(width, chain):
+    # CTAs outside the team read a step's counters when the team is levels
+    # ahead: nothing may have cleared them
+    g = swinging(12, width, chain, 50)
+    G = lb.Graph.from_csr(g)
+    try:
+        for opts in (dict(), dict(small_edges=100)):
+            G.set_options(test_barrier_skip=2, **opts)
+            check(G, g, 0)
+            modes = G.trace()["mode"]
+            assert (modes == 4).sum() >= 12 and (modes == 0).sum() >= 12
+    finally:
+        G.close()
+
+
+@pytest.mark.parametrize("kind", ["uniform", "gaps"])
+def test_late_reads_with_a_distance_threshold(kind):
+    g = far_graph(kind)
+    src = int(gg.pick_sources(g, 1, seed=3)[0])
+    ref, _ = oracle.dijkstra(g, src)
+    G = lb.Graph.from_csr(g)
+    try:
+        for opts in (dict(), dict(small_edges=2000)):
+            G.set_options(test_barrier_skip=2, **opts)
+            d, rc = G.sssp(src, "WD")
+            assert rc == lb.LB_OK and np.array_equal(d, ref)
+    finally:
+        G.close()
