@@ -870,6 +870,10 @@ __global__ void __launch_bounds__(kBlock, SSSP ? LB_QUERY_MIN_BLOCKS_SSSP : LB_Q
                 if (a.prev_error) *a.prev_error = ctl->error;
                 ctl->error = 0;
                 ctl->t_start = q.t0;
+                // what a query that ends at a wait's limit reports
+                ctl->level = ctl->trace_len = ctl->in_cnt = 0u;
+                ctl->step = ctl->in_edges = 0u;
+                ctl->relaxed = ctl->pushes = 0ull;
             }
         }
         if (blockIdx.x == 0) {

@@ -250,3 +250,22 @@ def test_late_reads_with_a_distance_threshold(kind):
             assert rc == lb.LB_OK and np.array_equal(d, ref)
     finally:
         G.close()
+
+
+def test_failed_query_reports_nothing_of_the_one_before():
+    g = gg.grid(40, 50, seed=1)
+    G = lb.Graph.from_csr(g)
+    try:
+        for kind, query in (("bfs", G.bfs), ("sssp", G.sssp)):
+            check(G, g, 7)
+            assert G.stats()["iterations"] > 0 and len(G.trace()) > 0
+            G.set_options(test_barrier_skip=1)
+            with pytest.raises(lb.LbError):
+                query(0, "WD")
+            st = G.stats()
+            assert st["status"] == lb.LB_ERR_TIMEOUT, kind
+            assert [st[k] for k in ("iterations", "steps", "edges_relaxed", "pushes")] == [0, 0, 0, 0], kind
+            assert len(G.trace()) == 0, kind
+            G.set_options(test_barrier_skip=0)
+    finally:
+        G.close()
