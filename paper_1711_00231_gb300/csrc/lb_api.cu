@@ -586,9 +586,7 @@ lb_status run_query(lb_graph *g, int kind, int s, int32_t src, void *out_dev, in
         QueryArgs a;
         a.status = (uint32_t *)out_dev;
         a.src = src;
-        // with a threshold (SSSP) an interval's iterations add up to at most
-        // its vertices and one more
-        a.max_levels = sssp && max_levels < 0x7FFFFFF0u ? 2u * max_levels + 64u : max_levels;
+        a.max_levels = sssp ? threshold_levels(g->n) : max_levels;
         a.time_limit_ns = time_limit_ns;
         a.number = g->query_number;
         a.seg_cap = fast_seg_cap(g->n);

@@ -20,6 +20,7 @@
 #include <stdint.h>
 
 #include "../../include/lb.h"
+#include "lb_rules.h"
 
 namespace lbk {
 

@@ -337,10 +337,9 @@ __device__ int32_t slot_status(const Slot *S) {
 // or the CTA goes on with the query by itself (solo_levels).
 enum : int { kAfterNone = 0, kAfterJob = 1, kAfterSolo = 2 };
 
-// Worklist iterations a query may take (with a threshold an interval's add
-// up to at most its vertices and one more).
+// Worklist iterations a query may take.
 __device__ __forceinline__ uint32_t level_cap(const GraphDev &g, int32_t kind) {
-    return kind == 1 && g.n < 0x7FFFFF00ll ? 2u * (uint32_t)g.n + 64u : (uint32_t)g.n;
+    return kind == 1 ? threshold_levels(g.n) : (uint32_t)g.n;
 }
 
 // A list the finishing CTA may go on with alone: few edges, short entries on

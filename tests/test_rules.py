@@ -1,0 +1,30 @@
+"""The query loops' arithmetic rules (csrc/lb_rules.h), compiled alone: no GPU."""
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1711_00231_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def call(tmp_path_factory):
+    """call(expression) -> its value, from a C++ program that includes the rules."""
+    d = tmp_path_factory.mktemp("rules")
+
+    def run(*exprs):
+        src = d / "rules.cpp"
+        body = "".join(f'  printf("%llu\\n", (unsigned long long)({e}));\n' for e in exprs)
+        src.write_text(f'#include <stdio.h>\n#include "lb_rules.h"\nusing namespace lbk;\nint main() {{\n{body}}}\n')
+        exe = d / "rules"
+        subprocess.check_call(["g++", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)])
+        return [int(x) for x in subprocess.check_output([str(exe)]).split()]
+
+    return run
+
+
+def test_iteration_cap_never_below_the_vertices(call):
+    # twice the vertices and some more, also where that passes 32 bits
+    ns = [1, 2, 1000, 1 << 30, (1 << 31) - 100, (1 << 31) - 33, (1 << 31) - 2, (1 << 31) - 1]
+    for n, k in zip(ns, call(*[f"threshold_levels({n}ll)" for n in ns])):
+        assert k == min(2 * n + 66, 0xFFFFFFF0) and k > n
