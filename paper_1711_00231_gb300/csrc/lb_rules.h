@@ -19,4 +19,13 @@ LB_HD inline uint32_t threshold_levels(int64_t n) {
     return k < 0xFFFFFFF0ull ? (uint32_t)k : 0xFFFFFFF0u;
 }
 
+// How a query goes on when the next iteration would be number `level`: it has
+// a list, or a pull of far vertices is due, or neither.  Work left at the cap
+// is an error, whichever kind it is.
+enum : int { kGoesOn = 0, kIsDone = 1, kIsCut = 2 };
+LB_HD inline int level_end(bool list, bool pull, uint32_t level, uint32_t cap) {
+    if (!list && !pull) return kIsDone;
+    return level <= cap ? kGoesOn : kIsCut;
+}
+
 }  // namespace lbk

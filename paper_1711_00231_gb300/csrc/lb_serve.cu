@@ -457,7 +457,8 @@ __device__ int finish_job(const Params &P, Slot *S, uint32_t kind) {
         const bool broken = (err & (kErrCapacity | kErrBounds)) != 0u;
         if (st.kind == 1) far_account(S, g, st.level, st.in_edges);
         const bool pull = st.kind == 1 && cnt == 0 && ((const volatile Slot *)S)->far_T != kInf;
-        if ((cnt > 0 || pull) && st.level + 1 <= level_cap(g, st.kind) && !broken) {
+        const int end = level_end(cnt > 0, pull, st.level + 1, level_cap(g, st.kind));
+        if (end == kGoesOn && !broken) {
             ws_list(st.ws, W, out).scan[cnt] = (int32_t)edges;
             S->par = out;
             S->in_cnt = (uint32_t)cnt;
@@ -468,7 +469,7 @@ __device__ int finish_job(const Params &P, Slot *S, uint32_t kind) {
             open_job(S, kJobRelax, (uint32_t)((edges + Tj - 1) / Tj), (uint32_t)(Tj / kTileGrain));
             return kAfterJob;
         }
-        if (cnt > 0 && !broken) atomicOr(&S->error, kErrIterCap);
+        if (end == kIsCut && !broken) atomicOr(&S->error, kErrIterCap);
         return end_query(P, S, g, st.kind);
     }
     complete_query(P, S, slot_status(S));  // kJobCheck
@@ -921,8 +922,8 @@ __device__ __noinline__ int solo_levels(const Params &P, Slot *S, SoloState &q, 
     }
     // leave: the query ends, or a regular list goes to the next job
     int after = kAfterNone;
-    const bool ends = (n == 0u && !(SSSP && T != kInf && from != kInf)) || level > level_cap(g, SSSP ? 1 : 0);
-    if (!ends && n > 0u) {
+    const int end = level_end(n > 0u, SSSP && T != kInf && from != kInf, level, level_cap(g, SSSP ? 1 : 0));
+    if (end == kGoesOn && n > 0u) {
         const NodeList in = ws_list(st.ws, W, b), out = ws_list(st.ws, W, b ^ 1u);
         FlushOut o;
         o.list = out;
@@ -965,8 +966,8 @@ __device__ __noinline__ int solo_levels(const Params &P, Slot *S, SoloState &q, 
             S->int_lists = q.int_lists;
             S->int_edges = q.int_edges;
         }
-        if (ends) {
-            if (n > 0u) atomicOr(&S->error, kErrIterCap);
+        if (end != kGoesOn) {
+            if (end == kIsCut) atomicOr(&S->error, kErrIterCap);
             s_after = end_query(P, S, g, SSSP ? 1 : 0);
         } else {
             // (an empty list with a threshold in force and the launch ending:

@@ -28,3 +28,11 @@ def test_iteration_cap_never_below_the_vertices(call):
     ns = [1, 2, 1000, 1 << 30, (1 << 31) - 100, (1 << 31) - 33, (1 << 31) - 2, (1 << 31) - 1]
     for n, k in zip(ns, call(*[f"threshold_levels({n}ll)" for n in ns])):
         assert k == min(2 * n + 66, 0xFFFFFFF0) and k > n
+
+
+def test_work_left_at_the_iteration_cap_is_an_error(call):
+    goes_on, done, cut = 0, 1, 2
+    cases = [((0, 0, 5, 10), done), ((0, 0, 11, 10), done), ((1, 0, 10, 10), goes_on), ((1, 0, 11, 10), cut),
+             ((0, 1, 10, 10), goes_on), ((0, 1, 11, 10), cut), ((1, 1, 11, 10), cut)]
+    got = call(*["level_end({}, {}, {}u, {}u)".format(*args) for args, _ in cases])
+    assert got == [want for _, want in cases]
