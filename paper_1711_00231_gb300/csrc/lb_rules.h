@@ -28,4 +28,7 @@ LB_HD inline int level_end(bool list, bool pull, uint32_t level, uint32_t cap) {
     return level <= cap ? kGoesOn : kIsCut;
 }
 
+// Iterations so far, after a list of `entries` entries.
+LB_HD inline uint32_t level_after(uint32_t level, uint32_t entries) { return level + (entries > 0u ? 1u : 0u); }
+
 }  // namespace lbk

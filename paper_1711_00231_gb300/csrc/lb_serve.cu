@@ -451,13 +451,15 @@ __device__ int finish_job(const Params &P, Slot *S, uint32_t kind) {
         const WsLayout W = ws_layout(g.n, g.m);
         if (cnt > W.cap) { atomicOr(&S->error, kErrCapacity); cnt = W.cap; }
         S->relaxed = ld_volatile(&S->relaxed) + st.in_edges;
-        S->level = st.level + 1;
+        // an empty list (solo_levels handed over before a pull) is no iteration
+        const uint32_t level = level_after(st.level, st.in_cnt);
+        S->level = level;
         const uint32_t out = st.par ^ 1u;
         const uint32_t err = atomicOr(&S->error, 0u);
         const bool broken = (err & (kErrCapacity | kErrBounds)) != 0u;
-        if (st.kind == 1) far_account(S, g, st.level, st.in_edges);
+        if (st.kind == 1 && st.in_cnt > 0) far_account(S, g, st.level, st.in_edges);
         const bool pull = st.kind == 1 && cnt == 0 && ((const volatile Slot *)S)->far_T != kInf;
-        const int end = level_end(cnt > 0, pull, st.level + 1, level_cap(g, st.kind));
+        const int end = level_end(cnt > 0, pull, level, level_cap(g, st.kind));
         if (end == kGoesOn && !broken) {
             ws_list(st.ws, W, out).scan[cnt] = (int32_t)edges;
             S->par = out;

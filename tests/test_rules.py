@@ -36,3 +36,7 @@ def test_work_left_at_the_iteration_cap_is_an_error(call):
              ((0, 1, 10, 10), goes_on), ((0, 1, 11, 10), cut), ((1, 1, 11, 10), cut)]
     got = call(*["level_end({}, {}, {}u, {}u)".format(*args) for args, _ in cases])
     assert got == [want for _, want in cases]
+
+
+def test_an_empty_list_is_no_iteration(call):
+    assert call("level_after(7u, 0u)", "level_after(7u, 1u)", "level_after(7u, 4000000000u)") == [7, 8, 8]
