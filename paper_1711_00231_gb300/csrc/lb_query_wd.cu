@@ -568,9 +568,9 @@ __device__ __forceinline__ bool fast_levels(const StepParams &p, const QueryArgs
                 }
                 q.pushes += q.fast_n;
             }
+            if (SSSP) far_engage(q, e, p.g.m);
             q.u.relaxed += e;
             q.u.iters += 1u;
-            if (SSSP) far_engage(q, e, p.g.m);
             q.u.level = level + 1u;
         }
         buf ^= 1u;

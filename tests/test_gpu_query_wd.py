@@ -269,3 +269,40 @@ def test_failed_query_reports_nothing_of_the_one_before():
             G.set_options(test_barrier_skip=0)
     finally:
         G.close()
+
+
+@pytest.mark.parametrize("before,edges,engages", [(6, 10.5, True), (6, 16, True), (6, 7.5, False), (5, 16, False)])
+def test_threshold_rule_on_fast_levels(before, edges, engages):
+    # `before` lists, then one of W one-edge entries that the team runs as a
+    # fast level.  The threshold comes in there if at least 6 iterations and
+    # fewer than a quarter of the graph's `edges` * W edges have been listed
+    # with it: W by the hub's list, W by this one.  Behind it 50 vertices at
+    # far distances: one list in plain order, many with a threshold.
+    W, far = 20000, 50
+    mids = before + np.arange(W)
+    c = before + W
+    y = c + 1 + np.arange(far)
+    src = [np.arange(before - 1), np.full(W, before - 1), mids, np.full(far, c), y]
+    dst = [1 + np.arange(before - 1), mids, np.full(W, c), y, np.full(far, c + far + 1)]
+    w = [np.ones(before - 1), np.ones(W), np.ones(W), 100000 * (1 + np.arange(far)), np.ones(far)]
+    m = int(edges * W)
+    pad = m - sum(len(x) for x in src)
+    u = c + far + 2 + np.arange(-(-pad // 4))  # not reached
+    src.append(np.repeat(u, 4)[:pad])
+    dst.append(np.tile(np.arange(4), u.size)[:pad])
+    w.append(np.ones(pad))
+    src, dst, w = (np.concatenate(x).astype(np.int64) for x in (src, dst, w))
+    g = gg.from_edges(int(u[-1]) + 1, src, dst, w)
+    assert g.m == m
+    # the first width comes from 1024 evenly spaced weights: none of the far ones
+    assert (g.weights[(np.arange(1024) * m) >> 10] == 1).all()
+    G = lb.Graph.from_csr(g)
+    try:
+        d, rc = G.sssp(0, "WD")
+        assert rc == lb.LB_OK and np.array_equal(d, oracle.dijkstra(g, 0)[0])
+        t = G.trace()
+        assert list(t["edges"][before - 1:before + 1]) == [W, W] and t["mode"][before] == 4
+        plain = before + 3  # the lists before, of the W, of c, of the far vertices
+        assert len(t) == plain if not engages else len(t) > plain + 3
+    finally:
+        G.close()
