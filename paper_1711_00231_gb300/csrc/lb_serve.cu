@@ -761,7 +761,8 @@ __device__ __noinline__ int solo_levels(const Params &P, Slot *S, SoloState &q, 
         const bool pull = SSSP && n == 0u && T != kInf && from != kInf;
         // the list stays with this CTA while it fits and the launch may go
         // on; clocks, the host's flag and admission every 16 levels (every level:
-        // serving burst 13.1 -> 14.2 ms)
+        // serving burst 13.1 -> 14.2 ms) and after every pull (milliseconds
+        // when many blocks hold far vertices)
         const bool look = (steps++ & 15u) == 0u;
         if (look && tid == 0) {
             const uint64_t now = global_ns();
@@ -838,6 +839,7 @@ __device__ __noinline__ int solo_levels(const Params &P, Slot *S, SoloState &q, 
                 q.int_edges = 0ull;
             }
             b ^= 1u;
+            steps = 0u;
             continue;
         }
         for (uint32_t i0 = 0; i0 < n; i0 += kE * kGroups) {

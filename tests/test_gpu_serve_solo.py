@@ -85,3 +85,49 @@ def test_wide_fronts_match_oracle(launch_ms):
     finally:
         S.close()
         G.close()
+
+
+def test_launch_limit_is_seen_after_every_pull():
+    # 190,000 far vertices in blocks of their own, nearly all at one distance:
+    # every pull reads all of their blocks (milliseconds) and queues ten
+    # vertices.  A launch of 1 ms has to end after each.
+    import torch
+    chain, mids, far, groups, pads = 33, 5000, 190000, 24, 1000
+    hub = chain + 1 + mids
+    fv = hub + 32 * (1 + np.arange(far))
+    sink = int(fv[-1]) + 1
+    n = sink + 1 + pads
+    deg = np.zeros(n, np.int64)
+    deg[:chain] = 1
+    deg[chain] = mids
+    deg[chain + 1:hub] = 1
+    deg[hub] = far
+    deg[fv] = 1
+    deg[sink + 1:] = 13000  # not reached: the mean weight stays 1
+    off = np.concatenate([[0], np.cumsum(deg)])
+    col = np.zeros(off[-1], np.int32)
+    w = np.ones(off[-1], np.uint32)
+    col[:chain] = 1 + np.arange(chain)
+    col[off[chain]:off[chain + 1]] = chain + 1 + np.arange(mids)
+    col[off[chain + 1]:off[hub]] = hub
+    heavy = slice(off[hub], off[hub + 1])
+    col[heavy] = fv
+    dist = np.full(far, 1 << 30)
+    dist[:10 * groups] = 64 << (np.arange(10 * groups) // 10)
+    w[heavy] = dist
+    col[off[fv]] = sink
+    col[off[sink + 1]:] = np.tile(np.arange(13000), pads)
+    sample = (np.arange(64) * off[-1]) >> 6
+    assert (w[sample] == 1).all()
+    g = gg.CSRGraph(n, int(off[-1]), off, col, w, "far", {})
+    G = lb.Graph.from_csr(g)
+    S = sv.Server([G], slots=4, mem_fraction=0.05, launch_ms=1)
+    try:
+        out = torch.empty(n, dtype=torch.int32, device="cuda")
+        status = S.run_batch([sv.Request(0.0, 0, 0, "sssp")], [out], timeout_s=120.0)
+        torch.cuda.synchronize()
+        assert status[0] == lb.LB_OK and np.array_equal(out.cpu().numpy().view(np.uint32), oracle.dijkstra(g, 0)[0])
+        assert S.info()["kernel_launches"] >= groups // 2
+    finally:
+        S.close()
+        G.close()
