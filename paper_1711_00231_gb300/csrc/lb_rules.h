@@ -31,4 +31,10 @@ LB_HD inline int level_end(bool list, bool pull, uint32_t level, uint32_t cap) {
 // Iterations so far, after a list of `entries` entries.
 LB_HD inline uint32_t level_after(uint32_t level, uint32_t entries) { return level + (entries > 0u ? 1u : 0u); }
 
+// Serving: whether a list of E edges, the last of `lists` lists with `edges`
+// edges, is one of a growing front.  After its largest lists a random graph's
+// query has a tail of short ones that a distance threshold only lengthens:
+// lone SSSP on 2^20 vertices and 2^21 edges 2.09 ms with it, 1.36 without.
+LB_HD inline bool front_grows(uint64_t E, uint32_t lists, uint64_t edges) { return E * lists >= edges; }
+
 }  // namespace lbk

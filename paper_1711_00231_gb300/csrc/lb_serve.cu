@@ -365,7 +365,7 @@ __device__ int end_query(const Params &P, Slot *S, const GraphDev &g, int32_t ki
 
 // SSSP, after a list of E edges in iteration `level` (single thread): the
 // interval's books, and the distance threshold once lists get long after
-// many iterations (a grid's).  A list past kServeFarMax by then belongs to a
+// many iterations while lists still grow (a grid's).  A list past kServeFarMax by then belongs to a
 // graph whose far set one CTA should not pull: random graphs that took the
 // whole-query kernel's rule got slower (Erdos-Renyi, 1M vertices, 8M edges:
 // 2.4 -> 4.2 ms).
@@ -400,6 +400,7 @@ __device__ void far_account(Slot *S, const GraphDev &g, uint32_t level, uint64_t
     V->int_lists = V->int_lists + 1u;
     V->int_edges = V->int_edges + E;
     if (V->far_engaged || level < 32u || E < kServeFarEdges || E > kServeFarMax) return;
+    if (!front_grows(E, V->int_lists, V->int_edges)) return;
     // first width: 32 * mean weight (of 64 evenly spaced edges) / mean degree
     unsigned long long w = 0;
 #pragma unroll 16
@@ -905,13 +906,15 @@ __device__ __noinline__ int solo_levels(const Params &P, Slot *S, SoloState &q, 
             if (tid == 0) {
                 volatile Slot *V = S;
                 V->relaxed = relaxed;
+                V->int_lists = q.int_lists;
+                V->int_edges = q.int_edges;
                 far_account(S, g, level, e);
+                q.int_lists = V->int_lists;
+                q.int_edges = V->int_edges;
                 if (V->far_engaged) {
                     q.engaged = 1u;
                     q.far.T = V->far_T;
                     q.delta = V->far_delta;
-                    q.int_lists = 0u;
-                    q.int_edges = 0ull;
                 }
             }
             __syncthreads();

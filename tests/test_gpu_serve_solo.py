@@ -131,3 +131,30 @@ def test_launch_limit_is_seen_after_every_pull():
     finally:
         S.close()
         G.close()
+
+
+def test_no_threshold_in_a_random_graphs_tail():
+    # the lists of iterations 32 and on are the query's last, short ones: no
+    # more iterations than in plain order (the host loop's)
+    import torch
+    g = gg.erdos_renyi(300000, 480000, seed=1)
+    src = 73589
+    G = lb.Graph.from_csr(g)
+    G.set_options(loop_mode=1)
+    ref, rc = G.sssp(src, "WD")
+    assert rc == lb.LB_OK and np.array_equal(ref, oracle.dijkstra(g, src)[0])
+    plain = G.stats()["iterations"]
+    t = G.trace()["edges"]
+    assert plain > 36 and ((t[32:] >= 4096) & (t[32:] <= 32768)).any()
+    S = sv.Server([G], slots=2, mem_fraction=0.05)
+    try:
+        out = torch.empty(g.n, dtype=torch.int32, device="cuda")
+        S.submit(0, src, "sssp", out)
+        done = []
+        while not done:
+            done = S.poll()
+        assert done[0][1] == lb.LB_OK and np.array_equal(out.cpu().numpy().view(np.uint32), ref)
+        assert done[0][3] <= plain + 3  # the order inside an iteration may change its number by a few
+    finally:
+        S.close()
+        G.close()

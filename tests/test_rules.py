@@ -40,3 +40,14 @@ def test_work_left_at_the_iteration_cap_is_an_error(call):
 
 def test_an_empty_list_is_no_iteration(call):
     assert call("level_after(7u, 0u)", "level_after(7u, 1u)", "level_after(7u, 4000000000u)") == [7, 8, 8]
+
+
+def test_threshold_needs_a_growing_front(call):
+    grid = [4 * (k + 1) for k in range(2000)]  # lists of a grid: longer by a little every iteration
+    rand = [1 << k for k in range(18)] + [400000, 300000, 120000, 50000] + [40000 - 2000 * k for k in range(19)]
+    exprs, want = [], []
+    for lists, grows in ((grid, True), (rand, False)):
+        for k in range(32, len(lists)):
+            exprs.append(f"front_grows({lists[k]}ull, {k + 1}u, {sum(lists[:k + 1])}ull)")
+            want.append(int(grows))
+    assert call(*exprs) == want
