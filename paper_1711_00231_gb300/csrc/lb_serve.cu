@@ -826,14 +826,9 @@ __device__ __noinline__ int solo_levels(const Params &P, Slot *S, SoloState &q, 
             if (tid == 0) {
                 q.fmin = kInf;
                 if (q.int_lists > 0u) {
-                    const unsigned long long avg = q.int_edges / q.int_lists;
                     const bool wide = (((g.n - 1) >> q.far.shift) >> 5) >= kPullWords;
-                    const unsigned long long least = wide ? kPullEdges * q.reads : 0ull;
-                    if (q.int_edges < least || avg < kSoloEdges / 8u) {
-                        if (q.delta < kFarMaxDelta) q.delta *= 2u;
-                    } else if (avg > kSoloEdges / 2u && q.int_edges > 4u * least) {
-                        q.delta = max(q.delta / 2u, 1u);
-                    }
+                    q.delta = next_width(q.delta, q.reads, q.int_lists, q.int_edges, wide ? kPullEdges * q.reads : 0ull,
+                                         kSoloEdges, kFarMaxDelta);
                 }
                 q.reads = 0u;
                 q.int_lists = 0u;

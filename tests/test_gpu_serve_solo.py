@@ -158,3 +158,23 @@ def test_no_threshold_in_a_random_graphs_tail():
     finally:
         S.close()
         G.close()
+
+
+def test_far_set_spread_over_the_graph():
+    # 1% of the edges heavy: their far ends keep thousands of blocks alive, so
+    # that pulls outweigh lists and intervals widen
+    import torch
+    g = gg.grid(1024, 1024, seed=1)
+    g.weights[:] = np.where(np.random.default_rng(1).random(g.m) < 0.01, 1000000, 1)
+    G = lb.Graph.from_csr(g)
+    S = sv.Server([G], slots=4, mem_fraction=0.05)
+    try:
+        src = [0, g.n // 2 + 300]
+        outs = [torch.empty(g.n, dtype=torch.int32, device="cuda") for _ in src]
+        status = S.run_batch([sv.Request(0.0, 0, s, "sssp") for s in src], outs, timeout_s=120.0)
+        torch.cuda.synchronize()
+        for s, o, st in zip(src, outs, status):
+            assert st == lb.LB_OK and np.array_equal(o.cpu().numpy().view(np.uint32), oracle.dijkstra(g, s)[0]), s
+    finally:
+        S.close()
+        G.close()

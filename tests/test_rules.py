@@ -51,3 +51,23 @@ def test_threshold_needs_a_growing_front(call):
             exprs.append(f"front_grows({lists[k]}ull, {k + 1}u, {sum(lists[:k + 1])}ull)")
             want.append(int(grows))
     assert call(*exprs) == want
+
+
+def test_interval_widens_while_its_pull_costs_more_than_its_lists(call):
+    big = 1 << 30
+    cases = [  # delta, reads, lists, edges, least -> width
+        ((8, 0, 8, 8 * 3000, 0), 8),            # cheap pull, lists of middle length: as it is
+        ((8, 2048 * 8, 8, 8 * 3000, 0), 8),
+        ((8, 2048 * 8 + 1, 8, 8 * 3000, 0), 16),  # the pull outweighs the lists
+        ((8, 100000, 8, 8 * 3000, 0), 16),
+        ((8, 100000, 8, 8 * 6000, 0), 16),      # also when the lists are long
+        ((8, 2048 * 2, 8, 8 * 6000, 0), 8),     # narrower would soon be too costly
+        ((8, 2048 * 2 - 1, 8, 8 * 6000, 0), 4),
+        ((8, 0, 8, 8 * 1000, 0), 16),           # short lists
+        ((8, 0, 8, 8 * 3000, 8 * 3000 + 1), 16),  # fewer edges than asked
+        ((8, 0, 8, 8 * 6000, 2 * 6000), 8),
+        ((1, 0, 8, 8 * 6000, 0), 1),
+        ((big, 1 << 40, 8, 8, 0), big),
+    ]
+    got = call(*["next_width({}u, {}ull, {}u, {}ull, {}ull, 8192u, {}u)".format(*a, big) for a, _ in cases])
+    assert got == [w for _, w in cases]
