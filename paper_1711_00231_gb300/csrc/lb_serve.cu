@@ -347,9 +347,13 @@ __device__ __forceinline__ uint32_t level_cap(const GraphDev &g, int32_t kind) {
 #ifndef LB_SOLO_EDGES
 #define LB_SOLO_EDGES 8192
 #endif
-constexpr uint32_t kSoloEdges = LB_SOLO_EDGES, kSoloAvgDeg = 8, kSoloMaxDeg = 64;
-__device__ __forceinline__ bool solo_fits(const WsLayout &W, int64_t cnt, uint64_t edges) {
-    return edges <= kSoloEdges && edges <= kSoloAvgDeg * (uint64_t)cnt && (int64_t)edges <= W.cap;
+#ifndef LB_SOLO_EDGES_BFS
+#define LB_SOLO_EDGES_BFS 4096
+#endif
+constexpr uint32_t kSoloEdges = LB_SOLO_EDGES, kSoloEdgesBfs = LB_SOLO_EDGES_BFS, kSoloAvgDeg = 8, kSoloMaxDeg = 64;
+__device__ __forceinline__ uint32_t solo_edges(int32_t kind) { return kind == 1 ? kSoloEdges : kSoloEdgesBfs; }
+__device__ __forceinline__ bool solo_fits(const WsLayout &W, int32_t kind, int64_t cnt, uint64_t edges) {
+    return edges <= solo_edges(kind) && edges <= kSoloAvgDeg * (uint64_t)cnt && (int64_t)edges <= W.cap;
 }
 
 // The query's worklist is empty (or it was stopped): overflow check or
@@ -440,7 +444,7 @@ __device__ int finish_job(const Params &P, Slot *S, uint32_t kind) {
         for (int64_t k = 0; k < grains && k < W.tcap; ++k) L.tstart[k] = 0;
         S->in_cnt = 1;
         S->in_edges = (uint64_t)deg;
-        if (solo_fits(W, 1, (uint64_t)deg)) return kAfterSolo;
+        if (solo_fits(W, st.kind, 1, (uint64_t)deg)) return kAfterSolo;
         const int64_t Tj = job_tile(P, deg);
         open_job(S, kJobRelax, (uint32_t)((deg + Tj - 1) / Tj), (uint32_t)(Tj / kTileGrain));
         return kAfterJob;
@@ -467,7 +471,7 @@ __device__ int finish_job(const Params &P, Slot *S, uint32_t kind) {
             S->in_cnt = (uint32_t)cnt;
             S->in_edges = (uint64_t)edges;
             S->out_pack = 0ull;
-            if (pull || solo_fits(W, cnt, (uint64_t)edges)) return kAfterSolo;
+            if (pull || solo_fits(W, st.kind, cnt, (uint64_t)edges)) return kAfterSolo;
             const int64_t Tj = job_tile(P, edges);
             open_job(S, kJobRelax, (uint32_t)((edges + Tj - 1) / Tj), (uint32_t)(Tj / kTileGrain));
             return kAfterJob;
@@ -657,7 +661,7 @@ __device__ void release_admit(const Params &P) {
 // iterations.  As jobs each took 11 us (24 us among 128 queries): claim, done
 // count, finalisation and the next job's opening are some fifteen dependent
 // L2 trips beside the tile's own.  The CTA that finishes a job whose next list
-// has at most kSoloEdges edges therefore goes on with the query alone, one
+// has at most solo_edges() edges therefore goes on with the query alone, one
 // level after another with only block barriers between them, until the list
 // grows, the query ends or the launch has to end (the next job is then opened
 // as usual).  Lists are kept in the query's own worklists as {vertex, first
@@ -667,8 +671,11 @@ __device__ void release_admit(const Params &P) {
 //
 // Measured: 512 x 543 grid alone in the engine, BFS 10.9 -> 4.0 us per
 // iteration, SSSP 17.4 -> 10.0 ms; a burst of 128 queries over 12 graphs 24.6
-// -> 13.1 ms.  kSoloEdges 4096 / 8192 / 16384: 15.0 / 13.7 / 19.1 ms (longer
-// lists are many rounds for one CTA); kE 2 / 3 / 4 / 6: 14.0 / 13.7 / 13.3 /
+// -> 13.1 ms.  kSoloEdges (SSSP) 4096 / 8192 / 16384: 15.0 / 13.7 / 19.1 ms (longer
+// lists are many rounds for one CTA); kSoloEdgesBfs 512 / 2048 / 4096 / 8192: lone
+// BFS on a 1024^2 grid 19.8 / 14.9 / 11.9 / 12.0, 2048^2 46.9 / 41.0 / 38.0 / 49.3 ms
+// (as jobs 48), Erdos-Renyi 4M vertices, 16M edges 1.022 / 1.022 / 1.023 / 1.048 ms,
+// 128 mixed queries 12.9 / 13.0 / 12.7 / 13.0 ms; kE 2 / 3 / 4 / 6: 14.0 / 13.7 / 13.3 /
 // 15.0 ms; kServeFarEdges 2048 / 4096 / 8192: 13.9 / 13.7 / 14.9 ms.
 struct SoloState {
     uint32_t out_n, out_e, out_maxdeg, fmin, leave;
@@ -780,7 +787,7 @@ __device__ __noinline__ int solo_levels(const Params &P, Slot *S, SoloState &q, 
         __syncthreads();
         if (n == 0u && !pull) break;
         if (level > level_cap(g, SSSP ? 1 : 0)) break;
-        if (n > 0u && (leave || e > kSoloEdges || maxdeg > kSoloMaxDeg || (int64_t)e > W.cap)) break;
+        if (n > 0u && (leave || e > solo_edges(SSSP ? 1 : 0) || maxdeg > kSoloMaxDeg || (int64_t)e > W.cap)) break;
         if (n == 0u && leave) break;
         const NodeList in = ws_list(st.ws, W, b), out = ws_list(st.ws, W, b ^ 1u);
         if (SSSP && pull) {

@@ -178,3 +178,20 @@ def test_far_set_spread_over_the_graph():
     finally:
         S.close()
         G.close()
+
+
+@pytest.mark.parametrize("k,deg", [(512, 8), (513, 8), (4095, 1), (4096, 1), (4097, 1)])
+def test_bfs_lists_at_the_single_cta_limit(k, deg):
+    import torch
+    g = fan(k, deg)
+    G = lb.Graph.from_csr(g)
+    S = sv.Server([G], slots=4, mem_fraction=0.05)
+    try:
+        outs = [torch.empty(g.n, dtype=torch.int32, device="cuda") for _ in range(2)]
+        status = S.run_batch([sv.Request(0.0, 0, 0, "bfs"), sv.Request(0.0, 0, 1, "bfs")], outs, timeout_s=60.0)
+        torch.cuda.synchronize()
+        for s, (o, st) in enumerate(zip(outs, status)):
+            assert st == lb.LB_OK and np.array_equal(o.cpu().numpy(), oracle.bfs(g, s)[0]), s
+    finally:
+        S.close()
+        G.close()
