@@ -637,13 +637,17 @@ __device__ void admit(const Params &P) {
     st_release_sys(&P.host->consumed, con);
 }
 
-// Takes the admission lock if free and, unless the grid is leaving, admits
+// Takes the admission lock if free and, unless the grid is leaving, looks at
+// the host's stop flag (for all CTAs: they read `stopping`) and admits
 // pending requests into free slots (thread 0 of a CTA).  Returns whether
 // the lock was taken; *admitted tells whether any request was admitted.
 __device__ bool try_admit(const Params &P, bool *admitted) {
     *admitted = false;
     if (atomicCAS(&P.sh->admit_lock, 0u, 1u) != 0u) return false;
-    if (__ldcg(&P.sh->stopping) == 0u) {
+    if (__ldcg(&P.sh->stopping) != 0u) return true;
+    if (ld_acquire_sys32(&P.host->stop) != 0u) {
+        atomicExch(&P.sh->stopping, 1u);
+    } else if (__ldcg(&P.sh->active) < (uint32_t)P.nslots) {
         const unsigned long long before = __ldcg(&P.sh->consumed);
         admit(P);
         *admitted = __ldcg(&P.sh->consumed) != before;
@@ -774,12 +778,12 @@ __device__ __noinline__ int solo_levels(const Params &P, Slot *S, SoloState &q, 
         const bool look = (steps++ & 15u) == 0u;
         if (look && tid == 0) {
             const uint64_t now = global_ns();
-            q.leave = now - t_launch > P.hard_ns || ld_acquire_sys32(&P.host->stop) != 0u ? 1u : 0u;
-            if (now - last_admit > kAdmitPeriodNs && __ldcg(&P.sh->active) < (uint32_t)P.nslots) {
+            if (now - last_admit > kAdmitPeriodNs) {
                 last_admit = now;
                 bool admitted = false;
                 if (try_admit(P, &admitted)) release_admit(P);
             }
+            q.leave = now - t_launch > P.hard_ns || __ldcg(&P.sh->stopping) != 0u ? 1u : 0u;
         }
         __syncthreads();
         if (tid == 0) q.out_n = q.out_e = q.out_maxdeg = 0u;
@@ -1013,6 +1017,7 @@ __global__ void __launch_bounds__(kBlock, LB_SERVE_MIN_BLOCKS) k_serve(Params P)
     __shared__ int s_exit;
     __shared__ uint32_t s_scan_from;
     __shared__ int s_next;
+    __shared__ int s_stop;  // this CTA claims nothing more
     __shared__ SoloState s_solo;
     const uint32_t warp = threadIdx.x >> 5;
     uint64_t idle_since = 0;
@@ -1026,7 +1031,10 @@ __global__ void __launch_bounds__(kBlock, LB_SERVE_MIN_BLOCKS) k_serve(Params P)
 #define PF_MARK(v)
 #define PF_ADD(i, v)
 #endif
-    if (threadIdx.x == 0) s_scan_from = blockIdx.x % (uint32_t)P.nslots;
+    if (threadIdx.x == 0) {
+        s_scan_from = blockIdx.x % (uint32_t)P.nslots;
+        s_stop = 0;
+    }
     const uint64_t t_launch = __ldcg(&P.sh->kernel_t0);  // written by k_serve_t0 before this launch
     for (;;) {
         // every thread has read the previous iteration's s_* values before
@@ -1042,20 +1050,23 @@ __global__ void __launch_bounds__(kBlock, LB_SERVE_MIN_BLOCKS) k_serve(Params P)
             // slot's claim and job words, and the claimable slots are tried
             // in order until a claim holds
             const uint32_t lane = threadIdx.x;
-            // past the launch's time limit a CTA claims nothing more and
-            // leaves (checked before every claim: a CTA that keeps finding
-            // work, such as the one that opens a slot's next job, would
-            // otherwise never see the limit)
-            int late = 0;
-            if (lane == 0) late = global_ns() - t_launch > P.hard_ns;
-            late = __shfl_sync(kFull, late, 0);
+            // past the launch's time limit, or once it has seen the host's
+            // stop, a CTA claims nothing more and leaves (checked before every
+            // claim: a CTA that keeps finding work, such as the one that
+            // opens a slot's next job, would otherwise never see it)
+            int late = 0, stop = 0;
+            if (lane == 0) {
+                late = global_ns() - t_launch > P.hard_ns;
+                stop = s_stop;
+            }
+            const int leave = __shfl_sync(kFull, late | stop, 0);
             const uint32_t scan_from = s_scan_from;
-            uint32_t nw = late ? 0u : ((uint32_t)P.nslots + 31u) >> 5;
+            uint32_t nw = leave ? 0u : ((uint32_t)P.nslots + 31u) >> 5;
             const uint32_t sw = scan_from >> 5;
             int found = -1;
             uint32_t f_kind = 0, f_tiles = 0, f_tile = 0, f_q = 0;
             unsigned long long seen_oldest = kNoOldest;  // oldest busy slot this scan saw
-            if (P.policy == 0 && !late) {
+            if (P.policy == 0 && !leave) {
                 // the oldest query in flight first: its iterations then run as
                 // if it were alone, and the other queries fill the CTAs its
                 // current iteration leaves idle
@@ -1158,7 +1169,7 @@ __global__ void __launch_bounds__(kBlock, LB_SERVE_MIN_BLOCKS) k_serve(Params P)
                     atomicMin(&P.sh->oldest, seen_oldest);
                 if (found >= 0) s_scan_from = (uint32_t)found;
                 s_slot = found;
-                s_exit = late;
+                s_exit = leave;
                 if (late) atomicOr(&P.sh->error, kErrDeadline);
                 if (found >= 0) {
                     s_kind = f_kind;
@@ -1187,7 +1198,7 @@ __global__ void __launch_bounds__(kBlock, LB_SERVE_MIN_BLOCKS) k_serve(Params P)
                     }
                     release_admit(P);
                 }
-                if (ld_acquire_sys32(&P.host->stop) != 0u || __ldcg(&P.sh->stopping) != 0u) s_exit = 1;
+                if (__ldcg(&P.sh->stopping) != 0u) s_exit = 1;
                 if (!s_exit) __nanosleep(256);
             } else if (s_slot >= 0) {
                 idle_since = 0;
@@ -1244,7 +1255,12 @@ __global__ void __launch_bounds__(kBlock, LB_SERVE_MIN_BLOCKS) k_serve(Params P)
             const int after = ((const volatile Slot *)S)->kind == 1
                                   ? solo_levels<true>(P, S, s_solo, s_wb[warp], t_launch, last_admit)
                                   : solo_levels<false>(P, S, s_solo, s_wb[warp], t_launch, last_admit);
-            if (threadIdx.x == 0) s_next = after;
+            if (threadIdx.x == 0) {
+                s_next = after;
+                // it left for the launch's end: no claim, not even of the job it
+                // has just opened (it would come back here, and leave again)
+                if (s_solo.leave) s_stop = 1;
+            }
         }
         if (threadIdx.x == 0) {
             const bool reopened = s_next == kAfterJob;
@@ -1258,12 +1274,13 @@ __global__ void __launch_bounds__(kBlock, LB_SERVE_MIN_BLOCKS) k_serve(Params P)
             // then runs without waiting for a scan to come by)
             s_scan_from = reopened ? (uint32_t)si : ((uint32_t)si + 1u) % (uint32_t)P.nslots;
             // busy CTAs also refill free slots, so that admission does not
-            // wait until some CTA runs out of work
+            // wait until some CTA runs out of work, and see the host's stop
             const uint64_t now = global_ns();
-            if (now - last_admit > kAdmitPeriodNs && __ldcg(&P.sh->active) < (uint32_t)P.nslots) {
+            if (now - last_admit > kAdmitPeriodNs) {
                 last_admit = now;
                 bool admitted = false;
                 if (try_admit(P, &admitted)) release_admit(P);
+                if (__ldcg(&P.sh->stopping) != 0u) s_stop = 1;
             }
 #if LB_SERVE_PROFILE
             PF_ADD(4, clock64() - c_d);

@@ -195,3 +195,51 @@ def test_bfs_lists_at_the_single_cta_limit(k, deg):
     finally:
         S.close()
         G.close()
+
+
+@pytest.mark.parametrize("policy", [0, 1])
+def test_stop_with_queries_in_flight(policy):
+    # strips of half a second and more, one of them an SSSP whose threshold is
+    # in force, beside a graph of long lists: a stop returns at once, and the
+    # queries go on at the next poll
+    import time
+    import torch
+    cg = [gg.grid(4, 20000, seed=1), gg.grid(64, 8000, seed=2), gg.erdos_renyi(1 << 20, 1 << 23, seed=3)]
+    G = [lb.Graph.from_csr(g) for g in cg]
+    S = sv.Server(G, slots=16, mem_fraction=0.1, launch_ms=5000, policy=policy)
+    try:
+        for wanted in ([(0, "sssp")], [(0, "bfs")], [(1, "sssp")], [(2, "sssp"), (0, "sssp"), (1, "bfs"), (0, "bfs")]):
+            outs = [torch.empty(cg[g].n, dtype=torch.int32, device="cuda") for g, _ in wanted]
+            torch.cuda.synchronize()
+            tick = {S.submit(g, 0, kind, o): i for i, ((g, kind), o) in enumerate(zip(wanted, outs))}
+            for pause in (0.0, 0.004, 0.05):
+                time.sleep(pause)
+                t0 = time.perf_counter()
+                S.stop()
+                assert time.perf_counter() - t0 < 1.0
+                for c in S.poll():  # starts the engine again
+                    assert c[1] == lb.LB_OK
+                    del tick[c[0]]
+            end = time.perf_counter() + 60
+            while tick and time.perf_counter() < end:
+                for c in S.poll():
+                    assert c[1] == lb.LB_OK
+                    del tick[c[0]]
+            assert not tick
+            torch.cuda.synchronize()
+            for (gi, kind), o in zip(wanted, outs):
+                got = o.cpu().numpy()
+                ref = oracle.bfs(cg[gi], 0)[0] if kind == "bfs" else oracle.dijkstra(cg[gi], 0)[0].view(np.int32)
+                assert np.array_equal(got, ref), (gi, kind)
+        # an engine is destroyed with a query in flight
+        last = torch.empty(cg[1].n, dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        S.submit(1, 0, "sssp", last)
+        time.sleep(0.02)
+        t0 = time.perf_counter()
+        S.close()
+        assert time.perf_counter() - t0 < 1.0
+    finally:
+        S.close()
+        for g in G:
+            g.close()
