@@ -170,6 +170,7 @@ struct lb_graph {
     int grid[kStrategies][2]{};
     int query_grid[2]{};        // whole-query WD launch (0: not yet computed)
     uint32_t query_number = 0;  // whole-query WD launches so far
+    bool team_picked = false;   // the SMs of its small-list team are chosen
 
     // batched host-output queries: the second result buffer, one error
     // word per query, the copy stream and the events that order each
@@ -300,6 +301,7 @@ lb_status alloc_lists(lb_graph *g, NodeList *L, int64_t &bytes, int64_t cap, int
 void free_workspace(lb_graph *g) {
     drop_execs(g);
     g->release(g->ctl, 1);
+    g->team_picked = false;
     g->release(g->bitmap, bitmap_alloc_words(g->n));
     g->release(g->fast_seg, fast_entries(g->n));
     g->release(g->out_internal, g->n);
@@ -365,7 +367,6 @@ lb_status ensure_workspace(lb_graph *g, int s) {
     if (!g->ctl) {
         LB_TRY(g->alloc(&g->ctl, 1));
         LB_CU(cudaMemsetAsync(g->ctl, 0, sizeof(Ctl), g->stream));
-        LB_CU(launch_team_pick(g->ctl, g->sms, g->stream));
     }
     if (!g->bitmap) LB_TRY(g->alloc(&g->bitmap, bitmap_alloc_words(g->n)));
     if (s == LB_NS || s == LB_NS_PHYS || s == LB_HP) LB_TRY(ensure_mdt(g));
@@ -420,6 +421,12 @@ lb_status ensure_workspace(lb_graph *g, int s) {
         g->have_tiles = want_tiles;
     }
     if (s == LB_WD && !g->fast_seg) LB_TRY(g->alloc(&g->fast_seg, fast_entries(g->n)));
+    // only the whole-query launch has a team (its pick takes an idle GPU: a
+    // CTA with 160 KB of shared memory per SM)
+    if (s == LB_WD && g->opt.loop_mode == 0 && !g->team_picked) {
+        LB_CU(launch_team_pick(g->ctl, g->sms, g->stream));
+        g->team_picked = true;
+    }
     if (s == LB_HP && !g->have_subs) {
         quiesce(g);
         drop_execs(g);
