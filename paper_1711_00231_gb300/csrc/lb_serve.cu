@@ -1024,7 +1024,7 @@ __global__ void __launch_bounds__(kBlock, LB_SERVE_MIN_BLOCKS) k_serve(Params P)
     uint64_t last_admit = 0;
 #if LB_SERVE_PROFILE
     unsigned long long pf[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    long long c_top = 0, c_mid = 0;
+    long long c_top = 0, c_mid = 0, c_b = 0;
 #define PF_MARK(v) (v) = clock64()
 #define PF_ADD(i, v) pf[i] += (unsigned long long)((v))
 #else
@@ -1237,7 +1237,7 @@ __global__ void __launch_bounds__(kBlock, LB_SERVE_MIN_BLOCKS) k_serve(Params P)
         __syncthreads();
         if (threadIdx.x == 0) {
 #if LB_SERVE_PROFILE
-            long long c_b = clock64();
+            c_b = clock64();
             PF_ADD(2, c_b - c_mid);
             PF_ADD(5, 1);
 #endif
