@@ -139,7 +139,10 @@ typedef struct lb_options {
                               LB_ERR_TIMEOUT with the device still usable.
                               Device loop: 2 makes the CTAs outside the
                               small-list team 200 us late in reading what a
-                              grid barrier published */
+                              grid barrier published; 3 and 4 make CTA 1 of
+                              the team leave before a step of the team, 5
+                              the whole team (LB_ERR_TIMEOUT as for 1, after
+                              4 s for 5) */
     int32_t bitmap_place;  /* 0..7 (0): where the visited / queued bitmap
                               starts inside its allocation, in steps of
                               min(1 MiB, one bitmap half rounded up to 4

@@ -92,7 +92,10 @@ constexpr int kFastSeg = LB_FAST_SEG;    // entries per CTA segment of a fast le
 enum : int32_t {
     kTestSkip = 1,       // CTA 1 leaves before its first grid barrier
     kTestLateReads = 2,  // CTAs outside the team are slow to read a step's counters after its barrier
-    kTestMax = 2,
+    kTestTeamSkip = 3,   // team CTA 1 leaves before its first regular step of the team
+    kTestFastSkip = 4,   // team CTA 1 leaves before its first fast level
+    kTestTeamGone = 5,   // every team CTA leaves before its first step (no time limit beside the waits')
+    kTestMax = 5,
 };
 
 constexpr uint32_t kMaxSms = 512;

@@ -939,7 +939,11 @@ __global__ void __launch_bounds__(kBlock, SSSP ? LB_QUERY_MIN_BLOCKS_SSSP : LB_Q
         } else if (!small) {
             team_mode = false;
         }
-        if (team_mode && fast_takes(p, a, q.u)) {
+        const bool fast = team_mode && fast_takes(p, a, q.u);
+        if (p.test_barrier_skip >= kTestTeamSkip && team_mode &&
+            (p.test_barrier_skip == kTestTeamGone || (q.rank == 1u && p.test_barrier_skip == (fast ? kTestFastSkip : kTestTeamSkip))))
+            return;
+        if (fast) {
             // uniform over the team: every CTA has the same state
             failed = !fast_levels<SSSP>(p, a, sync, q, s_wb[threadIdx.x >> 5]);
             // the team hands over, as after a regular level

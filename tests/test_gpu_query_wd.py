@@ -306,3 +306,44 @@ def test_threshold_rule_on_fast_levels(before, edges, engages):
         assert len(t) == plain if not engages else len(t) > plain + 3
     finally:
         G.close()
+
+
+@pytest.mark.parametrize("hook,graph", [(3, "spokes"), (3, "swing"), (4, "grid"), (4, "swing"), (5, "grid"), (5, "spokes")])
+def test_bounded_waits_of_the_team(hook, graph):
+    # a CTA of the team that never arrives (3: regular steps, 4: fast levels)
+    # or a team that never publishes (5): the waits run out, those of the CTAs
+    # outside the team too, and the next queries are exact
+    import time
+    g = {"grid": lambda: gg.grid(40, 50, seed=1), "spokes": lambda: swinging(1, 100, 4, 60),
+         "swing": lambda: swinging(3, 40000, 3, 50)}[graph]()
+    G = lb.Graph.from_csr(g)
+    try:
+        check(G, g, 0)
+        for query in (G.bfs, G.sssp):
+            G.set_options(test_barrier_skip=hook)
+            t = time.perf_counter()
+            with pytest.raises(lb.LbError) as ei:
+                query(0, "WD")
+            assert ei.value.status == lb.LB_ERR_TIMEOUT
+            assert 1.5 < time.perf_counter() - t < 8.0
+            G.set_options(test_barrier_skip=0)
+            check(G, g, 0)
+    finally:
+        G.close()
+
+
+def test_bounded_wait_of_the_host_loops_small_levels():
+    g = gg.grid(64, 64, seed=1)
+    G = lb.Graph.from_csr(g)
+    try:
+        G.set_options(test_barrier_skip=1, loop_mode=1)
+        for query in (G.bfs, G.sssp):
+            with pytest.raises(lb.LbError) as ei:
+                query(0, "WD")
+            assert ei.value.status == lb.LB_ERR_TIMEOUT
+        G.set_options(test_barrier_skip=0, loop_mode=1)
+        check(G, g, 0)
+        G.set_options(loop_mode=0)
+        check(G, g, 0)
+    finally:
+        G.close()
