@@ -305,7 +305,7 @@ lb_status lb_release_workspaces(lb_graph *g);
  * 2048) in the paper's form, and the binned form with the histogram MDT or
  * 256 / 2048 x thread bin 8 / 32 / 128; NS_PHYS -- the granule size; BS, EP
  * -- CTAs per SM, each timed once.  Then, for WD, small_edges 0 (no
- * persistent small-list launch and no conditional node for it) against the
+ * small-list team: every level on the whole grid) against the
  * fastest grid option, and the eight bitmap placements (bitmap_place) of
  * each of the three fastest grid options.  Wherever the final choice is
  * made, the three fastest candidates are timed twice more and ranked by

@@ -1196,9 +1196,8 @@ lb_status lb_autotune(lb_graph *g, int32_t kind, lb_strategy s, const int32_t *s
             best_o = top[0];
         }
     }
-    // For WD, whether the persistent small-list launch is worth its
-    // conditional node (a few microseconds per level on graphs that never
-    // run it), decided on the fastest grid option and applied to all three.
+    // For WD, whether levels with small lists are better left to the whole
+    // grid than to the small-list team, decided on the fastest grid option and applied to all three.
     if (!top.empty() && s == LB_WD && top[0].small_edges != 0) {
         std::vector<lb_options> two{top[0], top[0]};
         two[1].small_edges = 0;

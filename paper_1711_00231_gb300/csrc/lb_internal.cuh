@@ -85,7 +85,7 @@ struct TraceRec {
 #ifndef LB_FAST_SEG
 #define LB_FAST_SEG 2048
 #endif
-constexpr int kFastTeam = LB_FAST_TEAM;  // CTAs of the small-list team (a multiple of 32)
+constexpr int kFastTeam = LB_FAST_TEAM;  // CTAs of the small-list team (a multiple of 64)
 constexpr int kFastSeg = LB_FAST_SEG;    // entries per CTA segment of a fast level's list (two buffers)
 
 // lb_options.test_barrier_skip

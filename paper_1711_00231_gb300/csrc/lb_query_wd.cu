@@ -105,7 +105,7 @@ __device__ __forceinline__ bool arrive_team(QuerySync *s, uint32_t size, uint32_
 //
 // The far set needs no list: every reached vertex below T has been expanded
 // with its final distance when the list is empty, so the vertices waiting
-// are exactly those at T or above.  A bit per block of 2^far_shift (>= 128)
+// are exactly those at T or above.  A bit per block of 2^far_shift (32 up to 2^24)
 // vertices, set when one is held back, keeps a pull from scanning all
 // distances: it reads the blocks with a set bit, queues what lies below the
 // new T, and clears the bits of blocks with nothing left.
@@ -376,7 +376,7 @@ __device__ __forceinline__ bool fast_exchange(Ctl *ctl, QueryState &q) {
 #pragma unroll
         for (int j = 0; j < kFastWords; ++j) {
             in += (uint32_t)(w[j] >> 28) & 0xFFFu;
-            // up to 2^25 / kFastWords each (the sum fits 32 bits): that never fits a fast level
+            // up to 2^26 / kFastWords each (the sum of all fits 32 bits): that never fits a fast level
             e += min((uint32_t)w[j] & ((1u << 28) - 1u), (1u << 26) / kFastWords);
             md = max(md, (uint32_t)(w[j] >> 40) & 127u);
             late |= (uint32_t)(w[j] >> 47) & 1u;
