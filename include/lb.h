@@ -269,7 +269,12 @@ lb_status lb_sssp_batch(lb_graph *g, const int32_t *srcs, int64_t k, lb_strategy
  * distances) on the graph's device; parents_dev: NULL or n int32 receiving
  * a shortest-path tree (parent[src] = src, -1 unreachable; the parent of v
  * is a u with an edge u->v and dist[u] + w(u,v) = dist[v]).  The call is
- * asynchronous on `stream`; its status is read with lb_last_stats(). */
+ * asynchronous on `stream`; its status is read with lb_last_stats().
+ * A WD query is one launch whose CTAs wait on one another, so it starts once
+ * the whole GPU has room for them: queries on several graphs and streams run
+ * one after another, and beside a running engine (lb_server) a query waits
+ * until that goes idle, is stopped or reaches launch_ms.  Queries of the
+ * other strategies run beside an engine with ctas_per_sm <= 3. */
 lb_status lb_bfs_dev(lb_graph *g, int32_t src, lb_strategy s, int32_t *out_dev, int32_t *parents_dev, void *stream);
 lb_status lb_sssp_dev(lb_graph *g, int32_t src, lb_strategy s, uint32_t *out_dev, int32_t *parents_dev,
                       void *stream);
